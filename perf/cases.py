@@ -330,3 +330,98 @@ def run(s):
     if s.op == "extend":
         result["q"] = s.q
     return result
+
+
+# ---- the same outputs in 64 bits
+
+def _rotated(x, pos, case):
+    """Rows x [n, heads, D] turned by pos [n] positions."""
+    D = case["head_dim"]
+    freq = case["theta"] ** (-2.0 * torch.arange(D // 2, dtype=torch.float64, device=DEVICE) / D)
+    ang = pos.double()[:, None, None] * freq
+    c, n = ang.cos(), ang.sin()
+    lo, hi = (x[..., 0::2], x[..., 1::2]) if case["pairing"] else (x[..., :D // 2], x[..., D // 2:])
+    a, b = lo * c - hi * n, hi * c + lo * n
+    return torch.stack((a, b), dim=-1).flatten(-2) if case["pairing"] else torch.cat((a, b), dim=-1)
+
+
+def _attended(q, k, v, pos, scale):
+    """Rows q [n, Hq, D] at positions pos over keys and values [T, Hkv, D]: outputs and log-sums."""
+    n, Hq, D = q.shape
+    T, Hkv = k.shape[:2]
+    g = Hq // Hkv
+    out, lse = torch.empty_like(q), q.new_empty(n, Hq)
+    rows = max(1, (1 << 28) // (T * g))
+    at = torch.arange(T, device=q.device)
+    for h in range(Hkv):
+        for r in range(0, n, rows):
+            x = q[r:r + rows, h * g:(h + 1) * g]
+            score = (x.reshape(-1, D) @ k[:, h].T).view(-1, g, T) * scale
+            score.masked_fill_(at > pos[r:r + rows, None, None], -math.inf)
+            total = score.logsumexp(-1)
+            lse[r:r + rows, h * g:(h + 1) * g] = total
+            out[r:r + rows, h * g:(h + 1) * g] = (score.sub_(total[..., None]).exp_().view(-1, T) @ v[:, h]).view(-1, g, D)
+    return out, lse
+
+
+def exact(case, seed):
+    """The outputs of run() in fp64, nothing rounded on the way; None for 8-bit codes."""
+    op, B = case["op"], case["page"]
+    if op == "fp8_store":
+        return None
+    s = prepare(case, seed)
+    w = s.w
+    gpu = lambda x: torch.as_tensor(np.asarray(x), dtype=torch.int64, device=DEVICE)   # noqa: E731
+    T = w.seq_len
+    page_off = np.concatenate([[0], np.cumsum(-(-T // B))])
+    slots = [gpu(w.free_pages[page_off[r] + np.arange(T[r]) // B].astype(np.int64) * B + np.arange(T[r]) % B) for r in range(len(T))]
+    pos = [gpu(w.recompute_pos[w.recompute_off[r]:w.recompute_off[r + 1]]) for r in range(len(T))]
+    src, dst, shift, kept, kept_row = [], [], [], [], []
+    for r in range(len(T)):
+        for u in range(w.unit_off[r], w.unit_off[r + 1]):
+            i, first = np.arange(w.unit_len[u]), w.unit_page_off[u]
+            if w.unit_page_off[u + 1] > first:
+                src.append(gpu(w.unit_pages[first + i // B].astype(np.int64) * B + i % B))
+                dst.append(slots[r][w.unit_target_pos[u]:w.unit_target_pos[u] + len(i)])
+                shift.append(gpu(w.unit_target_pos[u] + i - w.unit_cached_pos[u] - w.unit_cached_stride[u] * i))
+            elif op == "extend":
+                pages = w.unit_retain_pages[w.unit_retain_page_off[u]:]
+                kept.append(gpu(pages[i // B].astype(np.int64) * B + i % B))
+                row = w.recompute_off[r] + np.searchsorted(w.recompute_pos[w.recompute_off[r]:w.recompute_off[r + 1]], w.unit_target_pos[u])
+                kept_row.append(gpu(row + i))
+    fresh = torch.cat([slots[r][pos[r]] for r in range(len(T))])
+
+    def layer(k, v, k_src, v_src, q, k_new, v_new):
+        rows = lambda t: t.to(DEVICE).flatten(0, 1).double()                           # noqa: E731
+        D = case["head_dim"]
+        k, v, q, k_raw, v_new = rows(k), rows(v), q.to(DEVICE).double(), k_new.to(DEVICE).double(), v_new.to(DEVICE).double()
+        if src:
+            at, to = torch.cat(src), torch.cat(dst)
+            if k_src is None:
+                rk, rv = k[at], v[at]
+            else:
+                rk, rv = ((t.to(DEVICE).flatten(0, 1)[at].view(torch.float8_e4m3fn).double() * SCALE8) if t.dtype == torch.uint8 else
+                          t.to(DEVICE).flatten(0, 1)[at].double() for t in (k_src, v_src))
+            k[to], v[to] = _rotated(rk, torch.cat(shift), case), rv
+        k_new = k_raw
+        if op == "extend":
+            every = torch.cat(pos)
+            q, k_new = _rotated(q, every, case), _rotated(k_raw, every, case)
+        k[fresh], v[fresh] = k_new, v_new
+        if kept:
+            k[torch.cat(kept)], v[torch.cat(kept)] = k_raw[torch.cat(kept_row)], v_new[torch.cat(kept_row)]
+        parts = [_attended(q[w.recompute_off[r]:w.recompute_off[r + 1]], k[slots[r]], v[slots[r]], pos[r], 1.0 / math.sqrt(D))
+                 for r in range(len(T))]
+        pool = (-1, B) + tuple(k.shape[1:])
+        return k.view(pool), v.view(pool), torch.cat([p[0] for p in parts]), torch.cat([p[1] for p in parts]), q
+
+    k_src, v_src = getattr(s, "k_src", None), getattr(s, "v_src", None)
+    if op == "prefill":
+        each = [layer(s.k[l], s.v[l], None, None, s.q[l], s.k_new[l], s.v_new[l]) for l in range(s.layers)]
+        k, v, out, lse, _ = (torch.stack(t) for t in zip(*each))
+        return {"k": k, "v": v, "out": out, "lse": lse, "status": None}
+    k, v, out, lse, q = layer(s.k, s.v, k_src, v_src, s.q, s.k_new, s.v_new)
+    result = {"k": None if op == "key8" else k, "v": v, "out": out, "lse": lse}
+    if op == "extend":
+        result["q"] = q
+    return result
