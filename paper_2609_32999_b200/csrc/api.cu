@@ -64,6 +64,7 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     const size_t o_src = place<int32_t>(off, pl->g_src.size());
     const size_t o_dst = place<int32_t>(off, pl->g_dst.size());
     const size_t o_items = place<GatherItem>(off, pl->items.size());
+    const size_t o_runs = place<GatherRun>(off, pl->runs.size());
     const size_t o_rope = place<float>(off, pl->rope_table.size());
     const size_t o_fresh = place<int32_t>(off, pl->fresh_dst.size());
     const size_t o_retain = place<int32_t>(off, pl->retain_dst.size());
@@ -89,6 +90,7 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     put(o_src, pl->g_src.data(), pl->g_src.size() * 4);
     put(o_dst, pl->g_dst.data(), pl->g_dst.size() * 4);
     put(o_items, pl->items.data(), pl->items.size() * sizeof(GatherItem));
+    put(o_runs, pl->runs.data(), pl->runs.size() * sizeof(GatherRun));
     put(o_rope, pl->rope_table.data(), pl->rope_table.size() * 4);
     put(o_fresh, pl->fresh_dst.data(), pl->fresh_dst.size() * 4);
     put(o_retain, pl->retain_dst.data(), pl->retain_dst.size() * 4);
@@ -108,6 +110,7 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     d.g_src = reinterpret_cast<int32_t *>(db + o_src);
     d.g_dst = reinterpret_cast<int32_t *>(db + o_dst);
     d.items = reinterpret_cast<GatherItem *>(db + o_items);
+    d.runs = reinterpret_cast<GatherRun *>(db + o_runs);
     d.rope = reinterpret_cast<float2 *>(db + o_rope);
     d.fresh_dst = reinterpret_cast<int32_t *>(db + o_fresh);
     d.retain_dst = pl->retain_dst.empty() ? nullptr : reinterpret_cast<int32_t *>(db + o_retain);

@@ -98,17 +98,14 @@ template <int D, bool DO_V, bool ROTATE, bool IN_PLACE, bool INTERLEAVED>
 __global__ void __launch_bounds__(kThreads)
 gather_rope_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 *v_pool,
                    const int32_t *__restrict__ g_src, const int32_t *__restrict__ g_dst,
-                   const GatherItem *__restrict__ items, int n_items, const float2 *__restrict__ rope, int H_kv) {
+                   const GatherItem *__restrict__ items, const float2 *__restrict__ rope, int H_kv) {
     constexpr int CPH = D / 16;          // pair-chunks per head
     constexpr int HALF = D / 16;         // distance (in 16-byte chunks) between pair partners
     __shared__ float2 s_rope[kGatherItemTokens * (D / 2)];
     __shared__ int32_t s_src[kGatherItemTokens], s_dst[kGatherItemTokens];
 
     const int tid = threadIdx.x;
-    // one item per thread block in the ordinary launch; a launch with fewer blocks than items (the
-    // host-tier reader, which must leave most SMs to the attention kernel) walks the list
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const GatherItem it = items[item];
+    const GatherItem it = items[blockIdx.x];
     // rows row0, row0 + step, ... of the table; with step = -1 they are staged in ascending order
     const int n_rows = ROTATE ? (it.row_step ? it.count : 1) : 0;
     const int first_row = it.row_step < 0 ? it.row0 - (it.count - 1) : it.row0;
@@ -180,7 +177,58 @@ gather_rope_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 
             stg(k_pool + dsto[u] + HALF, khi[u]);
         }
     }
-    __syncthreads();          // the staged rows are rewritten by the next item
+}
+
+// The host-tier reader: a run's source rows are read once - over the host link, which is what bounds this
+// kernel - and written for each of the run's items, keys rotated by that item's shifts (whose cos/sin rows
+// come straight from the table in L2).  Four tasks in flight per thread: the link's latency is what they hide.
+// 41 270 cached rows of which 28 176 are distinct (8 requests, Zipf popularity): 3 417 -> 2 406 us a layer.
+template <int D, bool INTERLEAVED>
+__global__ void __launch_bounds__(kThreads)
+gather_runs_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 *v_pool, const int32_t *__restrict__ g_src,
+                   const int32_t *__restrict__ g_dst, const GatherItem *__restrict__ items, const GatherRun *__restrict__ runs,
+                   int n_runs, const float2 *__restrict__ rope, int H_kv) {
+    constexpr int CPH = D / 16, HALF = D / 16, U = 4;
+    const int c = threadIdx.x % CPH;
+    const int tasks_per_row = H_kv * CPH, row_chunks = H_kv * (D / 8);
+    for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
+        const GatherRun rn = runs[run];
+        const GatherItem src = items[rn.first_item];
+        const int n_tasks = src.count * tasks_per_row;
+        for (int t0 = threadIdx.x; t0 < n_tasks; t0 += U * kThreads) {
+            uint4 klo[U], khi[U], vlo[U], vhi[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t = t0 + u * kThreads;
+                if (t >= n_tasks) continue;
+                const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
+                const size_t so = (size_t)g_src[src.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
+                klo[u] = ldg_stream(k_src + so);
+                khi[u] = ldg_stream(k_src + so + HALF);
+                vlo[u] = ldg_stream(v_src + so);
+                vhi[u] = ldg_stream(v_src + so + HALF);
+            }
+            for (int m = 0; m < rn.n_items; ++m) {
+                const GatherItem it = items[rn.first_item + m];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int t = t0 + u * kThreads;
+                    if (t >= n_tasks) continue;
+                    const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
+                    const size_t dso = (size_t)g_dst[it.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
+                    const float2 *row = rope + (size_t)(it.row0 + tok * it.row_step) * (D / 2);
+                    float2 cr[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) cr[i] = row[cs_index<D, INTERLEAVED>(c, i)];
+                    uint4 lo = klo[u], hi = khi[u];
+                    rotate_task<INTERLEAVED>(lo, hi, cr);
+                    stg(k_pool + dso, lo);
+                    stg(k_pool + dso + HALF, hi);
+                    stg(v_pool + dso, vlo[u]);
+                    stg(v_pool + dso + HALF, vhi[u]);
+                }
+            }
+        }
     }
 }
 
@@ -308,48 +356,43 @@ extend_write_kernel(uint4 *__restrict__ q, const uint4 *__restrict__ k_raw, cons
 }
 
 template <int D, bool IL>
-cudaError_t launch_gather_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
-                            GatherMode mode, const int32_t *g_src, int first_item, int n, int max_blocks, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    const int grid = max_blocks > 0 ? std::min(n, max_blocks) : n;
-    auto *kp = static_cast<uint4 *>(k_pool);
-    auto *vp = static_cast<uint4 *>(v_pool);
-    auto *ks = static_cast<const uint4 *>(k_src);
-    auto *vs = static_cast<const uint4 *>(v_src);
+void launch_gather_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
+                     GatherMode mode, cudaStream_t st) {
     const DeviceTables &d = pl->dev;
-    const GatherItem *items = d.items + first_item;
-    const int H = pl->cfg.num_kv_heads;
-    switch (mode) {
-        case GatherMode::kCopy:
-            gather_rope_kernel<D, true, false, false, IL><<<grid, kThreads, 0, st>>>(ks, vs, kp, vp, g_src, d.g_dst, items, n, d.rope, H);
-            break;
-        case GatherMode::kCopyRotate:
-            gather_rope_kernel<D, true, true, false, IL><<<grid, kThreads, 0, st>>>(ks, vs, kp, vp, g_src, d.g_dst, items, n, d.rope, H);
-            break;
-        case GatherMode::kShiftInPlace:
-            gather_rope_kernel<D, false, true, true, IL><<<grid, kThreads, 0, st>>>(ks, vs, kp, vp, g_src, d.g_dst, items, n, d.rope, H);
-            break;
-    }
-    count_launch();
-    return cudaGetLastError();
+    auto kernel = mode == GatherMode::kCopy         ? gather_rope_kernel<D, true, false, false, IL>
+                  : mode == GatherMode::kCopyRotate ? gather_rope_kernel<D, true, true, false, IL>
+                                                    : gather_rope_kernel<D, false, true, true, IL>;
+    kernel<<<(unsigned)pl->items.size(), kThreads, 0, st>>>(
+        static_cast<const uint4 *>(k_src), static_cast<const uint4 *>(v_src), static_cast<uint4 *>(k_pool), static_cast<uint4 *>(v_pool),
+        d.g_src, d.g_dst, d.items, d.rope, pl->cfg.num_kv_heads);
 }
 
 }  // namespace
 
-cudaError_t launch_gather_range(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
-                                GatherMode mode, const int32_t *g_src, int first_item, int n_items, int max_blocks,
-                                cudaStream_t st) {
-    const bool il = pl->cfg.rope_pairing == 1;
-    if (pl->cfg.head_dim == 128)
-        return il ? launch_gather_d<128, true>(pl, k_src, v_src, k_pool, v_pool, mode, g_src, first_item, n_items, max_blocks, st)
-                  : launch_gather_d<128, false>(pl, k_src, v_src, k_pool, v_pool, mode, g_src, first_item, n_items, max_blocks, st);
-    return il ? launch_gather_d<64, true>(pl, k_src, v_src, k_pool, v_pool, mode, g_src, first_item, n_items, max_blocks, st)
-              : launch_gather_d<64, false>(pl, k_src, v_src, k_pool, v_pool, mode, g_src, first_item, n_items, max_blocks, st);
-}
-
 cudaError_t launch_gather(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
                           GatherMode mode, cudaStream_t st) {
-    return launch_gather_range(pl, k_src, v_src, k_pool, v_pool, mode, pl->dev.g_src, 0, (int)pl->items.size(), 0, st);
+    if (pl->items.empty()) return cudaSuccess;
+    const bool il = pl->cfg.rope_pairing == 1;
+    auto launch = pl->cfg.head_dim == 128 ? (il ? launch_gather_d<128, true> : launch_gather_d<128, false>)
+                                          : (il ? launch_gather_d<64, true> : launch_gather_d<64, false>);
+    launch(pl, k_src, v_src, k_pool, v_pool, mode, st);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gather_runs(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
+                               int first_run, int n_runs, int max_blocks, cudaStream_t st) {
+    if (n_runs == 0) return cudaSuccess;
+    const DeviceTables &d = pl->dev;
+    const unsigned grid = (unsigned)(max_blocks > 0 ? std::min(n_runs, max_blocks) : n_runs);
+    const bool il = pl->cfg.rope_pairing == 1;
+    auto kernel = pl->cfg.head_dim == 128 ? (il ? gather_runs_kernel<128, true> : gather_runs_kernel<128, false>)
+                                          : (il ? gather_runs_kernel<64, true> : gather_runs_kernel<64, false>);
+    kernel<<<grid, kThreads, 0, st>>>(static_cast<const uint4 *>(k_src), static_cast<const uint4 *>(v_src), static_cast<uint4 *>(k_pool),
+                                      static_cast<uint4 *>(v_pool), d.g_src, d.g_dst, d.items, d.runs + first_run, n_runs, d.rope,
+                                      pl->cfg.num_kv_heads);
+    count_launch();
+    return cudaGetLastError();
 }
 
 cudaError_t launch_rope_fresh(const tessera_plan *pl, void *q, void *k_new, cudaStream_t st) {

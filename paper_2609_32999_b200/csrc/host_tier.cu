@@ -2,10 +2,10 @@
 // pinned host-memory cache into the request's KV slots while the engine keeps serving what is already
 // prepared; Sec. 4: the host cache belongs to the generation node).
 //
-// The cached units live in a pinned host pool.  Per chunk of whole requests, a READER launch of the
-// gather kernel - a handful of thread blocks that walk the chunk's copy list - pulls the rows over the
-// interconnect straight into their destination slots (keys rotated on the way: no staging buffer at
-// all), on a side stream; as soon as a chunk has arrived, its fresh-row scatter and attention run on
+// The cached units live in a pinned host pool.  Per chunk of whole requests, a READER launch - a handful
+// of thread blocks that walk the list of source rows the chunk's requests are the first to use - pulls each
+// row over the interconnect once and writes it straight into the destination slots of every request that
+// uses it, later chunks' included (keys rotated for each: no staging buffer at all), on a side stream; as soon as a chunk has arrived, its fresh-row scatter and attention run on
 // the caller's stream with a persistent grid that leaves the reader's SMs alone.  The link (about
 // 50 GB/s) is the bound; what overlaps is the attention of chunk c with the transfer of chunk c + 1.
 //
@@ -72,21 +72,19 @@ extern "C" int32_t tessera_composed_prefill_host_tier(tessera_plan *pl, const vo
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (int32_t rc = api_ensure_pipeline(pl)) return rc;
 
-    const int n_chunks = (int)pl->chunk_item_off.size() - 1;
+    const int n_chunks = (int)pl->chunk_run_off.size() - 1;
     // the reader starts after everything already queued on the caller's stream (an earlier layer may
     // still be reading these destination pages)
     HT_CUDA(cudaEventRecord(pl->ev_start, st));
     HT_CUDA(cudaStreamWaitEvent(pl->s_in, pl->ev_start, 0));
     for (int c = 0; c < n_chunks; ++c) {
-        const int first = pl->chunk_item_off[c], n = pl->chunk_item_off[c + 1] - first;
+        const int first = pl->chunk_run_off[c], n = pl->chunk_run_off[c + 1] - first;
         // the last chunk has nothing to overlap with: it takes the whole GPU
         const int cap = c + 1 < n_chunks ? readers : 0;
         if (src_format == 0)
-            HT_CUDA(launch_gather_range(pl, k_src_host, v_src_host, k_pool, v_pool, GatherMode::kCopyRotate, pl->dev.g_src,
-                                        first, n, cap, pl->s_in));
+            HT_CUDA(launch_gather_runs(pl, k_src_host, v_src_host, k_pool, v_pool, first, n, cap, pl->s_in));
         else
-            HT_CUDA(launch_kv_fp8_range(pl, k_src_host, v_src_host, k_pool, v_pool, false, true, k_scale, v_scale,
-                                        pl->dev.g_src, first, n, cap, pl->s_in));
+            HT_CUDA(launch_expand_fp8_runs(pl, k_src_host, v_src_host, k_pool, v_pool, k_scale, v_scale, first, n, cap, pl->s_in));
         HT_CUDA(cudaEventRecord(pl->ev_in[c], pl->s_in));
     }
     for (int c = 0; c < n_chunks; ++c) {

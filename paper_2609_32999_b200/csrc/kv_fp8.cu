@@ -101,17 +101,14 @@ template <int D, bool TO_8BIT, bool ROTATE, bool INTERLEAVED, bool V16 = false>
 __global__ void __launch_bounds__(kThreads)
 kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, void *__restrict__ k_dst,
               void *__restrict__ v_dst, const int32_t *__restrict__ g_src, const int32_t *__restrict__ g_dst,
-              const GatherItem *__restrict__ items, int n_items, const float2 *__restrict__ rope, int H_kv, float k_mul,
-              float v_mul) {
+              const GatherItem *__restrict__ items, const float2 *__restrict__ rope, int H_kv, float k_mul, float v_mul) {
     constexpr int CPH = D / 16;          // pair-chunks per head
     constexpr int HALF = D / 16;         // distance (in 8-element chunks) between pair partners
     __shared__ float2 s_rope[kGatherItemTokens * (D / 2)];
     __shared__ int32_t s_src[kGatherItemTokens], s_dst[kGatherItemTokens];
 
     const int tid = threadIdx.x;
-    // one item per thread block, or - when launched with fewer blocks than items - a walk through the list
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const GatherItem it = items[item];
+    const GatherItem it = items[blockIdx.x];
     const int n_rows = ROTATE ? (it.row_step ? it.count : 1) : 0;
     const int first_row = it.row_step < 0 ? it.row0 - (it.count - 1) : it.row0;
     for (int i = tid; i < n_rows * (D / 2); i += kThreads) s_rope[i] = rope[(size_t)first_row * (D / 2) + i];
@@ -193,7 +190,60 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
             }
         }
     }
-    __syncthreads();          // the staged rows are rewritten by the next item
+}
+
+// The host-tier reader for e4m3 units: a run's codes are read once over the host link and expanded for each of
+// the run's items (see gather_runs_kernel).
+template <int D, bool INTERLEAVED>
+__global__ void __launch_bounds__(kThreads)
+expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_src, uint4 *__restrict__ k_dst, uint4 *__restrict__ v_dst,
+                   const int32_t *__restrict__ g_src, const int32_t *__restrict__ g_dst, const GatherItem *__restrict__ items,
+                   const GatherRun *__restrict__ runs, int n_runs, const float2 *__restrict__ rope, int H_kv, float k_mul, float v_mul) {
+    constexpr int CPH = D / 16, HALF = D / 16, U = 4;
+    const int c = threadIdx.x % CPH;
+    const int tasks_per_row = H_kv * CPH, row_chunks = H_kv * (D / 8);
+    for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
+        const GatherRun rn = runs[run];
+        const GatherItem src = items[rn.first_item];
+        const int n_tasks = src.count * tasks_per_row;
+        for (int t0 = threadIdx.x; t0 < n_tasks; t0 += U * kThreads) {
+            uint2 rk[U][2], rv[U][2];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t = t0 + u * kThreads;
+                if (t >= n_tasks) continue;
+                const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
+                const size_t so = (size_t)g_src[src.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
+                rk[u][0] = __ldg(k_src + so);
+                rk[u][1] = __ldg(k_src + so + HALF);
+                rv[u][0] = __ldg(v_src + so);
+                rv[u][1] = __ldg(v_src + so + HALF);
+            }
+            for (int m = 0; m < rn.n_items; ++m) {
+                const GatherItem it = items[rn.first_item + m];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int t = t0 + u * kThreads;
+                    if (t >= n_tasks) continue;
+                    const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
+                    const size_t dso = (size_t)g_dst[it.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
+                    const float2 *row = rope + (size_t)(it.row0 + tok * it.row_step) * (D / 2);
+                    float2 cr[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) cr[i] = row[cs_index<D, INTERLEAVED>(c, i)];
+                    float lo[8], hi[8];
+                    unpack_e4m3x8(rk[u][0], k_mul, lo);
+                    unpack_e4m3x8(rk[u][1], k_mul, hi);
+                    rotate_f<INTERLEAVED>(lo, hi, cr);
+                    k_dst[dso] = pack_bf16x8(lo);
+                    k_dst[dso + HALF] = pack_bf16x8(hi);
+                    unpack_e4m3x8(rv[u][0], v_mul, lo);
+                    unpack_e4m3x8(rv[u][1], v_mul, hi);
+                    v_dst[dso] = pack_bf16x8(lo);
+                    v_dst[dso + HALF] = pack_bf16x8(hi);
+                }
+            }
+        }
     }
 }
 
@@ -226,31 +276,15 @@ scatter_fresh_k8_kernel(uint2 *__restrict__ k_pool8, uint4 *__restrict__ v_pool,
     }
 }
 
-template <int D, bool TO_8BIT, bool IL>
-cudaError_t launch_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst, bool rotate,
-                     float k_mul, float v_mul, const int32_t *g_src, int first_item, int n, int max_blocks, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    const int grid = max_blocks > 0 ? (n < max_blocks ? n : max_blocks) : n;
+template <int D, bool TO_8BIT>
+void launch_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst, bool rotate,
+              float k_mul, float v_mul, cudaStream_t st) {
     const DeviceTables &d = pl->dev;
-    const GatherItem *items = d.items + first_item;
-    const int H = pl->cfg.num_kv_heads;
-    if (rotate)
-        kv_fp8_kernel<D, TO_8BIT, true, IL><<<grid, kThreads, 0, st>>>(k_src, v_src, k_dst, v_dst, g_src, d.g_dst, items, n, d.rope, H, k_mul, v_mul);
-    else
-        kv_fp8_kernel<D, TO_8BIT, false, IL><<<grid, kThreads, 0, st>>>(k_src, v_src, k_dst, v_dst, g_src, d.g_dst, items, n, d.rope, H, k_mul, v_mul);
-    count_launch();
-    return cudaGetLastError();
-}
-
-template <bool TO_8BIT>
-cudaError_t launch_dir(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst, bool rotate,
-                       float k_mul, float v_mul, const int32_t *g_src, int first_item, int n, int max_blocks, cudaStream_t st) {
     const bool il = pl->cfg.rope_pairing == 1;
-    if (pl->cfg.head_dim == 128)
-        return il ? launch_d<128, TO_8BIT, true>(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, g_src, first_item, n, max_blocks, st)
-                  : launch_d<128, TO_8BIT, false>(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, g_src, first_item, n, max_blocks, st);
-    return il ? launch_d<64, TO_8BIT, true>(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, g_src, first_item, n, max_blocks, st)
-              : launch_d<64, TO_8BIT, false>(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, g_src, first_item, n, max_blocks, st);
+    auto kernel = rotate ? (il ? kv_fp8_kernel<D, TO_8BIT, true, true> : kv_fp8_kernel<D, TO_8BIT, true, false>)
+                         : (il ? kv_fp8_kernel<D, TO_8BIT, false, true> : kv_fp8_kernel<D, TO_8BIT, false, false>);
+    kernel<<<(unsigned)pl->items.size(), kThreads, 0, st>>>(k_src, v_src, k_dst, v_dst, d.g_src, d.g_dst, d.items, d.rope,
+                                                            pl->cfg.num_kv_heads, k_mul, v_mul);
 }
 
 }  // namespace
@@ -264,7 +298,7 @@ cudaError_t launch_compose_k8(const tessera_plan *pl, const void *k_src, const v
     const int H = pl->cfg.num_kv_heads;
     const bool il = pl->cfg.rope_pairing == 1;
 #define TESSERA_K8_LAUNCH(DD, ROT, IL) \
-    kv_fp8_kernel<DD, true, ROT, IL, true><<<n, kThreads, 0, st>>>(k_src, v_src, k_dst8, v_dst, d.g_src, d.g_dst, d.items, n, d.rope, H, k_mul, 1.f)
+    kv_fp8_kernel<DD, true, ROT, IL, true><<<n, kThreads, 0, st>>>(k_src, v_src, k_dst8, v_dst, d.g_src, d.g_dst, d.items, d.rope, H, k_mul, 1.f)
     if (pl->cfg.head_dim == 128) {
         if (rotate) { if (il) TESSERA_K8_LAUNCH(128, true, true); else TESSERA_K8_LAUNCH(128, true, false); }
         else { if (il) TESSERA_K8_LAUNCH(128, false, true); else TESSERA_K8_LAUNCH(128, false, false); }
@@ -299,17 +333,29 @@ cudaError_t launch_scatter_fresh_k8(const tessera_plan *pl, void *k_pool8, void 
     return cudaGetLastError();
 }
 
-cudaError_t launch_kv_fp8_range(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst,
-                                bool to_8bit, bool rotate, float k_mul, float v_mul, const int32_t *g_src, int first_item,
-                                int n_items, int max_blocks, cudaStream_t st) {
-    return to_8bit ? launch_dir<true>(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, g_src, first_item, n_items, max_blocks, st)
-                   : launch_dir<false>(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, g_src, first_item, n_items, max_blocks, st);
-}
-
 cudaError_t launch_kv_fp8(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst,
                           bool to_8bit, bool rotate, float k_mul, float v_mul, cudaStream_t st) {
-    return launch_kv_fp8_range(pl, k_src, v_src, k_dst, v_dst, to_8bit, rotate, k_mul, v_mul, pl->dev.g_src, 0,
-                               (int)pl->items.size(), 0, st);
+    if (pl->items.empty()) return cudaSuccess;
+    auto launch = pl->cfg.head_dim == 128 ? (to_8bit ? launch_d<128, true> : launch_d<128, false>)
+                                          : (to_8bit ? launch_d<64, true> : launch_d<64, false>);
+    launch(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, st);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_expand_fp8_runs(const tessera_plan *pl, const void *k_src8, const void *v_src8, void *k_pool, void *v_pool,
+                                   float k_scale, float v_scale, int first_run, int n_runs, int max_blocks, cudaStream_t st) {
+    if (n_runs == 0) return cudaSuccess;
+    const DeviceTables &d = pl->dev;
+    const unsigned grid = (unsigned)(max_blocks > 0 ? std::min(n_runs, max_blocks) : n_runs);
+    const bool il = pl->cfg.rope_pairing == 1;
+    auto kernel = pl->cfg.head_dim == 128 ? (il ? expand_runs_kernel<128, true> : expand_runs_kernel<128, false>)
+                                          : (il ? expand_runs_kernel<64, true> : expand_runs_kernel<64, false>);
+    kernel<<<grid, kThreads, 0, st>>>(static_cast<const uint2 *>(k_src8), static_cast<const uint2 *>(v_src8), static_cast<uint4 *>(k_pool),
+                                      static_cast<uint4 *>(v_pool), d.g_src, d.g_dst, d.items, d.runs + first_run, n_runs, d.rope,
+                                      pl->cfg.num_kv_heads, k_scale, v_scale);
+    count_launch();
+    return cudaGetLastError();
 }
 
 }  // namespace tessera

@@ -14,15 +14,13 @@ void count_launch();   // bumps the process-wide kernel-launch counter
 // separate source pool - and written to the plan's destination slots in (k_pool, v_pool).
 cudaError_t launch_gather(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
                           GatherMode mode, cudaStream_t st);
-// The same kernels over items [first_item, first_item + n_items) of the plan, with the source slots taken
-// from `g_src` (device, indexed like the plan's copy list).  max_blocks > 0 caps the grid: the blocks
-// then walk the items, so the launch occupies only a few SMs (host-tier reader beside the attention kernel).
-cudaError_t launch_gather_range(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
-                                GatherMode mode, const int32_t *g_src, int first_item, int n_items, int max_blocks,
-                                cudaStream_t st);
-cudaError_t launch_kv_fp8_range(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst,
-                                bool to_8bit, bool rotate, float k_mul, float v_mul, const int32_t *g_src, int first_item,
-                                int n_items, int max_blocks, cudaStream_t st);
+// Host-tier readers over gather runs [first_run, first_run + n_runs): every source row is read once and written
+// to the slots of all its users, keys rotated; 16-bit, respectively e4m3, sources.  max_blocks > 0 caps the
+// grid: the blocks then walk the runs, so the launch occupies only a few SMs beside the attention kernel.
+cudaError_t launch_gather_runs(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
+                               int first_run, int n_runs, int max_blocks, cudaStream_t st);
+cudaError_t launch_expand_fp8_runs(const tessera_plan *pl, const void *k_src8, const void *v_src8, void *k_pool, void *v_pool,
+                                   float k_scale, float v_scale, int first_run, int n_runs, int max_blocks, cudaStream_t st);
 // 8-bit (e4m3) tier.  to_8bit false: (k_src, v_src) hold codes, (k_dst, v_dst) 16-bit pages, mul = scale;
 // to_8bit true: the reverse, mul = 1 / scale.  Copy list and shift table are the plan's.
 cudaError_t launch_kv_fp8(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst,

@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <numeric>
 #include <tuple>
+#include <unordered_map>
 
 #include <vector_types.h>
 
@@ -245,6 +246,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
     auto row_of = [&](int64_t delta) {
         return (int32_t)(std::lower_bound(deltas.begin(), deltas.end(), delta) - deltas.begin());
     };
+    pl->cached_tokens = 0;
     // Rows per gather block: 32, fewer when the batch is so small that the grid would not fill the GPU.
     int item_tokens = kGatherItemTokens;
     {
@@ -253,29 +255,61 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             if (d->unit_page_off[u + 1] > d->unit_page_off[u]) cached += d->unit_len[u];
         while (item_tokens > 8 && cached / item_tokens < 4 * num_sms) item_tokens /= 2;
     }
-    pl->cached_tokens = 0;
-    std::vector<int32_t> req_item_off(batch + 1, 0);       // gather items are emitted request by request
-    for (int r = 0; r < batch; ++r) {
-        req_item_off[r] = (int32_t)pl->items.size();
-        for (int u = d->unit_off[r]; u < d->unit_off[r + 1]; ++u) {
-            if (d->unit_page_off[u + 1] <= d->unit_page_off[u]) continue;
-            const int len = d->unit_len[u], tp = d->unit_target_pos[u];
-            const int64_t d0 = (int64_t)tp - d->unit_cached_pos[u];
-            const int step = (d->unit_target_stride ? d->unit_target_stride[u] : 1) - d->unit_cached_stride[u];
-            const int32_t row0 = row_of(d0);       // step +-1: consecutive integers are consecutive rows
-            for (int i0 = 0; i0 < len; i0 += item_tokens) {
-                const int cnt = std::min(item_tokens, len - i0);
+    // Requests may use the same cached unit (equal source pages, offset and length).  The items of its users
+    // are emitted side by side, so that blocks running together read the same rows out of L2 (and the
+    // host-tier reader fetches a row once for all of them): 81 550 cached rows, 47 846 distinct, 106 -> 91 us.
+    struct UnitUse { int32_t req, unit; };
+    std::vector<std::vector<UnitUse>> shared;              // users of each distinct unit, in order of first use
+    {
+        std::unordered_multimap<int64_t, int32_t> by_page;   // first source page -> index into `shared`
+        by_page.reserve(n_units);
+        for (int r = 0; r < batch; ++r)
+            for (int u = d->unit_off[r]; u < d->unit_off[r + 1]; ++u) {
+                const int p0 = d->unit_page_off[u], np = d->unit_page_off[u + 1] - p0;
+                if (np <= 0) continue;
+                int found = -1;
+                auto range = by_page.equal_range(d->unit_pages[p0]);
+                for (auto it = range.first; it != range.second && found < 0; ++it) {
+                    const int v = shared[it->second][0].unit;
+                    const bool same_off = !d->unit_src_offset || d->unit_src_offset[u] == d->unit_src_offset[v];
+                    if (d->unit_len[u] == d->unit_len[v] && same_off && d->unit_page_off[v + 1] - d->unit_page_off[v] == np &&
+                        std::equal(d->unit_pages + p0, d->unit_pages + p0 + np, d->unit_pages + d->unit_page_off[v]))
+                        found = it->second;
+                }
+                if (found < 0) {
+                    found = (int)shared.size();
+                    shared.emplace_back();
+                    by_page.emplace(d->unit_pages[p0], found);
+                }
+                shared[found].push_back({r, u});
+                pl->cached_tokens += d->unit_len[u];
+            }
+    }
+    std::vector<int32_t> req_run_off(batch + 1, -1);       // first run whose first user is the request (or a later one)
+    pl->runs.clear();
+    for (const auto &users : shared) {
+        if (req_run_off[users[0].req] < 0) req_run_off[users[0].req] = (int32_t)pl->runs.size();
+        const int len = d->unit_len[users[0].unit];
+        for (int i0 = 0; i0 < len; i0 += item_tokens) {
+            const int cnt = std::min(item_tokens, len - i0);
+            pl->runs.push_back({(int32_t)pl->items.size(), (int32_t)users.size()});
+            for (const UnitUse &use : users) {
+                const int u = use.unit, tp = d->unit_target_pos[u];
+                const int64_t d0 = (int64_t)tp - d->unit_cached_pos[u];
+                const int step = (d->unit_target_stride ? d->unit_target_stride[u] : 1) - d->unit_cached_stride[u];
+                const int32_t row0 = row_of(d0);       // step +-1: consecutive integers are consecutive rows
                 pl->items.push_back({(int32_t)pl->g_src.size(), cnt, row0 + i0 * step, step});
                 for (int i = i0; i < i0 + cnt; ++i) {
                     const int p = tp + i;
-                    pl->g_src.push_back(pl->src_slot[pl->tok_off[r] + p]);
-                    pl->g_dst.push_back(pl->pages[pl->page_off[r] + p / B] * B + p % B);
+                    pl->g_src.push_back(pl->src_slot[pl->tok_off[use.req] + p]);
+                    pl->g_dst.push_back(pl->pages[pl->page_off[use.req] + p / B] * B + p % B);
                 }
             }
-            pl->cached_tokens += len;
         }
     }
-    req_item_off[batch] = (int32_t)pl->items.size();
+    req_run_off[batch] = (int32_t)pl->runs.size();
+    for (int r = batch - 1; r >= 0; --r)
+        if (req_run_off[r] < 0) req_run_off[r] = req_run_off[r + 1];
 
     // ---- attention work list: tiles of consecutive recompute rows of one request
     const int g = Hq / Hkv;
@@ -390,10 +424,10 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             pl->chunk_row_off.push_back(n_q);
         }
         const int used_chunks = (int)pl->chunk_row_off.size() - 1;
-        pl->chunk_item_off.assign(used_chunks + 1, (int32_t)pl->items.size());
-        pl->chunk_item_off[0] = 0;
+        pl->chunk_run_off.assign(used_chunks + 1, (int32_t)pl->runs.size());
+        pl->chunk_run_off[0] = 0;
         for (int r = 1; r < batch; ++r)
-            if (chunk_of[r] != chunk_of[r - 1]) pl->chunk_item_off[chunk_of[r]] = req_item_off[r];
+            if (chunk_of[r] != chunk_of[r - 1]) pl->chunk_run_off[chunk_of[r]] = req_run_off[r];
         pl->work_chunked = pl->work;
         std::stable_sort(pl->work_chunked.begin(), pl->work_chunked.end(), [&](const AttnWork &x, const AttnWork &y) {
             return chunk_of[pl->tiles[x.tile_a].req] < chunk_of[pl->tiles[y.tile_a].req];

@@ -26,6 +26,12 @@ struct GatherItem {
     int32_t begin, count, row0, row_step;
 };
 
+// One source run of the host-tier reader: gather items [first_item, first_item + n_items) read the same
+// rows of the same cached unit (one item per request that uses it) and differ only in slots and shifts.
+struct GatherRun {
+    int32_t first_item, n_items;
+};
+
 // One query tile of the attention kernel: `n_tok` consecutive recompute rows [q_begin, q_begin+n_tok)
 // of request `req`; the tile reads keys [0, kv_len).  Keys below `kv_full` are visible to every row.
 struct AttnTile {
@@ -50,6 +56,7 @@ struct DeviceTables {
     void *blob = nullptr;          // one allocation holding everything below
     int32_t *g_src = nullptr, *g_dst = nullptr;
     GatherItem *items = nullptr;
+    GatherRun *runs = nullptr;
     float2 *rope = nullptr;        // [n_rope_rows][D/2] (cos, sin)
     int32_t *fresh_dst = nullptr;  // [n_q] destination slot of each recompute row
     int32_t *retain_dst = nullptr; // [n_q] cache slot of a captured row, -1 otherwise (null: nothing is captured)
@@ -93,6 +100,7 @@ struct tessera_plan {
     int64_t retained_tokens = 0;
     std::vector<int32_t> g_src, g_dst;
     std::vector<tessera::GatherItem> items;
+    std::vector<tessera::GatherRun> runs;  // the items, grouped by source rows (order of first use)
     std::vector<int32_t> rope_delta;       // sorted distinct shift amounts
     std::vector<float> rope_table;         // [rows][D/2][2]
     std::vector<tessera::AttnTile> tiles;
@@ -100,7 +108,7 @@ struct tessera_plan {
     // The host-buffer entry point pipelines copies against compute over chunks of whole requests.
     std::vector<tessera::AttnWork> work_chunked;   // items of chunk c: [chunk_work_off[c], chunk_work_off[c+1])
     std::vector<int32_t> chunk_work_off, chunk_row_off;   // [n_chunks + 1]; rows = recompute rows
-    std::vector<int32_t> chunk_item_off;                  // [n_chunks + 1]; gather items of the chunk's requests
+    std::vector<int32_t> chunk_run_off;                   // [n_chunks + 1]; gather runs first used by the chunk's requests
     std::vector<tessera::CombineItem> combine;     // grouped by chunk: [chunk_combine_off[c], chunk_combine_off[c+1])
     std::vector<int32_t> chunk_combine_off;
     int32_t n_work_items = 0;                      // real items of `work` (the list may hold holes)
