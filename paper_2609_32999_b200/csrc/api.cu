@@ -80,7 +80,7 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     const size_t o_status = place<int32_t>(off, 4);
     const size_t o_invf = place<double>(off, pl->inv_freq.size());
     // split-KV workspace: one slot per (tile, KV head, part)
-    const size_t n_slots = pl->max_parts > 1 ? pl->tiles.size() * pl->cfg.num_kv_heads * pl->max_parts : 0;
+    const size_t n_slots = pl->n_slots;
     const size_t o_wsml = place<float2>(off, n_slots * kAttnTileRows);
     const size_t o_wso = place<float>(off, n_slots * kAttnTileRows * pl->cfg.head_dim);
     const size_t table_bytes = o_wsml;    // the workspace behind it needs no upload

@@ -125,7 +125,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                const AttnWork *__restrict__ work, int n_work, const int32_t *__restrict__ q_pos,
                const int32_t *__restrict__ page_off, const int32_t *__restrict__ pages,
                const int32_t *__restrict__ seq_len, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse,
-               int H_q, int g, int H_kv, int page_size, int num_pool_pages, float scale_log2, int max_parts,
+               int H_q, int g, int page_size, int num_pool_pages, float scale_log2,
                float *__restrict__ ws_o, float2 *__restrict__ ws_ml, int *status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -596,9 +596,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             const float l_tot[2] = {quad_sum(l_row[q][0]), quad_sum(l_row[q][1])};
             const uint32_t tO = tmem + kTmemO + q * 128 + lane_base;
             uint32_t o[kD / 2];
-            if (it.wk.n_parts > 1) {
+            if (it.wk.slot_a >= 0) {
                 // split-KV part: unnormalised accumulator, reference maximum and sum go to the workspace
-                const size_t slot = ((size_t)(q ? it.wk.tile_b : it.wk.tile_a) * H_kv + kvh) * max_parts + it.wk.part;
+                const size_t slot = q ? it.wk.slot_b : it.wk.slot_a;
                 if constexpr (kD == 128) tmem_ld_16x256b_x16(tO, o); else tmem_ld_16x256b_x8(tO, o);
                 tmem_wait_ld();
 #pragma unroll
@@ -678,42 +678,48 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
 
 // Merges the parts of a split-KV launch: for every row, O = sum_p O_p 2^(m_p - m) / sum_p l_p 2^(m_p - m)
 // with m = max_p m_p.  One warp per row (lanes walk head_dim), 8 rows per block, kRows / 8 blocks per
-// (tile, KV head) item; all parts of a row are loaded before any is used.
+// (tile, KV head) item; the parts of a row are loaded in batches before any of a batch is used.
 template <int kD>
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const CombineItem *__restrict__ items, const AttnTile *__restrict__ tiles,
                     const float *__restrict__ ws_o, const float2 *__restrict__ ws_ml, __nv_bfloat16 *__restrict__ out,
-                    float *__restrict__ lse, int H_q, int H_kv, int g, int max_parts) {
+                    float *__restrict__ lse, int H_q, int g) {
     constexpr int kBlocksPerItem = kRows / 8;
     const CombineItem it = items[blockIdx.x / kBlocksPerItem];
     const AttnTile t = tiles[it.tile];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = (blockIdx.x % kBlocksPerItem) * 8 + warp;
     if (row >= t.n_tok * g) return;
-    const size_t slot0 = ((size_t)it.tile * H_kv + it.kvh) * max_parts;
-    float2 ml[kSplitMaxParts];
-    float4 o[kSplitMaxParts];
-#pragma unroll
-    for (int p = 0; p < kSplitMaxParts; ++p)
-        if (p < it.n_parts) {
-            ml[p] = ws_ml[(slot0 + p) * kRows + row];
-            o[p] = lane * 4 < kD ? *reinterpret_cast<const float4 *>(ws_o + ((slot0 + p) * kRows + row) * kD + lane * 4)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    float m = -INFINITY;
-#pragma unroll
-    for (int p = 0; p < kSplitMaxParts; ++p)
-        if (p < it.n_parts) m = fmaxf(m, ml[p].x);
+    constexpr int kBatch = 8;          // one batch holds all parts as a rule
+    float m = -INFINITY, l = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    float l = 0.f;
+    for (int p0 = 0; p0 < it.n_parts; p0 += kBatch) {
+        float2 ml[kBatch];
+        float4 o[kBatch];
 #pragma unroll
-    for (int p = 0; p < kSplitMaxParts; ++p)
-        if (p < it.n_parts) {
+        for (int p = 0; p < kBatch; ++p) {
+            // L2 loads: the workspace is rewritten by every launch
+            const size_t r = (size_t)(it.slot0 + p0 + p) * kRows + row;
+            const bool there = p0 + p < it.n_parts;
+            ml[p] = there ? __ldcg(ws_ml + r) : make_float2(-INFINITY, 0.f);
+            o[p] = there && lane * 4 < kD ? __ldcg(reinterpret_cast<const float4 *>(ws_o + r * kD + lane * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float mb = m;
+#pragma unroll
+        for (int p = 0; p < kBatch; ++p) mb = fmaxf(mb, ml[p].x);
+        // the first part holds the key at position 0, which every row sees: mb is finite from the first batch on
+        const float w0 = exp2f(m - mb);
+        m = mb;
+        l *= w0;
+        acc.x *= w0; acc.y *= w0; acc.z *= w0; acc.w *= w0;
+#pragma unroll
+        for (int p = 0; p < kBatch; ++p) {
             const float w = exp2f(ml[p].x - m);
             l += ml[p].y * w;
             acc.x = fmaf(o[p].x, w, acc.x); acc.y = fmaf(o[p].y, w, acc.y);
             acc.z = fmaf(o[p].z, w, acc.z); acc.w = fmaf(o[p].w, w, acc.w);
         }
+    }
     const float inv = 1.f / l;
     const int tok = t.q_begin + row / g, head = it.kvh * g + row % g;
     uint2 pk;
@@ -751,14 +757,14 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
     const unsigned grid = (unsigned)std::min<size_t>(n_work, (size_t)sms);
     attn_tc_kernel<D, kMaxPages, K8><<<grid, kThreads, Geo<D>::kSmemAlloc, st>>>(
         tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.page_off, d.pages, d.seq_len,
-        static_cast<__nv_bfloat16 *>(out), lse, Hq, g, Hkv, ps, pl->num_pool_pages, scale_log2, pl->max_parts, d.ws_o, d.ws_ml, d.status);
+        static_cast<__nv_bfloat16 *>(out), lse, Hq, g, ps, pl->num_pool_pages, scale_log2, d.ws_o, d.ws_ml, d.status);
     count_launch();
-    if (pl->max_parts > 1) {
+    if (!pl->combine.empty()) {
         const int c0 = chunk < 0 ? 0 : pl->chunk_combine_off[chunk];
         const int c1 = chunk < 0 ? (int)pl->combine.size() : pl->chunk_combine_off[chunk + 1];
         if (c1 > c0) {
             attn_combine_kernel<D><<<(c1 - c0) * (kRows / 8), 256, 0, st>>>(d.combine + c0, d.tiles, d.ws_o, d.ws_ml, static_cast<__nv_bfloat16 *>(out),
-                                                                          lse, Hq, Hkv, g, pl->max_parts);
+                                                                          lse, Hq, g);
             count_launch();
         }
     }

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <functional>
 #include <numeric>
 #include <tuple>
 #include <unordered_map>
@@ -21,6 +22,10 @@ std::string fmt(const char *f, long a = 0, long b = 0, long c = 0) {
     snprintf(buf, sizeof buf, f, a, b, c);
     return buf;
 }
+
+// Merge of a split list in SM cycles: the launch and its first loads, and 65 KB of partial results per slot
+// written and read back through L2.
+constexpr int64_t kMergeCycles = 5000, kMergeCyclesPerSlot = 30;
 
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
@@ -342,39 +347,93 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             first = last;
         }
         auto steps_of = [&](int32_t tile) { return (pl->tiles[tile].kv_len + page - 1) / page; };
-        // Split-KV: a batch with fewer items than SMs (a single request, typically) splits each item's
-        // key range into parts that run as separate thread blocks and are merged afterwards.
-        pl->max_parts = 1;
-        if (!pairs.empty() && (int)pairs.size() * Hkv < num_sms) {
-            int longest = 1;
-            for (auto &pr : pairs) longest = std::max(longest, steps_of(pr.second >= 0 ? pr.second : pr.first));
-            const int want = num_sms / ((int)pairs.size() * Hkv);     // stay within one wave of blocks
-            pl->max_parts = std::max(1, std::min({want, kSplitMaxParts, longest / kSplitMinSteps}));
+        // Modelled cycles of an item (clock64 on a B200): item fetch 700, epilogue + first step 3 150 per tile,
+        // 3 180 per step of both tiles, 1 650 per step of one.
+        auto model_cycles = [](int steps_a, int steps_b, int n_tiles) -> int64_t {
+            const int both = std::min(steps_a, steps_b), single = std::max(steps_a, steps_b) - both;
+            return 700 + (int64_t)n_tiles * 3150 + (int64_t)both * 3180 + (int64_t)single * 1650;
+        };
+        // Split-KV: the key ranges of a batch that leaves SMs idle are cut into parts of at most `limit` steps
+        // that run as separate items and are merged afterwards.
+        //   items <= SMs / 2 : the smallest limit whose parts still fit one round (one item per SM).  A common
+        //                      limit, not a common part count: short tiles are not cut as often as long ones
+        //                      (5 312 tokens, 48 items: parts of at most 14 steps before, 9 now; attention
+        //                      39.4 -> 35.7 us; 5 requests of 2 048 tokens, 2 KV heads of 64: the whole layer
+        //                      41.0 -> 28.6 us).
+        //   items <= kSplitMaxRounds x SMs : the limit with the least modelled time, if that is at least 5 %
+        //                      below the uncut list's (168 items of 260 steps take two rounds on 148 SMs; cut in
+        //                      parts they fill all rounds).
+        //   more             : never; the rounds are even enough and the merge only costs.
+        auto parts_of = [&](int steps, int limit) {
+            return std::max(1, std::min({(steps + limit - 1) / limit, kSplitMaxParts, steps / kSplitMinSteps}));
+        };
+        auto long_steps = [&](const std::pair<int32_t, int32_t> &pr) { return steps_of(pr.second >= 0 ? pr.second : pr.first); };
+        int longest = 1;
+        for (auto &pr : pairs) longest = std::max(longest, long_steps(pr));
+        auto items_at = [&](int limit) {
+            int64_t n = 0;
+            for (auto &pr : pairs) n += parts_of(long_steps(pr), limit);
+            return n * Hkv;
+        };
+        // time of the list cut at `limit`: longest-first assignment to the least-loaded SM, plus the merge
+        auto modelled = [&](int limit) -> int64_t {
+            std::vector<int64_t> cost;
+            int64_t slots = 0;
+            for (auto &pr : pairs) {
+                const int sl = long_steps(pr), sa = pr.second >= 0 ? steps_of(pr.first) : 0, parts = parts_of(sl, limit);
+                const int len = (sl + parts - 1) / parts;
+                for (int b0 = 0; b0 < sl; b0 += len) {
+                    const int n_b = std::min(sl, b0 + len) - b0, n_a = std::max(0, std::min(sa, b0 + len) - b0);
+                    cost.insert(cost.end(), Hkv, model_cycles(n_a, n_b, n_a > 0 ? 2 : 1));
+                    if (parts > 1) slots += (n_a > 0 ? 2 : 1) * Hkv;
+                }
+            }
+            std::sort(cost.begin(), cost.end(), std::greater<int64_t>());
+            std::vector<int64_t> load(num_sms, 0);      // a heap, least-loaded SM first
+            int64_t end = 0;
+            for (int64_t c : cost) {
+                std::pop_heap(load.begin(), load.end(), std::greater<int64_t>());
+                end = std::max(end, load.back() += c);
+                std::push_heap(load.begin(), load.end(), std::greater<int64_t>());
+            }
+            return end + (slots ? kMergeCycles + slots * kMergeCyclesPerSlot : 0);
+        };
+        int limit = longest;
+        const int64_t uncut = (int64_t)pairs.size() * Hkv;
+        if (uncut > 0 && 2 * uncut <= num_sms) {
+            while (limit > kSplitMinSteps && items_at(limit - 1) <= num_sms) --limit;
+        } else if (uncut > 0 && uncut <= (int64_t)kSplitMaxRounds * num_sms) {
+            int64_t all = 0;
+            for (auto &pr : pairs)
+                all += Hkv * model_cycles(pr.second >= 0 ? steps_of(pr.first) : 0, long_steps(pr), pr.second >= 0 ? 2 : 1);
+            int64_t best = modelled(longest) * 95 / 100;
+            if (best > all / num_sms)           // otherwise no cut can reach it
+                for (int l = longest * 3 / 4; l >= 2 * kSplitMinSteps && items_at(l) <= 2 * kSplitMaxRounds * num_sms; l = l * 5 / 6) {
+                    const int64_t m = modelled(l);
+                    if (m < best) best = m, limit = l;
+                }
         }
         pl->combine.clear();
+        pl->n_slots = 0;
         for (auto &pr : pairs) {
             const int32_t a = pr.first, b2 = pr.second;
-            const int sa = steps_of(a), sl = steps_of(b2 >= 0 ? b2 : a);       // sa <= sl: positions ascend
-            const int parts = std::max(1, std::min(pl->max_parts, sl / kSplitMinSteps));
-            const int chunk = (sl + parts - 1) / parts;
+            const int sa = steps_of(a), sl = long_steps(pr);                   // sa <= sl: positions ascend
+            const int parts = parts_of(sl, limit), len = (sl + parts - 1) / parts;
+            const int parts_b = (sl + len - 1) / len, parts_a = b2 >= 0 ? (sa + len - 1) / len : parts_b;
             for (int h = 0; h < Hkv; ++h) {
-                int parts_a = 0, parts_b = 0;
-                for (int p2 = 0; p2 < parts; ++p2) {
-                    const int sb = p2 * chunk, se = std::min(sl, sb + chunk);
-                    if (sb >= se) break;
-                    if (b2 < 0 || sb < sa) {
-                        pl->work.push_back({a, b2, h, sb, se, p2, parts, 0});
-                        ++parts_a;
-                        if (b2 >= 0) ++parts_b;
-                    } else {
-                        pl->work.push_back({b2, -1, h, sb, se, p2, parts, 0});   // tile a is already finished
-                        ++parts_b;
-                    }
+                if (parts == 1) {
+                    pl->work.push_back({a, b2, h, 0, sl, -1, -1, 0});
+                    continue;
                 }
-                if (parts > 1) {
-                    pl->combine.push_back({a, h, parts_a, 0});
-                    if (b2 >= 0) pl->combine.push_back({b2, h, parts_b, 0});
+                const int32_t slot_a = pl->n_slots, slot_b = slot_a + parts_a;
+                for (int p2 = 0; p2 < parts_b; ++p2) {
+                    const int sb = p2 * len, se = std::min(sl, sb + len);
+                    if (p2 < parts_a) pl->work.push_back({a, b2, h, sb, se, slot_a + p2, b2 >= 0 ? slot_b + p2 : -1, 0});
+                    else pl->work.push_back({b2, -1, h, sb, se, slot_b + p2, -1, 0});   // tile a is already finished
                 }
+                pl->combine.push_back({a, h, parts_a, slot_a});
+                if (b2 >= 0) pl->combine.push_back({b2, h, parts_b, slot_b});
+                pl->n_slots += parts_a + (b2 >= 0 ? parts_b : 0);
             }
         }
         // cost of an item = its (tile, 128-key step) count, kept in the item for the sorts
@@ -449,9 +508,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         sort_items(pl->work.begin(), pl->work.end());
         // With few items per thread block the spread of the blocks' finishing times is what costs (config 3:
         // 7 items per block, slowest block 8-10 % above the mean with the plain walk): the items are then
-        // assigned greedily to the least-loaded block by modelled cycles (item fetch 700, epilogue + first
-        // step 3 150 per tile, 3 180 per step of both tiles, 1 650 per step of one - measured with clock64)
-        // and laid out so that the kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1
+        // assigned greedily to the least-loaded block by modelled cycles and laid out so that the kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1
         // - b : b)) hands every block its own list; holes are marked tile_a = -1.  Measured: config 3 +6 %,
         // config 4 +-0.  With many items per block (config 5: 131) the plain walk is already even and keeps
         // neighbours in the list - the same request and head - on the GPU at the same time, which the
@@ -462,8 +519,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             auto cycles = [&](const AttnWork &w) -> int64_t {
                 const int sa = std::min(w.step_end, steps_of(w.tile_a)) - w.step_begin;
                 const int sb = w.tile_b >= 0 ? std::min(w.step_end, steps_of(w.tile_b)) - w.step_begin : 0;
-                const int both = std::min(sa, sb), single = std::max(sa, sb) - both, nt = w.tile_b >= 0 ? 2 : 1;
-                return 700 + (int64_t)nt * 3150 + (int64_t)both * 3180 + (int64_t)single * 1650;
+                return model_cycles(sa, sb, w.tile_b >= 0 ? 2 : 1);
             };
             std::vector<int> order(list.size());
             std::iota(order.begin(), order.end(), 0);

@@ -14,8 +14,9 @@ namespace tessera {
 constexpr int kGatherItemTokens = 32;   // token rows per thread block of the gather kernel
 constexpr int kAttnTileRows = 128;      // query rows (tokens x grouped heads) per tcgen05 tile
 constexpr int kDefaultSMs = 148;         // SM count assumed by a host-only plan (a B200); device plans ask the device
-constexpr int kSplitMinSteps = 4;        // never split below this many 128-key steps per part
-constexpr int kSplitMaxParts = 8;
+constexpr int kSplitMinSteps = 2;        // never split below this many 128-key steps per part
+constexpr int kSplitMaxParts = 32;
+constexpr int kSplitMaxRounds = 4;       // batches of more attention items per SM than this are never split
 constexpr int kHostChunks = 4;          // request chunks of the host-buffer entry point's copy / compute pipeline
 constexpr int kLptMaxItemsPerBlock = 16;  // above this many attention items per thread block the plain serpentine walk is kept
 constexpr int kAttnCostBands = 16;      // cost bands of the attention work list (longest band first)
@@ -40,16 +41,17 @@ struct AttnTile {
 
 // One thread block of the tcgen05 attention kernel: KV head `kvh` of query tiles tile_a and tile_b
 // (consecutive tiles of one request; tile_b = -1 when the request has an odd tile left over).
-// With split-KV the item covers only the 128-key steps [step_begin, step_end) and is part `part` of
-// `n_parts`; a part in which tile_a would have nothing to do names the longer tile alone.
+// With split-KV the item covers only the 128-key steps [step_begin, step_end) and leaves its tiles' partial
+// results in workspace slots slot_a / slot_b (-1: the item covers the whole key range of its tiles and writes
+// the outputs); a part in which tile_a would have nothing to do names the longer tile alone.
 struct AttnWork {
-    int32_t tile_a, tile_b, kvh, step_begin, step_end, part, n_parts;
+    int32_t tile_a, tile_b, kvh, step_begin, step_end, slot_a, slot_b;
     int32_t cost;      // (tile, step) count of the item: the host's sort key, not read by the kernel
 };
 
 // One (query tile, KV head) whose partial results have to be merged after a split-KV launch.
 struct CombineItem {
-    int32_t tile, kvh, n_parts, pad;
+    int32_t tile, kvh, n_parts, slot0;   // partial results in workspace slots [slot0, slot0 + n_parts)
 };
 
 struct DeviceTables {
@@ -112,7 +114,7 @@ struct tessera_plan {
     std::vector<tessera::CombineItem> combine;     // grouped by chunk: [chunk_combine_off[c], chunk_combine_off[c+1])
     std::vector<int32_t> chunk_combine_off;
     int32_t n_work_items = 0;                      // real items of `work` (the list may hold holes)
-    int32_t max_parts = 1;                         // split-KV parts per item (1 = no split)
+    int32_t n_slots = 0;                           // split-KV workspace slots (0 = nothing is split)
     int32_t attn_kernel = 0;
     int32_t tile_tokens = 0;
 
