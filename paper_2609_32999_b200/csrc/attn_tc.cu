@@ -28,6 +28,7 @@
 
 #include <algorithm>
 
+#include "device_mem.cuh"
 #include "launch.h"
 #include "plan.h"
 #include "sm100_ptx.cuh"
@@ -136,11 +137,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     constexpr uint32_t kSmemQ = G::kSmemQ, kSmemRing = G::kSmemRing;
     __shared__ __align__(8) Barriers bars;
     __shared__ uint32_t s_tmem_base;
-    __shared__ int s_abort;
+    __shared__ int s_abort, s_skip;
 
-    // A block of a launch in which another block already gave up on a wait does not start, so a
-    // stalled launch ends after one round of timeouts rather than one per block.
-    if (*reinterpret_cast<volatile int *>(status) != 0) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int pps = kStep / page_size;                 // pages per step: 1, 2, 4, 8 or 16
 
@@ -208,9 +206,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         prefetch_tmap(&tmap_o);
     }
     tc_fence_before();
+    // Nothing above touches global memory the stream's earlier kernels write, so it runs beside their tail.
+    grid_wait();
+    grid_release();
+    // A block of a launch in which another block already gave up on a wait does not start, so a
+    // stalled launch ends after one round of timeouts rather than one per block.
+    if (tid == 0) s_skip = *reinterpret_cast<volatile int *>(status) != 0;
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem_base;
+    if (s_skip) {
+        if (warp == 9) tmem_dealloc(tmem, kTmemCols);
+        return;
+    }
     volatile int *abort_flag = &s_abort;
 
     // Registers move from the producer / MMA warp group to the softmax warps, which hold a whole
@@ -685,6 +693,8 @@ attn_combine_kernel(const CombineItem *__restrict__ items, const AttnTile *__res
                     const float *__restrict__ ws_o, const float2 *__restrict__ ws_ml, __nv_bfloat16 *__restrict__ out,
                     float *__restrict__ lse, int H_q, int g) {
     constexpr int kBlocksPerItem = kRows / 8;
+    grid_wait();
+    grid_release();
     const CombineItem it = items[blockIdx.x / kBlocksPerItem];
     const AttnTile t = tiles[it.tile];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -746,29 +756,23 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
     }
     if (!make_q_tmap(&to, out, pl->n_q, Hq, D, g, kRows / g, err)) return cudaErrorInvalidValue;   // `out` has the layout of a 16-bit q
     if (!make_pool_tmap(&tv, v_pool, pl->num_pool_pages, ps, Hkv, D, err)) return cudaErrorInvalidValue;
-    {
-        cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<D, kMaxPages, K8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<D>::kSmemAlloc);
-        if (e != cudaSuccess) { *err = "cudaFuncSetAttribute(shared memory)"; return e; }
-    }
+    cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<D, kMaxPages, K8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<D>::kSmemAlloc);
+    if (e != cudaSuccess) { *err = "cudaFuncSetAttribute(shared memory)"; return e; }
     const DeviceTables &d = pl->dev;
     const float scale_log2 = pl->sm_scale * 1.4426950408889634f * qk_scale;
     // persistent: one thread block per SM (fewer when the list is shorter)
     const int sms = max_blocks > 0 ? std::min(max_blocks, pl->num_sms) : pl->num_sms;
     const unsigned grid = (unsigned)std::min<size_t>(n_work, (size_t)sms);
-    attn_tc_kernel<D, kMaxPages, K8><<<grid, kThreads, Geo<D>::kSmemAlloc, st>>>(
-        tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.page_off, d.pages, d.seq_len,
+    e = launch_kernel(
+        attn_tc_kernel<D, kMaxPages, K8>, grid, kThreads, Geo<D>::kSmemAlloc, st, pl->chained && chunk < 0, tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.page_off, d.pages, d.seq_len,
         static_cast<__nv_bfloat16 *>(out), lse, Hq, g, ps, pl->num_pool_pages, scale_log2, d.ws_o, d.ws_ml, d.status);
-    count_launch();
-    if (!pl->combine.empty()) {
+    if (e == cudaSuccess && !pl->combine.empty()) {
         const int c0 = chunk < 0 ? 0 : pl->chunk_combine_off[chunk];
         const int c1 = chunk < 0 ? (int)pl->combine.size() : pl->chunk_combine_off[chunk + 1];
-        if (c1 > c0) {
-            attn_combine_kernel<D><<<(c1 - c0) * (kRows / 8), 256, 0, st>>>(d.combine + c0, d.tiles, d.ws_o, d.ws_ml, static_cast<__nv_bfloat16 *>(out),
-                                                                          lse, Hq, g);
-            count_launch();
-        }
+        if (c1 > c0)
+            e = launch_kernel(attn_combine_kernel<D>, (unsigned)(c1 - c0) * (kRows / 8), 256, 0, st, pl->chained && chunk < 0,
+                              d.combine + c0, d.tiles, d.ws_o, d.ws_ml, static_cast<__nv_bfloat16 *>(out), lse, Hq, g);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) *err = "kernel launch";
     return e;
 }

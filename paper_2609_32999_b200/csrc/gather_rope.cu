@@ -9,28 +9,13 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "device_mem.cuh"
 #include "launch.h"
 #include "plan.h"
 
 namespace tessera {
 
 namespace {
-
-__device__ __forceinline__ uint4 ldg_stream(const uint4 *p) {
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ uint4 ldg_plain(const uint4 *p) {
-    uint4 v;
-    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ void stg(uint4 *p, const uint4 &v) {
-    asm volatile("st.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
 
 // One rotary pair in fp32: (x, y) -> (x cos - y sin, y cos + x sin).  A table entry that is exactly
 // (1, 0) - a shift of zero, or a frequency of zero - returns the inputs themselves, so such elements
@@ -104,6 +89,8 @@ gather_rope_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 
     __shared__ float2 s_rope[kGatherItemTokens * (D / 2)];
     __shared__ int32_t s_src[kGatherItemTokens], s_dst[kGatherItemTokens];
 
+    grid_wait();
+    grid_release();
     const int tid = threadIdx.x;
     const GatherItem it = items[blockIdx.x];
     // rows row0, row0 + step, ... of the table; with step = -1 they are staged in ascending order
@@ -238,6 +225,8 @@ __global__ void __launch_bounds__(256)
 scatter_fresh_kernel(uint4 *__restrict__ k_pool, uint4 *__restrict__ v_pool,
                      const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new,
                      const int32_t *__restrict__ fresh_dst, int64_t first_chunk, int64_t n_chunks, int row_chunks) {
+    grid_wait();
+    grid_release();
     for (int64_t e = first_chunk + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < first_chunk + n_chunks;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = e / row_chunks;
@@ -257,6 +246,8 @@ rope_fresh_kernel(uint4 *__restrict__ q, uint4 *__restrict__ k_new, const int32_
                   const double *__restrict__ inv_freq, int H_q, int H_kv) {
     constexpr int CPH = D / 16, HALF = D / 16;
     __shared__ float2 s_cs[D / 2];
+    grid_wait();
+    grid_release();
     const int j = blockIdx.x, tid = threadIdx.x;
     if (tid < D / 2) {
         double sn, cs;
@@ -299,6 +290,8 @@ extend_write_kernel(uint4 *__restrict__ q, const uint4 *__restrict__ k_raw, cons
     constexpr int CPH = D / 16, HALF = D / 16;
     __shared__ float2 s_cs[kExtendRows][D / 2];
     __shared__ int32_t s_dst[kExtendRows], s_keep[kExtendRows];
+    grid_wait();
+    grid_release();
     const int tid = threadIdx.x;
     const int j0 = blockIdx.x * kExtendRows;
     const int rows = min(kExtendRows, n_q - j0);
@@ -356,15 +349,15 @@ extend_write_kernel(uint4 *__restrict__ q, const uint4 *__restrict__ k_raw, cons
 }
 
 template <int D, bool IL>
-void launch_gather_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
-                     GatherMode mode, cudaStream_t st) {
+cudaError_t launch_gather_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
+                                   GatherMode mode, cudaStream_t st) {
     const DeviceTables &d = pl->dev;
     auto kernel = mode == GatherMode::kCopy         ? gather_rope_kernel<D, true, false, false, IL>
                   : mode == GatherMode::kCopyRotate ? gather_rope_kernel<D, true, true, false, IL>
                                                     : gather_rope_kernel<D, false, true, true, IL>;
-    kernel<<<(unsigned)pl->items.size(), kThreads, 0, st>>>(
-        static_cast<const uint4 *>(k_src), static_cast<const uint4 *>(v_src), static_cast<uint4 *>(k_pool), static_cast<uint4 *>(v_pool),
-        d.g_src, d.g_dst, d.items, d.rope, pl->cfg.num_kv_heads);
+    return launch_kernel(kernel, (unsigned)pl->items.size(), kThreads, 0, st, pl->chained, static_cast<const uint4 *>(k_src),
+                         static_cast<const uint4 *>(v_src), static_cast<uint4 *>(k_pool), static_cast<uint4 *>(v_pool), d.g_src, d.g_dst,
+                         d.items, d.rope, pl->cfg.num_kv_heads);
 }
 
 }  // namespace
@@ -375,9 +368,7 @@ cudaError_t launch_gather(const tessera_plan *pl, const void *k_src, const void 
     const bool il = pl->cfg.rope_pairing == 1;
     auto launch = pl->cfg.head_dim == 128 ? (il ? launch_gather_d<128, true> : launch_gather_d<128, false>)
                                           : (il ? launch_gather_d<64, true> : launch_gather_d<64, false>);
-    launch(pl, k_src, v_src, k_pool, v_pool, mode, st);
-    count_launch();
-    return cudaGetLastError();
+    return launch(pl, k_src, v_src, k_pool, v_pool, mode, st);
 }
 
 cudaError_t launch_gather_runs(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
@@ -388,11 +379,11 @@ cudaError_t launch_gather_runs(const tessera_plan *pl, const void *k_src, const 
     const bool il = pl->cfg.rope_pairing == 1;
     auto kernel = pl->cfg.head_dim == 128 ? (il ? gather_runs_kernel<128, true> : gather_runs_kernel<128, false>)
                                           : (il ? gather_runs_kernel<64, true> : gather_runs_kernel<64, false>);
-    kernel<<<grid, kThreads, 0, st>>>(static_cast<const uint4 *>(k_src), static_cast<const uint4 *>(v_src), static_cast<uint4 *>(k_pool),
-                                      static_cast<uint4 *>(v_pool), d.g_src, d.g_dst, d.items, d.runs + first_run, n_runs, d.rope,
-                                      pl->cfg.num_kv_heads);
-    count_launch();
-    return cudaGetLastError();
+    // never chained: the launches of one call follow one another on a side stream, ordered by events, and a
+    // successor resident beside its predecessor would hold SMs the attention kernel runs on
+    return launch_kernel(kernel, grid, kThreads, 0, st, false, static_cast<const uint4 *>(k_src), static_cast<const uint4 *>(v_src),
+                         static_cast<uint4 *>(k_pool), static_cast<uint4 *>(v_pool), d.g_src, d.g_dst, d.items, d.runs + first_run,
+                         n_runs, d.rope, pl->cfg.num_kv_heads);
 }
 
 cudaError_t launch_rope_fresh(const tessera_plan *pl, void *q, void *k_new, cudaStream_t st) {
@@ -403,15 +394,9 @@ cudaError_t launch_rope_fresh(const tessera_plan *pl, void *q, void *k_new, cuda
     const int Hq = pl->cfg.num_q_heads, Hkv = pl->cfg.num_kv_heads;
     const unsigned n = (unsigned)pl->n_q;
     const bool il = pl->cfg.rope_pairing == 1;
-    if (pl->cfg.head_dim == 128) {
-        if (il) rope_fresh_kernel<128, true><<<n, 128, 0, st>>>(qp, kp, d.q_pos, d.inv_freq, Hq, Hkv);
-        else rope_fresh_kernel<128, false><<<n, 128, 0, st>>>(qp, kp, d.q_pos, d.inv_freq, Hq, Hkv);
-    } else {
-        if (il) rope_fresh_kernel<64, true><<<n, 128, 0, st>>>(qp, kp, d.q_pos, d.inv_freq, Hq, Hkv);
-        else rope_fresh_kernel<64, false><<<n, 128, 0, st>>>(qp, kp, d.q_pos, d.inv_freq, Hq, Hkv);
-    }
-    count_launch();
-    return cudaGetLastError();
+    auto kernel = pl->cfg.head_dim == 128 ? (il ? rope_fresh_kernel<128, true> : rope_fresh_kernel<128, false>)
+                                          : (il ? rope_fresh_kernel<64, true> : rope_fresh_kernel<64, false>);
+    return launch_kernel(kernel, n, 128, 0, st, pl->chained, qp, kp, d.q_pos, d.inv_freq, Hq, Hkv);
 }
 
 cudaError_t launch_extend_write(const tessera_plan *pl, void *k_pool, void *v_pool, void *q, const void *k_new_raw,
@@ -426,15 +411,9 @@ cudaError_t launch_extend_write(const tessera_plan *pl, void *k_pool, void *v_po
     auto *kc = static_cast<uint4 *>(k_cache), *vc = static_cast<uint4 *>(v_cache);
     const int32_t *keep = pl->retained_tokens > 0 ? d.retain_dst : nullptr;
     const bool il = pl->cfg.rope_pairing == 1;
-    if (pl->cfg.head_dim == 128) {
-        if (il) extend_write_kernel<128, true><<<blocks, 256, 0, st>>>(qp, kr, vn, kp, vp, kc, vc, d.q_pos, d.fresh_dst, keep, d.inv_freq, n_q, Hq, Hkv);
-        else extend_write_kernel<128, false><<<blocks, 256, 0, st>>>(qp, kr, vn, kp, vp, kc, vc, d.q_pos, d.fresh_dst, keep, d.inv_freq, n_q, Hq, Hkv);
-    } else {
-        if (il) extend_write_kernel<64, true><<<blocks, 256, 0, st>>>(qp, kr, vn, kp, vp, kc, vc, d.q_pos, d.fresh_dst, keep, d.inv_freq, n_q, Hq, Hkv);
-        else extend_write_kernel<64, false><<<blocks, 256, 0, st>>>(qp, kr, vn, kp, vp, kc, vc, d.q_pos, d.fresh_dst, keep, d.inv_freq, n_q, Hq, Hkv);
-    }
-    count_launch();
-    return cudaGetLastError();
+    auto kernel = pl->cfg.head_dim == 128 ? (il ? extend_write_kernel<128, true> : extend_write_kernel<128, false>)
+                                          : (il ? extend_write_kernel<64, true> : extend_write_kernel<64, false>);
+    return launch_kernel(kernel, blocks, 256, 0, st, pl->chained, qp, kr, vn, kp, vp, kc, vc, d.q_pos, d.fresh_dst, keep, d.inv_freq, n_q, Hq, Hkv);
 }
 
 cudaError_t launch_scatter_fresh(const tessera_plan *pl, void *k_pool, void *v_pool, const void *k_new,
@@ -446,11 +425,9 @@ cudaError_t launch_scatter_fresh(const tessera_plan *pl, void *k_pool, void *v_p
     if (rows == 0) return cudaSuccess;
     const int64_t n_chunks = rows * row_chunks;
     const int blocks = (int)std::min<int64_t>((n_chunks + 255) / 256, (int64_t)pl->num_sms * 16);
-    scatter_fresh_kernel<<<blocks, 256, 0, st>>>(static_cast<uint4 *>(k_pool), static_cast<uint4 *>(v_pool),
-                                                static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new),
-                                                pl->dev.fresh_dst, row0 * row_chunks, n_chunks, row_chunks);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(scatter_fresh_kernel, blocks, 256, 0, st, pl->chained && chunk < 0, static_cast<uint4 *>(k_pool),
+                         static_cast<uint4 *>(v_pool), static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new),
+                         pl->dev.fresh_dst, row0 * row_chunks, n_chunks, row_chunks);
 }
 
 }  // namespace tessera

@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "device_mem.cuh"
 #include "launch.h"
 #include "plan.h"
 
@@ -107,6 +108,8 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
     __shared__ float2 s_rope[kGatherItemTokens * (D / 2)];
     __shared__ int32_t s_src[kGatherItemTokens], s_dst[kGatherItemTokens];
 
+    grid_wait();
+    grid_release();
     const int tid = threadIdx.x;
     const GatherItem it = items[blockIdx.x];
     const int n_rows = ROTATE ? (it.row_step ? it.count : 1) : 0;
@@ -140,10 +143,10 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
             const int chunk = (w / CPH) * (D / 8) + c;
             const size_t so = (size_t)s_src[tok[u]] * row_chunks + chunk;
             dso[u] = (size_t)s_dst[tok[u]] * row_chunks + chunk;
-            rk[u][0] = __ldg(ks + so);
-            rk[u][1] = __ldg(ks + so + HALF);
-            rv[u][0] = __ldg(vs + so);
-            rv[u][1] = __ldg(vs + so + HALF);
+            rk[u][0] = ldg_stream(ks + so);
+            rk[u][1] = ldg_stream(ks + so + HALF);
+            rv[u][0] = ldg_stream(vs + so);
+            rv[u][1] = ldg_stream(vs + so + HALF);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -214,10 +217,10 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
                 if (t >= n_tasks) continue;
                 const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
                 const size_t so = (size_t)g_src[src.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
-                rk[u][0] = __ldg(k_src + so);
-                rk[u][1] = __ldg(k_src + so + HALF);
-                rv[u][0] = __ldg(v_src + so);
-                rv[u][1] = __ldg(v_src + so + HALF);
+                rk[u][0] = ldg_stream(k_src + so);
+                rk[u][1] = ldg_stream(k_src + so + HALF);
+                rv[u][0] = ldg_stream(v_src + so);
+                rv[u][1] = ldg_stream(v_src + so + HALF);
             }
             for (int m = 0; m < rn.n_items; ++m) {
                 const GatherItem it = items[rn.first_item + m];
@@ -250,9 +253,11 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
 // bf16 -> e4m3 codes of (value * mul): 8 elements per thread, grid-stride.
 __global__ void __launch_bounds__(256)
 quantize_e4m3_kernel(const uint4 *__restrict__ src, uint2 *__restrict__ dst, int64_t n_chunks, float mul) {
+    grid_wait();
+    grid_release();
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_chunks; e += (int64_t)gridDim.x * blockDim.x) {
         float f[8];
-        unpack_bf16x8(__ldg(src + e), f);
+        unpack_bf16x8(ldg_stream(src + e), f);
         dst[e] = pack_e4m3x8(f, mul);
     }
 }
@@ -263,28 +268,30 @@ __global__ void __launch_bounds__(256)
 scatter_fresh_k8_kernel(uint2 *__restrict__ k_pool8, uint4 *__restrict__ v_pool, const uint4 *__restrict__ k_new,
                         const uint4 *__restrict__ v_new, const int32_t *__restrict__ fresh_dst, int64_t n_chunks,
                         int row_chunks, float k_mul) {
+    grid_wait();
+    grid_release();
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_chunks; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = e / row_chunks;
         const int c = (int)(e - j * row_chunks);
         const size_t o = (size_t)fresh_dst[j] * row_chunks + c;
         if (k_new) {
             float f[8];
-            unpack_bf16x8(__ldg(k_new + e), f);
+            unpack_bf16x8(ldg_stream(k_new + e), f);
             k_pool8[o] = pack_e4m3x8(f, k_mul);
         }
-        if (v_new) v_pool[o] = __ldg(v_new + e);
+        if (v_new) v_pool[o] = ldg_stream(v_new + e);
     }
 }
 
 template <int D, bool TO_8BIT>
-void launch_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst, bool rotate,
-              float k_mul, float v_mul, cudaStream_t st) {
+cudaError_t launch_d(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst, bool rotate,
+                     float k_mul, float v_mul, cudaStream_t st) {
     const DeviceTables &d = pl->dev;
     const bool il = pl->cfg.rope_pairing == 1;
     auto kernel = rotate ? (il ? kv_fp8_kernel<D, TO_8BIT, true, true> : kv_fp8_kernel<D, TO_8BIT, true, false>)
                          : (il ? kv_fp8_kernel<D, TO_8BIT, false, true> : kv_fp8_kernel<D, TO_8BIT, false, false>);
-    kernel<<<(unsigned)pl->items.size(), kThreads, 0, st>>>(k_src, v_src, k_dst, v_dst, d.g_src, d.g_dst, d.items, d.rope,
-                                                            pl->cfg.num_kv_heads, k_mul, v_mul);
+    return launch_kernel(kernel, (unsigned)pl->items.size(), kThreads, 0, st, pl->chained, k_src, v_src, k_dst, v_dst, d.g_src, d.g_dst,
+                         d.items, d.rope, pl->cfg.num_kv_heads, k_mul, v_mul);
 }
 
 }  // namespace
@@ -297,27 +304,22 @@ cudaError_t launch_compose_k8(const tessera_plan *pl, const void *k_src, const v
     const DeviceTables &d = pl->dev;
     const int H = pl->cfg.num_kv_heads;
     const bool il = pl->cfg.rope_pairing == 1;
-#define TESSERA_K8_LAUNCH(DD, ROT, IL) \
-    kv_fp8_kernel<DD, true, ROT, IL, true><<<n, kThreads, 0, st>>>(k_src, v_src, k_dst8, v_dst, d.g_src, d.g_dst, d.items, d.rope, H, k_mul, 1.f)
-    if (pl->cfg.head_dim == 128) {
-        if (rotate) { if (il) TESSERA_K8_LAUNCH(128, true, true); else TESSERA_K8_LAUNCH(128, true, false); }
-        else { if (il) TESSERA_K8_LAUNCH(128, false, true); else TESSERA_K8_LAUNCH(128, false, false); }
-    } else {
-        if (rotate) { if (il) TESSERA_K8_LAUNCH(64, true, true); else TESSERA_K8_LAUNCH(64, true, false); }
-        else { if (il) TESSERA_K8_LAUNCH(64, false, true); else TESSERA_K8_LAUNCH(64, false, false); }
-    }
-#undef TESSERA_K8_LAUNCH
-    count_launch();
-    return cudaGetLastError();
+    auto pick = [&](auto dim) {
+        constexpr int D = decltype(dim)::value;
+        return rotate ? (il ? kv_fp8_kernel<D, true, true, true, true> : kv_fp8_kernel<D, true, true, false, true>)
+                      : (il ? kv_fp8_kernel<D, true, false, true, true> : kv_fp8_kernel<D, true, false, false, true>);
+    };
+    auto kernel = pl->cfg.head_dim == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
+    return launch_kernel(kernel, (unsigned)n, kThreads, 0, st, pl->chained, k_src, v_src, k_dst8, v_dst, d.g_src, d.g_dst, d.items, d.rope, H,
+                         k_mul, 1.f);
 }
 
-cudaError_t launch_quantize_e4m3(const void *src_bf16, void *dst8, int64_t n_elems, float mul, cudaStream_t st) {
+cudaError_t launch_quantize_e4m3(const void *src_bf16, void *dst8, int64_t n_elems, float mul, bool chained, cudaStream_t st) {
     const int64_t n_chunks = n_elems / 8;
     if (n_chunks == 0) return cudaSuccess;
     const int blocks = (int)std::min<int64_t>((n_chunks + 255) / 256, 148 * 16);
-    quantize_e4m3_kernel<<<blocks, 256, 0, st>>>(static_cast<const uint4 *>(src_bf16), static_cast<uint2 *>(dst8), n_chunks, mul);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(quantize_e4m3_kernel, (unsigned)blocks, 256, 0, st, chained, static_cast<const uint4 *>(src_bf16),
+                         static_cast<uint2 *>(dst8), n_chunks, mul);
 }
 
 cudaError_t launch_scatter_fresh_k8(const tessera_plan *pl, void *k_pool8, void *v_pool, const void *k_new,
@@ -326,11 +328,9 @@ cudaError_t launch_scatter_fresh_k8(const tessera_plan *pl, void *k_pool8, void 
     const int row_chunks = pl->cfg.num_kv_heads * pl->cfg.head_dim / 8;
     const int64_t n_chunks = pl->n_q * row_chunks;
     const int blocks = (int)std::min<int64_t>((n_chunks + 255) / 256, (int64_t)pl->num_sms * 16);
-    scatter_fresh_k8_kernel<<<blocks, 256, 0, st>>>(static_cast<uint2 *>(k_pool8), static_cast<uint4 *>(v_pool),
-                                                   static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new),
-                                                   pl->dev.fresh_dst, n_chunks, row_chunks, k_mul);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(scatter_fresh_k8_kernel, (unsigned)blocks, 256, 0, st, pl->chained, static_cast<uint2 *>(k_pool8),
+                         static_cast<uint4 *>(v_pool), static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new),
+                         pl->dev.fresh_dst, n_chunks, row_chunks, k_mul);
 }
 
 cudaError_t launch_kv_fp8(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst,
@@ -338,9 +338,7 @@ cudaError_t launch_kv_fp8(const tessera_plan *pl, const void *k_src, const void 
     if (pl->items.empty()) return cudaSuccess;
     auto launch = pl->cfg.head_dim == 128 ? (to_8bit ? launch_d<128, true> : launch_d<128, false>)
                                           : (to_8bit ? launch_d<64, true> : launch_d<64, false>);
-    launch(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, st);
-    count_launch();
-    return cudaGetLastError();
+    return launch(pl, k_src, v_src, k_dst, v_dst, rotate, k_mul, v_mul, st);
 }
 
 cudaError_t launch_expand_fp8_runs(const tessera_plan *pl, const void *k_src8, const void *v_src8, void *k_pool, void *v_pool,
@@ -351,11 +349,9 @@ cudaError_t launch_expand_fp8_runs(const tessera_plan *pl, const void *k_src8, c
     const bool il = pl->cfg.rope_pairing == 1;
     auto kernel = pl->cfg.head_dim == 128 ? (il ? expand_runs_kernel<128, true> : expand_runs_kernel<128, false>)
                                           : (il ? expand_runs_kernel<64, true> : expand_runs_kernel<64, false>);
-    kernel<<<grid, kThreads, 0, st>>>(static_cast<const uint2 *>(k_src8), static_cast<const uint2 *>(v_src8), static_cast<uint4 *>(k_pool),
-                                      static_cast<uint4 *>(v_pool), d.g_src, d.g_dst, d.items, d.runs + first_run, n_runs, d.rope,
-                                      pl->cfg.num_kv_heads, k_scale, v_scale);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kernel, grid, kThreads, 0, st, false, static_cast<const uint2 *>(k_src8), static_cast<const uint2 *>(v_src8),
+                         static_cast<uint4 *>(k_pool), static_cast<uint4 *>(v_pool), d.g_src, d.g_dst, d.items, d.runs + first_run,
+                         n_runs, d.rope, pl->cfg.num_kv_heads, k_scale, v_scale);
 }
 
 }  // namespace tessera

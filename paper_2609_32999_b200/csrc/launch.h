@@ -10,6 +10,25 @@ enum class GatherMode { kCopy, kCopyRotate, kShiftInPlace };
 
 void count_launch();   // bumps the process-wide kernel-launch counter
 
+// Launches and counts `kernel`.  `chained`: it may become resident while its predecessor in the stream still runs
+// (the kernel itself waits, see grid_wait()); behind anything but a kernel that is an ordinary launch too.
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool chained, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e == cudaSuccess) count_launch();
+    return e;
+}
+
 // Sources are read from (k_src, v_src) - the destination pools themselves unless the plan names a
 // separate source pool - and written to the plan's destination slots in (k_pool, v_pool).
 cudaError_t launch_gather(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_pool, void *v_pool,
@@ -50,7 +69,7 @@ cudaError_t launch_attn_tc_k8(const tessera_plan *pl, void *k_pool8, void *v_poo
 cudaError_t launch_compose_k8(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst8, void *v_dst,
                               bool rotate, float k_mul, cudaStream_t st);
 // bf16 rows -> e4m3 codes of (value * mul), nearest-even, saturating: n_elems elements (a multiple of 8).
-cudaError_t launch_quantize_e4m3(const void *src_bf16, void *dst8, int64_t n_elems, float mul, cudaStream_t st);
+cudaError_t launch_quantize_e4m3(const void *src_bf16, void *dst8, int64_t n_elems, float mul, bool chained, cudaStream_t st);
 // Fresh rows into an 8-bit key pool (codes of k_new * k_mul) and a 16-bit value pool (bit copies).
 cudaError_t launch_scatter_fresh_k8(const tessera_plan *pl, void *k_pool8, void *v_pool, const void *k_new,
                                     const void *v_new, float k_mul, cudaStream_t st);

@@ -442,6 +442,11 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             if (w.tile_b >= 0) c += std::min(w.step_end, steps_of(w.tile_b)) - w.step_begin;
             w.cost = c;
         }
+        // Launch latency is a visible part of a layer only while the attention list fits the SMs once (2 items,
+        // 304 tokens: 20.6 -> 19.1 us a layer; 144 items, 5 312 tokens: 62.3 -> 56.2).  With longer lists a chained
+        // attention kernel measured slower than an ordinary launch (8 192 rows in 1 024 items, 16 requests: 481 us
+        // a layer against 450; 82 291 rows in 20 696 items: 13.1 ms against 12.4).
+        pl->chained = (int)pl->work.size() <= num_sms;
         pl->mma_pairs = 0;
         for (const AttnWork &w : pl->work) pl->mma_pairs += (int64_t)w.cost * kAttnTileRows * page;
         auto cost = [](const AttnWork &w) { return w.cost; };

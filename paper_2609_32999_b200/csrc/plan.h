@@ -114,6 +114,8 @@ struct tessera_plan {
     std::vector<tessera::CombineItem> combine;     // grouped by chunk: [chunk_combine_off[c], chunk_combine_off[c+1])
     std::vector<int32_t> chunk_combine_off;
     int32_t n_work_items = 0;                      // real items of `work` (the list may hold holes)
+    // Kernels of the plan's calls are launched chained (see launch_kernel): at most one attention item per SM.
+    bool chained = false;
     int32_t n_slots = 0;                           // split-KV workspace slots (0 = nothing is split)
     int32_t attn_kernel = 0;
     int32_t tile_tokens = 0;
