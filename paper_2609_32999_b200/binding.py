@@ -125,7 +125,8 @@ def _dev(t) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
-        stream = torch.cuda.current_stream()
+        # the handle alone: torch.cuda.current_stream() builds a Stream object, 3.3 us of an 8 us call
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None

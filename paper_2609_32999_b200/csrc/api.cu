@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cuda_runtime.h>
 
+#include "blob_pool.h"
 #include "launch.h"
 #include "plan.h"
 
@@ -104,7 +105,7 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     put(o_comb, pl->combine.data(), pl->combine.size() * sizeof(CombineItem));
     put(o_invf, pl->inv_freq.data(), pl->inv_freq.size() * sizeof(double));
     put(o_seq, pl->seq_len.data(), pl->seq_len.size() * 4);
-    TS_CUDA(cudaMalloc(&d.blob, off));
+    TS_CUDA(blob_acquire(&d.blob, off, &d.blob_bytes, st));
     TS_CUDA(cudaMemcpyAsync(d.blob, hb, table_bytes, cudaMemcpyHostToDevice, st));
     char *db = static_cast<char *>(d.blob);
     d.g_src = reinterpret_cast<int32_t *>(db + o_src);
@@ -213,7 +214,7 @@ int32_t tessera_plan_create(const tessera_model_cfg *cfg, const tessera_compose_
     if (!pl->host_only) {
         st = upload(pl, static_cast<cudaStream_t>(stream));
         if (st != TESSERA_OK) {
-            if (pl->dev.blob) cudaFree(pl->dev.blob);
+            if (pl->dev.blob) blob_release(pl->dev.blob, pl->dev.blob_bytes, pl->device);
             delete pl;
             return st;
         }
@@ -232,7 +233,11 @@ int32_t tessera_plan_destroy(tessera_plan *pl) {
         if (pl->ev_out) cudaEventDestroy(pl->ev_out);
         if (pl->s_in) cudaStreamDestroy(pl->s_in);
         if (pl->s_out) cudaStreamDestroy(pl->s_out);
-        void *bufs[] = {pl->dev.blob, pl->dev.st_q, pl->dev.st_k, pl->dev.st_v, pl->dev.st_o, pl->dev.st_lse, pl->dev.q8};
+        if (pl->dev.blob) {
+            cudaError_t e = blob_release(pl->dev.blob, pl->dev.blob_bytes, pl->device);
+            if (e != cudaSuccess) rc = cuda_fail(e, "release of the plan's device memory");
+        }
+        void *bufs[] = {pl->dev.st_q, pl->dev.st_k, pl->dev.st_v, pl->dev.st_o, pl->dev.st_lse, pl->dev.q8};
         for (void *b : bufs)
             if (b) {
                 cudaError_t e = cudaFree(b);

@@ -56,6 +56,7 @@ struct CombineItem {
 
 struct DeviceTables {
     void *blob = nullptr;          // one allocation holding everything below
+    size_t blob_bytes = 0;
     int32_t *g_src = nullptr, *g_dst = nullptr;
     GatherItem *items = nullptr;
     GatherRun *runs = nullptr;

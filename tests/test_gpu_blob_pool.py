@@ -1,0 +1,72 @@
+"""Device memory of destroyed plans is reused by later ones: results stay right, memory stays bounded, also with
+plans of several sizes alive at once and on several threads."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_32999_b200 import binding as tb
+from paper_2609_32999_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(w, t, out):
+    plan = tb.Plan(w)
+    plan.kv_compose(t.k_pool, t.v_pool)
+    plan.partial_prefill_attn(t.k_pool, t.v_pool, t.q, t.k_new, t.v_new, out, None)
+    return plan
+
+
+def test_results_and_memory_over_many_plans():
+    ws = [wl.config(1), wl.config(2), wl.config(3, requests_override=2)]
+    ts = [wl.make_tensors(w, device="cuda:0", seed=i) for i, w in enumerate(ws)]
+    ref = [torch.zeros_like(t.q) for t in ts]
+    keep = [_layer(w, t, o) for w, t, o in zip(ws, ts, ref)]
+    torch.cuda.synchronize()
+    for p in keep:
+        p.destroy()
+    free0 = torch.cuda.mem_get_info()[0]
+    rng = np.random.default_rng(0)
+    out = [torch.zeros_like(t.q) for t in ts]
+    alive = []
+    for _ in range(60):
+        i = int(rng.integers(3))
+        out[i].zero_()
+        alive.append(_layer(ws[i], ts[i], out[i]))
+        if len(alive) > 3:
+            alive.pop(int(rng.integers(4))).destroy()          # work of the others may still be queued
+        torch.cuda.synchronize()
+        assert torch.equal(out[i], ref[i])
+    for p in alive:
+        p.destroy()
+    assert free0 - torch.cuda.mem_get_info()[0] <= 128 << 20
+
+
+def test_plans_on_several_threads():
+    w = wl.config(2)
+    ts = [wl.make_tensors(w, device="cuda:0", seed=9) for _ in range(4)]
+    outs = [torch.zeros_like(t.q) for t in ts]
+    errors = []
+
+    def work(k):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(10):
+                    p = _layer(w, ts[k], outs[k])
+                    assert p.status() == 0
+                    p.destroy()
+        except Exception as e:       # noqa: BLE001
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    assert not errors
+    for o in outs[1:]:
+        assert torch.equal(outs[0], o)
