@@ -7,10 +7,11 @@
 //   warps 0-7  : softmax.  All eight work on one tile at a time and alternate between the tiles; a
 //                warp owns 16 rows (TMEM lanes) and reads them as an MMA accumulator fragment, the
 //                four threads of a row in one warp - no two warps ever exchange anything
-//   warp 8     : TMA producer - Q tiles once per item, then K and V of every step through one ring of
-//                four 32 KB shared-memory slots; page ids come from the request's block table
+//   warp 8     : TMA producer for Q (once per item) and K, warp 11 for V: K and V of every step go through one
+//                ring of four 32 KB shared-memory slots; page ids come from the request's block table.  (One
+//                thread issues one box at a time, and a step of 16-token pages takes 32: with one warp for
+//                both, a step of a lone tile took 1 864 ns, with two 1 561; 64-token pages 1 550 either way.)
 //   warp 9, 10 : issue tcgen05.mma for tile 0 / tile 1 (one lane each); warp 9 owns the TMEM allocation
-//   warp 11    : idle (completes the warp group that hands its registers to the softmax warps)
 // Per tile and step:  S = Q K^T (both operands in shared memory) -> 128 fp32 TMEM columns;
 // softmax reads S and writes P as bf16 back over part of those columns; O += P V takes P straight
 // from TMEM, so probabilities never touch shared memory.  Each issuing warp sends P.V of step j and
@@ -42,7 +43,7 @@ using namespace ptx;
 constexpr int kStep = 128;         // keys per step (two pages)
 constexpr int kRows = 128;         // rows per query tile
 constexpr int kRing = 4;           // K/V ring slots (two steps of look-ahead; a fifth slot measured no faster)
-constexpr int kThreads = 384;        // 8 softmax warps, producer, MMA, 2 idle warps (register donors)
+constexpr int kThreads = 384;        // 8 softmax warps, 2 producers, 2 MMA issuers
 // setmaxnreg moves registers inside the pool the block got at launch (threads x registers per thread
 // under __launch_bounds__): the raised and lowered counts together must fit in it, or the raise
 // waits forever.
@@ -225,13 +226,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     // 128-column row of S plus the packed probabilities.
     if (warp >= 8) {
     reg_dealloc<kRegsOther>();
-    if (warp == 8) {
-        // ------------------------------------------------------------------ TMA producer
+    if (warp == 8 || warp == 11) {
+        // ------------------------------------------------------------------ TMA producers: warp 8 for Q and K, warp 11 for V
+        const int kv = warp == 8 ? 0 : 1;
         // A tile holds (128 / g) tokens x g heads = q_rows rows; when g does not divide 128 the last
         // rows of the 128-row MMA tile are padding and are zeroed once (TMA never writes them; their
         // results are never stored).
         const int q_rows = (kRows / g) * g;
-        if (q_rows < kRows) {
+        if (kv == 0 && q_rows < kRows) {
             for (int q = 0; q < 2; ++q)
 #pragma unroll
                 for (int hf = 0; hf < kQKHalves; ++hf) {
@@ -252,7 +254,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             const Item it = load_item(w);
             if (it.n_tiles == 0) continue;
             const int kvh = it.wk.kvh;
-            if (lane == 0) {
+            if (kv == 0 && lane == 0) {
                 for (int q = 0; q < it.n_tiles; ++q) {
                     const AttnTile &t = q ? it.t1 : it.t0;
                     // the previous item's last S MMA has read this buffer
@@ -278,23 +280,20 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                     for (int k = 0; k < kMaxPages; ++k) pg[k] = __shfl_sync(0xffffffffu, my_page, (pps * jj + k) & 31);
                     if (lane == 0) {
                         const int j = j0 + jj;
+                        const int item = ring_base + 2 * j + kv, slot = item % kRing;
+                        mbar_wait(smem_u32(&bars.empty[slot]), ((item / kRing) & 1) ^ 1, abort_flag, status, 1 + kv);
+                        const uint32_t fb = smem_u32(&bars.full[slot]);
+                        const int halves = kv ? G::kHalves : kQKHalves;
+                        mbar_expect_tx(fb, (uint32_t)halves * kHalfBytes);
+                        const uint32_t dst = smem_u32(sm + kSmemRing + slot * kSlotBytes);
+                        const CUtensorMap *tm = kv ? &tmap_v : &tmap_k;
 #pragma unroll
-                        for (int kv = 0; kv < 2; ++kv) {
-                            const int item = ring_base + 2 * j + kv, slot = item % kRing;
-                            mbar_wait(smem_u32(&bars.empty[slot]), ((item / kRing) & 1) ^ 1, abort_flag, status, 1 + kv);
-                            const uint32_t fb = smem_u32(&bars.full[slot]);
-                            const int halves = kv ? G::kHalves : kQKHalves;
-                            mbar_expect_tx(fb, (uint32_t)halves * kHalfBytes);
-                            const uint32_t dst = smem_u32(sm + kSmemRing + slot * kSlotBytes);
-                            const CUtensorMap *tm = kv ? &tmap_v : &tmap_k;
+                        for (int k = 0; k < kMaxPages; ++k)
+                            if (k < pps) {
 #pragma unroll
-                            for (int k = 0; k < kMaxPages; ++k)
-                                if (k < pps) {
-#pragma unroll
-                                    for (int hf = 0; hf < G::kHalves; ++hf)
-                                        if (hf < halves) tma_load_4d(dst + hf * kHalfBytes + k * page_bytes, tm, fb, hf * 64, kvh, 0, pg[k]);
-                                }
-                        }
+                                for (int hf = 0; hf < G::kHalves; ++hf)
+                                    if (hf < halves) tma_load_4d(dst + hf * kHalfBytes + k * page_bytes, tm, fb, hf * 64, kvh, 0, pg[k]);
+                            }
                     }
                     __syncwarp();
                 }
