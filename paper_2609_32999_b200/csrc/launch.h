@@ -12,21 +12,34 @@ void count_launch();   // bumps the process-wide kernel-launch counter
 
 // Launches and counts `kernel`.  `chained`: it may become resident while its predecessor in the stream still runs
 // (the kernel itself waits, see grid_wait()); behind anything but a kernel that is an ordinary launch too.
+// `cluster`: thread blocks per cluster (2: blocks 2 i and 2 i + 1 run on the two SMs of one TPC).
 template <class... P, class... A>
-cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool chained, A... args) {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_clusters(void (*kernel)(P...), unsigned grid, unsigned block, unsigned cluster, size_t smem, cudaStream_t st,
+                            bool chained, A... args) {
+    cudaLaunchAttribute attr[2]{};
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = chained ? 1 : 0;
+    cfg.attrs = attr;
+    if (chained) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     if (e == cudaSuccess) count_launch();
     return e;
+}
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool chained, A... args) {
+    return launch_clusters(kernel, grid, block, 1, smem, st, chained, args...);
 }
 
 // Sources are read from (k_src, v_src) - the destination pools themselves unless the plan names a

@@ -436,17 +436,25 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 pl->n_slots += parts_a + (b2 >= 0 ? parts_b : 0);
             }
         }
+        auto cycles_of = [&](const AttnWork &w) {
+            const int sa = std::min(w.step_end, steps_of(w.tile_a)) - w.step_begin;
+            const int sb = w.tile_b >= 0 ? std::min(w.step_end, steps_of(w.tile_b)) - w.step_begin : 0;
+            return model_cycles(sa, sb, w.tile_b >= 0 ? 2 : 1);
+        };
         // cost of an item = its (tile, 128-key step) count, kept in the item for the sorts
         for (AttnWork &w : pl->work) {
             int c = std::min(w.step_end, steps_of(w.tile_a)) - w.step_begin;
             if (w.tile_b >= 0) c += std::min(w.step_end, steps_of(w.tile_b)) - w.step_begin;
             w.cost = c;
         }
-        // Launch latency is a visible part of a layer only while the attention list fits the SMs once (2 items,
-        // 304 tokens: 20.6 -> 19.1 us a layer; 144 items, 5 312 tokens: 62.3 -> 56.2).  With longer lists a chained
-        // attention kernel measured slower than an ordinary launch (8 192 rows in 1 024 items, 16 requests: 481 us
-        // a layer against 450; 82 291 rows in 20 696 items: 13.1 ms against 12.4).
-        pl->chained = (int)pl->work.size() <= num_sms;
+        // Launch latency is a visible part of a layer while the attention takes tens of microseconds: 2 items
+        // 20.6 -> 19.1 us a layer, 144 items of 9 steps 51.5 -> 51.2 (62.3 -> 56.2 before the lists were cut by modelled
+        // time), 240 items of up to 8 steps 53.0 -> 48.3, 1 680 short items 121.1 -> 114.6.  Layers whose attention runs
+        // for hundreds of microseconds, near the power limit, lose: 1 024 items (219 us modelled) 436 -> 444 us, 1 152
+        // items (1 870 us) 2 715 -> 2 742, 20 696 items 12.35 -> 12.6 ms.
+        int64_t modelled_cycles = 0;
+        for (const AttnWork &w : pl->work) modelled_cycles += cycles_of(w);
+        pl->chained = modelled_cycles / num_sms <= kChainedCycles;
         pl->mma_pairs = 0;
         for (const AttnWork &w : pl->work) pl->mma_pairs += (int64_t)w.cost * kAttnTileRows * page;
         auto cost = [](const AttnWork &w) { return w.cost; };
@@ -521,19 +529,14 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         auto lpt_layout = [&](std::vector<AttnWork> &list) {
             const int G = num_sms;
             if ((int)list.size() <= G || (int)list.size() > kLptMaxItemsPerBlock * G) return;
-            auto cycles = [&](const AttnWork &w) -> int64_t {
-                const int sa = std::min(w.step_end, steps_of(w.tile_a)) - w.step_begin;
-                const int sb = w.tile_b >= 0 ? std::min(w.step_end, steps_of(w.tile_b)) - w.step_begin : 0;
-                return model_cycles(sa, sb, w.tile_b >= 0 ? 2 : 1);
-            };
             std::vector<int> order(list.size());
             std::iota(order.begin(), order.end(), 0);
-            std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cycles(list[a]) > cycles(list[b]); });
+            std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cycles_of(list[a]) > cycles_of(list[b]); });
             std::vector<int64_t> load(G, 0);
             std::vector<std::vector<int>> mine(G);
             for (int i : order) {
                 const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-                load[b] += cycles(list[i]);
+                load[b] += cycles_of(list[i]);
                 mine[b].push_back(i);
             }
             size_t rounds = 0;

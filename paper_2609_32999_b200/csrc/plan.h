@@ -16,6 +16,7 @@ constexpr int kAttnTileRows = 128;      // query rows (tokens x grouped heads) p
 constexpr int kDefaultSMs = 148;         // SM count assumed by a host-only plan (a B200); device plans ask the device
 constexpr int kSplitMinSteps = 2;        // never split below this many 128-key steps per part
 constexpr int kSplitMaxParts = 32;
+constexpr int kChainedCycles = 300000;   // modelled attention cycles per SM up to which launches are chained
 constexpr int kSplitMaxRounds = 4;       // batches of more attention items per SM than this are never split
 constexpr int kHostChunks = 4;          // request chunks of the host-buffer entry point's copy / compute pipeline
 constexpr int kLptMaxItemsPerBlock = 16;  // above this many attention items per thread block the plain serpentine walk is kept
@@ -115,7 +116,7 @@ struct tessera_plan {
     std::vector<tessera::CombineItem> combine;     // grouped by chunk: [chunk_combine_off[c], chunk_combine_off[c+1])
     std::vector<int32_t> chunk_combine_off;
     int32_t n_work_items = 0;                      // real items of `work` (the list may hold holes)
-    // Kernels of the plan's calls are launched chained (see launch_kernel): at most one attention item per SM.
+    // Kernels of the plan's calls are launched chained (see launch_kernel): the attention is short.
     bool chained = false;
     int32_t n_slots = 0;                           // split-KV workspace slots (0 = nothing is split)
     int32_t attn_kernel = 0;
