@@ -25,7 +25,7 @@ std::string fmt(const char *f, long a = 0, long b = 0, long c = 0) {
 
 // Merge of a split list in SM cycles: the launch and its first loads, and 65 KB of partial results per slot
 // written and read back through L2.
-constexpr int64_t kMergeCycles = 5000, kMergeCyclesPerSlot = 30;
+constexpr int64_t kMergeCycles = 9000, kMergeCyclesPerSlot = 30;
 
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
@@ -347,11 +347,12 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             first = last;
         }
         auto steps_of = [&](int32_t tile) { return (pl->tiles[tile].kv_len + page - 1) / page; };
-        // Modelled cycles of an item (clock64 on a B200): item fetch 700, epilogue + first step 3 150 per tile,
-        // 3 180 per step of both tiles, 1 650 per step of one.
+        // Modelled cycles of an item (clock64 on a B200): item fetch 1 700, epilogue and what the first step takes
+        // longer than a later one 4 700 per tile, 3 180 per step of both tiles, 2 400 per step of a lone one (whose
+        // softmax and MMAs wait for each other).
         auto model_cycles = [](int steps_a, int steps_b, int n_tiles) -> int64_t {
             const int both = std::min(steps_a, steps_b), single = std::max(steps_a, steps_b) - both;
-            return 700 + (int64_t)n_tiles * 3150 + (int64_t)both * 3180 + (int64_t)single * 1650;
+            return 1700 + (int64_t)n_tiles * 4700 + (int64_t)both * 3180 + (int64_t)single * 2400;
         };
         // Split-KV: the key ranges of a batch that leaves SMs idle are cut into parts of at most `limit` steps
         // that run as separate items and are merged afterwards.
@@ -360,9 +361,12 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         //                      (5 312 tokens, 48 items: parts of at most 14 steps before, 9 now; attention
         //                      39.4 -> 35.7 us; 5 requests of 2 048 tokens, 2 KV heads of 64: the whole layer
         //                      41.0 -> 28.6 us).
-        //   items <= kSplitMaxRounds x SMs : the limit with the least modelled time, if that is at least 5 %
+        //   items <= kSplitMaxRounds x SMs : the limit with the least modelled time, if that is at least 10 %
         //                      below the uncut list's (168 items of 260 steps take two rounds on 148 SMs; cut in
-        //                      parts they fill all rounds).
+        //                      parts they fill all rounds).  Attention of n requests of two tiles each, 12 288
+        //                      keys: 80 items 185 -> 150 us, 96 items 195 -> 162, 152 items 368 -> 310; 4 096 keys:
+        //                      left alone, a cut gains nothing (152 items 140 us, cut in 456 130-146).  128 items of
+        //                      77 to 224 steps: layer 570 -> 502 us.
         //   more             : never; the rounds are even enough and the merge only costs.
         auto parts_of = [&](int steps, int limit) {
             return std::max(1, std::min({(steps + limit - 1) / limit, kSplitMaxParts, steps / kSplitMinSteps}));
@@ -406,7 +410,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             int64_t all = 0;
             for (auto &pr : pairs)
                 all += Hkv * model_cycles(pr.second >= 0 ? steps_of(pr.first) : 0, long_steps(pr), pr.second >= 0 ? 2 : 1);
-            int64_t best = modelled(longest) * 95 / 100;
+            int64_t best = modelled(longest) * 90 / 100;
             if (best > all / num_sms)           // otherwise no cut can reach it
                 for (int l = longest * 3 / 4; l >= 2 * kSplitMinSteps && items_at(l) <= 2 * kSplitMaxRounds * num_sms; l = l * 5 / 6) {
                     const int64_t m = modelled(l);
