@@ -433,11 +433,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         const int rows[2] = {lane16 + (lane >> 2), lane16 + (lane >> 2) + 8};
         const int cq = (lane & 3) * 2;                                 // first of the thread's two columns in every group of 8
         int step_base[2] = {0, 0};                     // steps of each tile in earlier work items (barrier phases go on)
-        // where this thread's two bf16 of (row, column group kk) go in the swizzled output tile: rows r and
-        // r + 8 share r % 8, so one table of eight offsets serves both
-        uint32_t stage_off[8];
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) stage_off[kk] = (uint32_t)(rows[0] * 128 + ((kk ^ (rows[0] & 7)) << 4) + cq * 2);
         auto quad_max = [](float v) {
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
             return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
@@ -636,15 +631,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             if constexpr (kD == 128) tmem_ld_16x256b_x16(tO, o); else tmem_ld_16x256b_x8(tO, o);
             tmem_wait_ld();
             if (full_tile) {
+                // One stmatrix stores four 8 x 8 blocks: rows [0, 8) and [8, 16) of column groups k and k + 1.  Lane
+                // 8 i + j addresses row j of block i (16 bytes: chunk k % 8 of the row, swizzled by j).
+                const uint32_t row_addr = smem_u32(stage) + (uint32_t)(lane16 + ((lane >> 3) & 1) * 8 + (lane & 7)) * 128;
 #pragma unroll
-                for (int rr = 0; rr < 2; ++rr)
+                for (int k = 0; k < kD / 8; k += 2) {
+                    uint32_t y[4];
 #pragma unroll
-                    for (int k = 0; k < kD / 8; ++k) {
-                        // columns 8k + cq, + 1 of row rows[rr]: 16-byte chunk k % 8 of 64-column half k / 8
+                    for (int i = 0; i < 4; ++i) {          // block i: rows of half i % 2, columns of group k + i / 2
                         float y0, y1;
-                        fma2(y0, y1, __uint_as_float(o[4 * k + 2 * rr]), __uint_as_float(o[4 * k + 2 * rr + 1]), inv[rr], 0.f);
-                        *reinterpret_cast<uint32_t *>(stage + (k >> 3) * kHalfBytes + rr * (8 * 128) + stage_off[k & 7]) = pack_bf16(y0, y1);
+                        const int e = 4 * (k + (i >> 1)) + 2 * (i & 1);
+                        fma2(y0, y1, __uint_as_float(o[e]), __uint_as_float(o[e + 1]), inv[i & 1], 0.f);
+                        y[i] = pack_bf16(y0, y1);
                     }
+                    stmatrix_x4(row_addr + (k >> 3) * kHalfBytes + ((((k & 7) + (lane >> 4)) ^ (lane & 7)) << 4), y);
+                }
             } else {
                 // a request's last, partly filled tile: 4-byte stores straight to `out`
 #pragma unroll
