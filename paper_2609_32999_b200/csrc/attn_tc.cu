@@ -614,11 +614,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                 continue;
             }
             const float inv[2] = {__frcp_rn(l_tot[0]), __frcp_rn(l_tot[1])};
-#pragma unroll
-            for (int rr = 0; rr < 2; ++rr)
-                if (lse && row_valid[q][rr] && (lane & 3) == 0)
-                    lse[(size_t)(t.q_begin + tok[q][rr]) * H_q + kvh * g + rows[rr] % g] =
-                        (m_row[q][rr] + log2f(l_tot[rr])) * 0.6931471805599453f;
             const bool full_tile = t.n_tok == kRows / g;
             uint8_t *stage = sm + G::kSmemStage;
             if (full_tile) {
@@ -668,6 +663,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                     bulk_commit();
                 }
             }
+#pragma unroll
+            for (int rr = 0; rr < 2; ++rr)
+                if (lse && row_valid[q][rr] && (lane & 3) == 0)
+                    lse[(size_t)(t.q_begin + tok[q][rr]) * H_q + kvh * g + rows[rr] % g] =
+                        (m_row[q][rr] + log2f(l_tot[rr])) * 0.6931471805599453f;
         }
         step_base[0] += n_steps0;
         step_base[1] += n_steps1;
