@@ -125,8 +125,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_o,
                const AttnTile *__restrict__ tiles,
                const AttnWork *__restrict__ work, int n_work, const int32_t *__restrict__ q_pos,
-               const int32_t *__restrict__ page_off, const int32_t *__restrict__ pages,
-               const int32_t *__restrict__ seq_len, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse,
+               const int32_t *__restrict__ pages, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse,
                int H_q, int g, int page_size, int num_pool_pages, float scale_log2,
                float *__restrict__ ws_o, float2 *__restrict__ ws_ml, int *status) {
     extern __shared__ uint8_t smem_raw[];
@@ -173,9 +172,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         it.n_steps0 = min(it.wk.step_end, (it.t0.kv_len + kStep - 1) / kStep) - it.step0;
         it.n_steps1 = it.n_tiles == 2 ? min(it.wk.step_end, (it.t1.kv_len + kStep - 1) / kStep) - it.step0 : 0;
         it.n_steps = max(it.n_steps0, it.n_steps1);
-        it.T = seq_len[it.t0.req];
+        it.T = it.wk.seq_len;
         it.req_pages = (it.T + page_size - 1) / page_size;
-        it.bt = pages + page_off[it.t0.req];
+        it.bt = pages + it.wk.page_begin;
         return it;
     };
 
@@ -769,7 +768,7 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
     // places blocks 2 i and 2 i + 1 that way by itself, a chained one wherever an SM becomes free: 1 680 items,
     // head_dim 64: 93 us of mean block time with neighbours together, 103 us without.
     e = launch_clusters(
-        attn_tc_kernel<D, kMaxPages, K8>, grid, kThreads, grid % 2 == 0 ? 2 : 1, Geo<D>::kSmemAlloc, st, pl->chained && chunk < 0, tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.page_off, d.pages, d.seq_len,
+        attn_tc_kernel<D, kMaxPages, K8>, grid, kThreads, grid % 2 == 0 ? 2 : 1, Geo<D>::kSmemAlloc, st, pl->chained && chunk < 0, tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.pages,
         static_cast<__nv_bfloat16 *>(out), lse, Hq, g, ps, pl->num_pool_pages, scale_log2, d.ws_o, d.ws_ml, d.status);
     if (e == cudaSuccess && !pl->combine.empty()) {
         const int c0 = chunk < 0 ? 0 : pl->chunk_combine_off[chunk];

@@ -426,14 +426,14 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             const int parts_b = (sl + len - 1) / len, parts_a = b2 >= 0 ? (sa + len - 1) / len : parts_b;
             for (int h = 0; h < Hkv; ++h) {
                 if (parts == 1) {
-                    pl->work.push_back({a, b2, h, 0, sl, -1, -1, 0});
+                    pl->work.push_back({a, b2, h, 0, sl, -1, -1, 0, 0, 0, 0, 0});
                     continue;
                 }
                 const int32_t slot_a = pl->n_slots, slot_b = slot_a + parts_a;
                 for (int p2 = 0; p2 < parts_b; ++p2) {
                     const int sb = p2 * len, se = std::min(sl, sb + len);
-                    if (p2 < parts_a) pl->work.push_back({a, b2, h, sb, se, slot_a + p2, b2 >= 0 ? slot_b + p2 : -1, 0});
-                    else pl->work.push_back({b2, -1, h, sb, se, slot_b + p2, -1, 0});   // tile a is already finished
+                    if (p2 < parts_a) pl->work.push_back({a, b2, h, sb, se, slot_a + p2, b2 >= 0 ? slot_b + p2 : -1, 0, 0, 0, 0, 0});
+                    else pl->work.push_back({b2, -1, h, sb, se, slot_b + p2, -1, 0, 0, 0, 0, 0});   // tile a is already finished
                 }
                 pl->combine.push_back({a, h, parts_a, slot_a});
                 if (b2 >= 0) pl->combine.push_back({b2, h, parts_b, slot_b});
@@ -450,6 +450,9 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             int c = std::min(w.step_end, steps_of(w.tile_a)) - w.step_begin;
             if (w.tile_b >= 0) c += std::min(w.step_end, steps_of(w.tile_b)) - w.step_begin;
             w.cost = c;
+            const int32_t req = pl->tiles[w.tile_a].req;
+            w.seq_len = pl->seq_len[req];
+            w.page_begin = pl->page_off[req];
         }
         // Launch latency is a visible part of a layer while the attention takes tens of microseconds: 2 items
         // 20.6 -> 19.1 us a layer, 144 items of 9 steps 51.5 -> 51.2 (62.3 -> 56.2 before the lists were cut by modelled

@@ -48,6 +48,9 @@ struct AttnTile {
 struct AttnWork {
     int32_t tile_a, tile_b, kvh, step_begin, step_end, slot_a, slot_b;
     int32_t cost;      // (tile, step) count of the item: the host's sort key, not read by the kernel
+    int32_t seq_len, page_begin;   // of the request: its length and first block-table entry (so that the loads of K and V
+                                   // wait for this record and the page ids only, not for a chain through the tiles)
+    int32_t pad0, pad1;
 };
 
 // One (query tile, KV head) whose partial results have to be merged after a split-KV launch.
