@@ -435,8 +435,9 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                     if (p2 < parts_a) pl->work.push_back({a, b2, h, sb, se, slot_a + p2, b2 >= 0 ? slot_b + p2 : -1, 0, 0, 0, 0, 0});
                     else pl->work.push_back({b2, -1, h, sb, se, slot_b + p2, -1, 0, 0, 0, 0, 0});   // tile a is already finished
                 }
-                pl->combine.push_back({a, h, parts_a, slot_a});
-                if (b2 >= 0) pl->combine.push_back({b2, h, parts_b, slot_b});
+                const AttnTile &ta = pl->tiles[a], &tb = pl->tiles[b2 >= 0 ? b2 : a];
+                pl->combine.push_back({a, h, parts_a, slot_a, ta.q_begin, ta.n_tok, 0, 0});
+                if (b2 >= 0) pl->combine.push_back({b2, h, parts_b, slot_b, tb.q_begin, tb.n_tok, 0, 0});
                 pl->n_slots += parts_a + (b2 >= 0 ? parts_b : 0);
             }
         }

@@ -56,6 +56,8 @@ struct AttnWork {
 // One (query tile, KV head) whose partial results have to be merged after a split-KV launch.
 struct CombineItem {
     int32_t tile, kvh, n_parts, slot0;   // partial results in workspace slots [slot0, slot0 + n_parts)
+    int32_t q_begin, n_tok;              // of the tile
+    int32_t pad0, pad1;
 };
 
 struct DeviceTables {
