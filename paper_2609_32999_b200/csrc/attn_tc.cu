@@ -692,11 +692,11 @@ template <int kD>
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const CombineItem *__restrict__ items, const float *__restrict__ ws_o, const float2 *__restrict__ ws_ml, __nv_bfloat16 *__restrict__ out,
                     float *__restrict__ lse, int H_q, int g) {
-    grid_wait();
-    grid_release();
     const CombineItem it = items[blockIdx.x / kCombineBlocks];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row0 = (blockIdx.x % kCombineBlocks) * 16 + warp * 2;
+    grid_wait();
+    grid_release();
     if (row0 >= it.n_tok * g) return;
     constexpr int kBatch = 4;          // one batch holds all parts as a rule
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};

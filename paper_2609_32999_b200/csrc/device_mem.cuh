@@ -7,8 +7,10 @@ namespace tessera {
 
 // Programmatic dependent launch: a kernel started through launch_kernel(.., chained = true) may be resident while
 // its predecessor in the stream still runs.  grid_wait() returns once every preceding grid has completed and its
-// writes are visible; every kernel launched that way calls it in all threads before its first access to global
-// memory (so a grid's completion implies its predecessors').  grid_release() lets the successor's blocks take the
+// writes are visible; every kernel launched that way calls it in all threads (so a grid's completion implies its
+// predecessors') before its first access to anything a kernel may have written.  The plan's tables are not among
+// that: they were copied before the first launch of the plan, and a chained kernel waits for copies and events
+// like any other.  grid_release() lets the successor's blocks take the
 // room that this grid's last wave leaves.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -89,8 +89,6 @@ gather_rope_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 
     __shared__ float2 s_rope[kGatherItemTokens * (D / 2)];
     __shared__ int32_t s_src[kGatherItemTokens], s_dst[kGatherItemTokens];
 
-    grid_wait();
-    grid_release();
     const int tid = threadIdx.x;
     const GatherItem it = items[blockIdx.x];
     // rows row0, row0 + step, ... of the table; with step = -1 they are staged in ascending order
@@ -101,6 +99,8 @@ gather_rope_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 
         s_dst[tid] = g_dst[it.begin + tid];
         s_src[tid] = IN_PLACE ? s_dst[tid] : g_src[it.begin + tid];
     }
+    grid_wait();
+    grid_release();
     __syncthreads();
 
     const int tasks_per_row = H_kv * CPH;
@@ -225,15 +225,17 @@ __global__ void __launch_bounds__(256)
 scatter_fresh_kernel(uint4 *__restrict__ k_pool, uint4 *__restrict__ v_pool,
                      const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new,
                      const int32_t *__restrict__ fresh_dst, int64_t first_chunk, int64_t n_chunks, int row_chunks) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, end = first_chunk + n_chunks;
+    int64_t e = first_chunk + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int32_t slot = e < end ? fresh_dst[e / row_chunks] : 0;
     grid_wait();
     grid_release();
-    for (int64_t e = first_chunk + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < first_chunk + n_chunks;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = e / row_chunks;
-        const int c = (int)(e - j * row_chunks);
-        const size_t o = (size_t)fresh_dst[j] * row_chunks + c;
+    while (e < end) {
+        const size_t o = (size_t)slot * row_chunks + (int)(e % row_chunks);
         if (k_new) stg(k_pool + o, ldg_stream(k_new + e));
         if (v_new) stg(v_pool + o, ldg_stream(v_new + e));
+        e += step;
+        if (e < end) slot = fresh_dst[e / row_chunks];
     }
 }
 
@@ -246,14 +248,14 @@ rope_fresh_kernel(uint4 *__restrict__ q, uint4 *__restrict__ k_new, const int32_
                   const double *__restrict__ inv_freq, int H_q, int H_kv) {
     constexpr int CPH = D / 16, HALF = D / 16;
     __shared__ float2 s_cs[D / 2];
-    grid_wait();
-    grid_release();
     const int j = blockIdx.x, tid = threadIdx.x;
     if (tid < D / 2) {
         double sn, cs;
         sincos((double)q_pos[j] * inv_freq[tid], &sn, &cs);
         s_cs[tid] = make_float2((float)cs, (float)sn);
     }
+    grid_wait();
+    grid_release();
     __syncthreads();
     const int c = tid % CPH;
     float2 cr[8];
@@ -290,8 +292,6 @@ extend_write_kernel(uint4 *__restrict__ q, const uint4 *__restrict__ k_raw, cons
     constexpr int CPH = D / 16, HALF = D / 16;
     __shared__ float2 s_cs[kExtendRows][D / 2];
     __shared__ int32_t s_dst[kExtendRows], s_keep[kExtendRows];
-    grid_wait();
-    grid_release();
     const int tid = threadIdx.x;
     const int j0 = blockIdx.x * kExtendRows;
     const int rows = min(kExtendRows, n_q - j0);
@@ -305,6 +305,8 @@ extend_write_kernel(uint4 *__restrict__ q, const uint4 *__restrict__ k_raw, cons
         s_dst[tid] = fresh_dst[j0 + tid];
         s_keep[tid] = retain_dst ? retain_dst[j0 + tid] : -1;
     }
+    grid_wait();
+    grid_release();
     __syncthreads();
     const int c = tid % CPH;                        // 256 and every task count below are multiples of CPH
     const int kv_tasks = H_kv * CPH, q_tasks = q ? H_q * CPH : 0;

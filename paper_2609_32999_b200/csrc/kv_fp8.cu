@@ -108,8 +108,6 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
     __shared__ float2 s_rope[kGatherItemTokens * (D / 2)];
     __shared__ int32_t s_src[kGatherItemTokens], s_dst[kGatherItemTokens];
 
-    grid_wait();
-    grid_release();
     const int tid = threadIdx.x;
     const GatherItem it = items[blockIdx.x];
     const int n_rows = ROTATE ? (it.row_step ? it.count : 1) : 0;
@@ -119,6 +117,8 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
         s_dst[tid] = g_dst[it.begin + tid];
         s_src[tid] = g_src[it.begin + tid];
     }
+    grid_wait();
+    grid_release();
     __syncthreads();
 
     const int tasks_per_row = H_kv * CPH;
