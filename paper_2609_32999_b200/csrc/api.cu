@@ -70,14 +70,11 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     const size_t o_fresh = place<int32_t>(off, pl->fresh_dst.size());
     const size_t o_retain = place<int32_t>(off, pl->retain_dst.size());
     const size_t o_qpos = place<int32_t>(off, pl->recompute_pos.size());
-    const size_t o_qreq = place<int32_t>(off, pl->q_req.size());
-    const size_t o_poff = place<int32_t>(off, pl->page_off.size());
     const size_t o_pages = place<int32_t>(off, pl->pages.size());
     const size_t o_tiles = place<AttnTile>(off, pl->tiles.size());
     const size_t o_work = place<AttnWork>(off, pl->work.size());
     const size_t o_workc = place<AttnWork>(off, pl->work_chunked.size());
     const size_t o_comb = place<CombineItem>(off, pl->combine.size());
-    const size_t o_seq = place<int32_t>(off, pl->seq_len.size());
     const size_t o_status = place<int32_t>(off, 4);
     const size_t o_invf = place<double>(off, pl->inv_freq.size());
     // split-KV workspace: one slot per (tile, KV head, part)
@@ -96,15 +93,12 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     put(o_fresh, pl->fresh_dst.data(), pl->fresh_dst.size() * 4);
     put(o_retain, pl->retain_dst.data(), pl->retain_dst.size() * 4);
     put(o_qpos, pl->recompute_pos.data(), pl->recompute_pos.size() * 4);
-    put(o_qreq, pl->q_req.data(), pl->q_req.size() * 4);
-    put(o_poff, pl->page_off.data(), pl->page_off.size() * 4);
     put(o_pages, pl->pages.data(), pl->pages.size() * 4);
     put(o_tiles, pl->tiles.data(), pl->tiles.size() * sizeof(AttnTile));
     put(o_work, pl->work.data(), pl->work.size() * sizeof(AttnWork));
     put(o_workc, pl->work_chunked.data(), pl->work_chunked.size() * sizeof(AttnWork));
     put(o_comb, pl->combine.data(), pl->combine.size() * sizeof(CombineItem));
     put(o_invf, pl->inv_freq.data(), pl->inv_freq.size() * sizeof(double));
-    put(o_seq, pl->seq_len.data(), pl->seq_len.size() * 4);
     TS_CUDA(blob_acquire(&d.blob, off, &d.blob_bytes, st));
     TS_CUDA(cudaMemcpyAsync(d.blob, hb, table_bytes, cudaMemcpyHostToDevice, st));
     char *db = static_cast<char *>(d.blob);
@@ -116,8 +110,6 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     d.fresh_dst = reinterpret_cast<int32_t *>(db + o_fresh);
     d.retain_dst = pl->retain_dst.empty() ? nullptr : reinterpret_cast<int32_t *>(db + o_retain);
     d.q_pos = reinterpret_cast<int32_t *>(db + o_qpos);
-    d.q_req = reinterpret_cast<int32_t *>(db + o_qreq);
-    d.page_off = reinterpret_cast<int32_t *>(db + o_poff);
     d.pages = reinterpret_cast<int32_t *>(db + o_pages);
     d.tiles = reinterpret_cast<AttnTile *>(db + o_tiles);
     d.work = reinterpret_cast<AttnWork *>(db + o_work);
@@ -125,7 +117,6 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     d.combine = reinterpret_cast<CombineItem *>(db + o_comb);
     d.ws_ml = reinterpret_cast<float2 *>(db + o_wsml);
     d.ws_o = reinterpret_cast<float *>(db + o_wso);
-    d.seq_len = reinterpret_cast<int32_t *>(db + o_seq);
     d.status = reinterpret_cast<int32_t *>(db + o_status);
     d.inv_freq = reinterpret_cast<double *>(db + o_invf);
     return TESSERA_OK;

@@ -168,7 +168,6 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
     pl->src_slot.assign((size_t)total, -1);
     pl->recompute_off.assign(d->recompute_off, d->recompute_off + batch + 1);
     pl->recompute_pos.assign(d->recompute_pos, d->recompute_pos + n_q);
-    pl->q_req.resize(n_q);
     pl->fresh_dst.resize(n_q);
     pl->g_src.clear(); pl->g_dst.clear(); pl->items.clear();
     std::vector<int32_t> unit_of((size_t)total, -1);
@@ -203,7 +202,6 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 return fail(TESSERA_UNSORTED_POSITIONS, fmt("request %ld: recompute positions not strictly ascending at index %ld", r, j));
             fresh[base + p] = 1;
             fresh_row[base + p] = j;
-            pl->q_req[j] = r;
             pl->fresh_dst[j] = pl->pages[pl->page_off[r] + p / B] * B + p % B;
             pl->qk_pairs += (int64_t)p + 1;
         }

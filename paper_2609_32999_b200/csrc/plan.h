@@ -70,8 +70,6 @@ struct DeviceTables {
     int32_t *fresh_dst = nullptr;  // [n_q] destination slot of each recompute row
     int32_t *retain_dst = nullptr; // [n_q] cache slot of a captured row, -1 otherwise (null: nothing is captured)
     int32_t *q_pos = nullptr;      // [n_q]
-    int32_t *q_req = nullptr;      // [n_q]
-    int32_t *page_off = nullptr;   // [batch+1]
     int32_t *pages = nullptr;      // block tables
     AttnTile *tiles = nullptr;
     AttnWork *work = nullptr;      // tcgen05 work items, longest first
@@ -79,7 +77,6 @@ struct DeviceTables {
     CombineItem *combine = nullptr;    // (tile, head) pairs to merge, grouped by request chunk
     float *ws_o = nullptr;             // split-KV partials: [slot][128 rows][128] unnormalised O ...
     float2 *ws_ml = nullptr;           // ... and [slot][128] (reference maximum in log2 units, sum)
-    int32_t *seq_len = nullptr;    // [batch]
     int32_t *status = nullptr;     // device status word(s)
     double *inv_freq = nullptr;    // [D/2] rotary frequencies
     // staging for the host-buffer entry point (allocated on first use)
@@ -103,7 +100,7 @@ struct tessera_plan {
                                            // kernel, target block count of split-KV and of the small-batch gather
 
     std::vector<int32_t> seq_len, tok_off, page_off, pages, src_slot;
-    std::vector<int32_t> recompute_off, recompute_pos, q_req, fresh_dst;
+    std::vector<int32_t> recompute_off, recompute_pos, fresh_dst;
     std::vector<int32_t> retain_dst;       // [n_q] or empty: cache slot of every captured recompute row
     int32_t retain_pool_pages = 0;         // > 0: captured units go to a separate cache pool of this many pages
     int64_t retained_tokens = 0;
