@@ -772,19 +772,21 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
     // persistent: one thread block per SM (fewer when the list is shorter)
     const int sms = max_blocks > 0 ? std::min(max_blocks, pl->num_sms) : pl->num_sms;
     unsigned grid = (unsigned)std::min<size_t>(n_work, (size_t)sms);
-    if (grid % 2 != 0 && grid < (unsigned)sms) ++grid;      // (a block without an item ends at once)
-    // Clusters of two, though the blocks share nothing by themselves: neighbours in the list read the same K/V pages
-    // at about the same time, and the two SMs of a TPC fetch a line that both ask for once.  An ordinary launch
-    // places blocks 2 i and 2 i + 1 that way by itself, a chained one wherever an SM becomes free: 1 680 items,
-    // head_dim 64: 93 us of mean block time with neighbours together, 103 us without.
+    // A chained grid comes in clusters of two, though the blocks share nothing by themselves: neighbours in the list
+    // read the same K/V pages at about the same time, and the two SMs of a TPC fetch a line that both ask for once.
+    // An ordinary launch places blocks 2 i and 2 i + 1 that way by itself, a chained one wherever an SM becomes free:
+    // 1 680 items, head_dim 64: 93 us of mean block time with neighbours together, 103 us without.  (Ordinary
+    // launches stay without: beside the host-tier reader not every TPC has both its SMs free.)
+    const bool chained = pl->chained && chunk < 0;
+    if (chained && grid % 2 != 0 && grid < (unsigned)sms) ++grid;      // (a block without an item ends at once)
     e = launch_clusters(
-        attn_tc_kernel<D, kMaxPages, K8>, grid, kThreads, grid % 2 == 0 ? 2 : 1, Geo<D>::kSmemAlloc, st, pl->chained && chunk < 0, tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.pages,
+        attn_tc_kernel<D, kMaxPages, K8>, grid, kThreads, chained && grid % 2 == 0 ? 2 : 1, Geo<D>::kSmemAlloc, st, chained, tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.pages,
         static_cast<__nv_bfloat16 *>(out), lse, Hq, g, ps, pl->num_pool_pages, scale_log2, d.ws_o, d.ws_ml, d.status);
     if (e == cudaSuccess && !pl->combine.empty()) {
         const int c0 = chunk < 0 ? 0 : pl->chunk_combine_off[chunk];
         const int c1 = chunk < 0 ? (int)pl->combine.size() : pl->chunk_combine_off[chunk + 1];
         if (c1 > c0)
-            e = launch_kernel(attn_combine_kernel<D>, (unsigned)(c1 - c0) * kCombineBlocks, 256, 0, st, pl->chained && chunk < 0,
+            e = launch_kernel(attn_combine_kernel<D>, (unsigned)(c1 - c0) * kCombineBlocks, 256, 0, st, chained,
                               d.combine + c0, d.ws_o, d.ws_ml, static_cast<__nv_bfloat16 *>(out), lse, Hq, g);
     }
     if (e != cudaSuccess) *err = "kernel launch";
