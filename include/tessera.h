@@ -15,7 +15,8 @@
  *     of the calling thread's last failure.  Nothing throws, aborts or traps.
  *   - "host" / "device" beside a pointer says where the memory lives.  The caller owns every
  *     buffer it passes; host arrays may be freed as soon as the call returns.  The library owns
- *     only the opaque plan (its host tables, device tables and staging buffers).
+ *     only the opaque plan (its host tables, device tables and staging buffers) and at most 64 MB of
+ *     device memory of destroyed plans, kept for later ones.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Device
  *     work is enqueued on it and the call returns without waiting, unless stated otherwise.
  *   - One plan serves every layer of its batch, one call after the other.  Calls on the SAME plan
@@ -154,7 +155,7 @@ typedef struct tessera_plan_info {
 TESSERA_API int32_t tessera_plan_create(const tessera_model_cfg *cfg, const tessera_compose_desc *desc,
                             int32_t num_pool_pages, uint32_t flags, tessera_plan **out, void *stream);
 
-/* Frees host and device tables.  The caller must have synchronised every stream that used the plan. */
+/* Frees the plan (device memory may be kept for later plans).  The caller must have synchronised every stream that used the plan. */
 TESSERA_API int32_t tessera_plan_destroy(tessera_plan *plan);
 
 /*

@@ -1,6 +1,5 @@
 #include "blob_pool.h"
 
-#include <deque>
 #include <mutex>
 
 #include <cuda.h>
@@ -16,16 +15,14 @@ struct Block {
     unsigned long long context;   // id of the context the block belongs to: a block does not outlive a device reset
 };
 
+// A fixed array: nothing here allocates host memory, so nothing throws through the C entry points.
 struct Pool {
     std::mutex mutex;
-    std::deque<Block> blocks;     // oldest first
+    Block blocks[kBlobPoolBlocks];     // oldest first
+    int count = 0;
     size_t held = 0;
 };
-
-Pool &pool() {
-    static Pool *p = new Pool;    // never destroyed: the driver may be gone before static destructors run
-    return *p;
-}
+Pool g_pool;
 
 // Id of the current context, 0 when it cannot be asked for (then nothing is pooled).
 unsigned long long context_id() {
@@ -41,9 +38,10 @@ unsigned long long context_id() {
 }
 
 // Takes block i out of the pool.
-Block take(Pool &pl, size_t i) {
+Block take(Pool &pl, int i) {
     const Block b = pl.blocks[i];
-    pl.blocks.erase(pl.blocks.begin() + (std::ptrdiff_t)i);
+    for (int k = i; k + 1 < pl.count; ++k) pl.blocks[k] = pl.blocks[k + 1];
+    --pl.count;
     pl.held -= b.bytes;
     return b;
 }
@@ -61,16 +59,16 @@ cudaError_t blob_acquire(void **p, size_t bytes, size_t *granted, cudaStream_t s
     while (step * 8 < bytes) step *= 2;
     bytes = (bytes + step - 1) / step * step;
     const unsigned long long context = context_id();
-    Pool &pl = pool();
+    Pool &pl = g_pool;
     std::lock_guard<std::mutex> lock(pl.mutex);
     if (capturing == cudaStreamCaptureStatusNone) {
-        size_t best = pl.blocks.size();
-        for (size_t i = 0; i < pl.blocks.size(); ++i) {
+        int best = -1;
+        for (int i = 0; i < pl.count; ++i) {
             const Block &b = pl.blocks[i];
             if (b.device != device || b.context != context || b.bytes < bytes || b.bytes > 2 * bytes) continue;
-            if (best == pl.blocks.size() || b.bytes < pl.blocks[best].bytes) best = i;
+            if (best < 0 || b.bytes < pl.blocks[best].bytes) best = i;
         }
-        if (best < pl.blocks.size()) {
+        if (best >= 0) {
             const Block b = take(pl, best);
             *p = b.p;
             *granted = b.bytes;
@@ -80,7 +78,7 @@ cudaError_t blob_acquire(void **p, size_t bytes, size_t *granted, cudaStream_t s
     e = cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation) {
         bool any = false;
-        for (size_t i = pl.blocks.size(); i-- > 0;)
+        for (int i = pl.count; i-- > 0;)
             if (pl.blocks[i].device == device) {
                 const Block b = take(pl, i);
                 if (b.context == context) any |= cudaFree(b.p) == cudaSuccess;
@@ -105,11 +103,9 @@ cudaError_t blob_release(void *p, size_t bytes, int device) {
     } else if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
         cudaFree(p);
     } else {
-        Pool &pl = pool();
+        Pool &pl = g_pool;
         std::lock_guard<std::mutex> lock(pl.mutex);
-        pl.blocks.push_back({p, bytes, device, context});
-        pl.held += bytes;
-        while (pl.held > kBlobPoolBytes) {
+        while (pl.count == kBlobPoolBlocks || (pl.count > 0 && pl.held + bytes > kBlobPoolBytes)) {
             const Block b = take(pl, 0);
             if (b.device != device) cudaSetDevice(b.device);
             if (context_id() == b.context) {
@@ -118,6 +114,8 @@ cudaError_t blob_release(void *p, size_t bytes, int device) {
             }
             if (b.device != device) cudaSetDevice(device);
         }
+        pl.blocks[pl.count++] = {p, bytes, device, context};
+        pl.held += bytes;
     }
     if (current != device) cudaSetDevice(current);
     return e;
