@@ -401,8 +401,7 @@ int32_t tessera_partial_prefill_attn_k8(tessera_plan *pl, void *k_pool8, float k
     const int64_t q_elems = pl->n_q * pl->cfg.num_q_heads * pl->cfg.head_dim;
     if (!pl->dev.q8) TS_CUDA(cudaMalloc(&pl->dev.q8, (size_t)q_elems));
     // the reciprocals are taken once, in fp32: every element is multiplied by it and rounded to e4m3
-    TS_CUDA(launch_quantize_e4m3(q, pl->dev.q8, q_elems, 1.0f / q_scale, pl->chained, st));
-    TS_CUDA(launch_scatter_fresh_k8(pl, k_pool8, v_pool, k_new, v_new, 1.0f / k_scale, st));
+    TS_CUDA(launch_fresh_k8(pl, q, pl->dev.q8, 1.0f / q_scale, k_pool8, v_pool, k_new, v_new, 1.0f / k_scale, st));
     std::string err;
     cudaError_t e = launch_attn_tc_k8(pl, k_pool8, v_pool, pl->dev.q8, out, lse, q_scale * k_scale, st, &err);
     if (e != cudaSuccess) return set_error(TESSERA_CUDA_ERROR, "tcgen05 attention launch (8-bit keys): " + err + " / " + cudaGetErrorString(e));

@@ -250,32 +250,28 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
     }
 }
 
-// bf16 -> e4m3 codes of (value * mul): 8 elements per thread, grid-stride.
+// What the 8-bit-key attention needs of the fresh rows, in one launch: q as e4m3 codes of (value * q_mul) in the
+// plan's buffer, and the recompute tokens' K and V into an 8-bit key pool (codes of k * k_mul) and a 16-bit value
+// pool (bit copies; Sec. 5.3: recomputed states override cached ones).  8 elements per thread and turn, the q
+// chunks first.  (Two launches before: one request of
+// 807 tokens 23.5 -> 21.5 us a layer.)
 __global__ void __launch_bounds__(256)
-quantize_e4m3_kernel(const uint4 *__restrict__ src, uint2 *__restrict__ dst, int64_t n_chunks, float mul) {
+fresh_k8_kernel(const uint4 *__restrict__ q, uint2 *__restrict__ q8, int64_t n_q_chunks, float q_mul, uint2 *__restrict__ k_pool8,
+                uint4 *__restrict__ v_pool, const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new,
+                const int32_t *__restrict__ fresh_dst, int64_t n_kv_chunks, int row_chunks, float k_mul) {
     grid_wait();
     grid_release();
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_chunks; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t n = n_q_chunks + n_kv_chunks;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         float f[8];
-        unpack_bf16x8(ldg_stream(src + e), f);
-        dst[e] = pack_e4m3x8(f, mul);
-    }
-}
-
-// Fresh rows of the recompute tokens into an 8-bit key pool and a 16-bit value pool (Sec. 5.3: recomputed
-// states override cached ones): K as the e4m3 code of (k * k_mul), V as a bit copy.
-__global__ void __launch_bounds__(256)
-scatter_fresh_k8_kernel(uint2 *__restrict__ k_pool8, uint4 *__restrict__ v_pool, const uint4 *__restrict__ k_new,
-                        const uint4 *__restrict__ v_new, const int32_t *__restrict__ fresh_dst, int64_t n_chunks,
-                        int row_chunks, float k_mul) {
-    grid_wait();
-    grid_release();
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_chunks; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = e / row_chunks;
-        const int c = (int)(e - j * row_chunks);
-        const size_t o = (size_t)fresh_dst[j] * row_chunks + c;
+        if (t < n_q_chunks) {
+            unpack_bf16x8(ldg_stream(q + t), f);
+            q8[t] = pack_e4m3x8(f, q_mul);
+            continue;
+        }
+        const int64_t e = t - n_q_chunks, j = e / row_chunks;
+        const size_t o = (size_t)fresh_dst[j] * row_chunks + (int)(e - j * row_chunks);
         if (k_new) {
-            float f[8];
             unpack_bf16x8(ldg_stream(k_new + e), f);
             k_pool8[o] = pack_e4m3x8(f, k_mul);
         }
@@ -314,23 +310,18 @@ cudaError_t launch_compose_k8(const tessera_plan *pl, const void *k_src, const v
                          k_mul, 1.f);
 }
 
-cudaError_t launch_quantize_e4m3(const void *src_bf16, void *dst8, int64_t n_elems, float mul, bool chained, cudaStream_t st) {
-    const int64_t n_chunks = n_elems / 8;
-    if (n_chunks == 0) return cudaSuccess;
-    const int blocks = (int)std::min<int64_t>((n_chunks + 255) / 256, 148 * 16);
-    return launch_kernel(quantize_e4m3_kernel, (unsigned)blocks, 256, 0, st, chained, static_cast<const uint4 *>(src_bf16),
-                         static_cast<uint2 *>(dst8), n_chunks, mul);
-}
-
-cudaError_t launch_scatter_fresh_k8(const tessera_plan *pl, void *k_pool8, void *v_pool, const void *k_new,
-                                    const void *v_new, float k_mul, cudaStream_t st) {
-    if (pl->n_q == 0 || (!k_new && !v_new)) return cudaSuccess;
+cudaError_t launch_fresh_k8(const tessera_plan *pl, const void *q, void *q8, float q_mul, void *k_pool8, void *v_pool,
+                            const void *k_new, const void *v_new, float k_mul, cudaStream_t st) {
     const int row_chunks = pl->cfg.num_kv_heads * pl->cfg.head_dim / 8;
-    const int64_t n_chunks = pl->n_q * row_chunks;
-    const int blocks = (int)std::min<int64_t>((n_chunks + 255) / 256, (int64_t)pl->num_sms * 16);
-    return launch_kernel(scatter_fresh_k8_kernel, (unsigned)blocks, 256, 0, st, pl->chained, static_cast<uint2 *>(k_pool8),
-                         static_cast<uint4 *>(v_pool), static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new),
-                         pl->dev.fresh_dst, n_chunks, row_chunks, k_mul);
+    const int64_t n_q_chunks = pl->n_q * pl->cfg.num_q_heads * pl->cfg.head_dim / 8;
+    const int64_t n_kv_chunks = k_new || v_new ? pl->n_q * row_chunks : 0;
+    const int64_t n = n_q_chunks + n_kv_chunks;
+    if (n == 0) return cudaSuccess;
+    const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)pl->num_sms * 16);
+    return launch_kernel(fresh_k8_kernel, blocks, 256, 0, st, pl->chained, static_cast<const uint4 *>(q), static_cast<uint2 *>(q8),
+                         n_q_chunks, q_mul, static_cast<uint2 *>(k_pool8), static_cast<uint4 *>(v_pool),
+                         static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new), pl->dev.fresh_dst, n_kv_chunks, row_chunks,
+                         k_mul);
 }
 
 cudaError_t launch_kv_fp8(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst, void *v_dst,

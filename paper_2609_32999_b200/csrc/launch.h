@@ -81,10 +81,9 @@ cudaError_t launch_attn_tc_k8(const tessera_plan *pl, void *k_pool8, void *v_poo
 // k_dst8, values as bit copies in the 16-bit v_dst.
 cudaError_t launch_compose_k8(const tessera_plan *pl, const void *k_src, const void *v_src, void *k_dst8, void *v_dst,
                               bool rotate, float k_mul, cudaStream_t st);
-// bf16 rows -> e4m3 codes of (value * mul), nearest-even, saturating: n_elems elements (a multiple of 8).
-cudaError_t launch_quantize_e4m3(const void *src_bf16, void *dst8, int64_t n_elems, float mul, bool chained, cudaStream_t st);
-// Fresh rows into an 8-bit key pool (codes of k_new * k_mul) and a 16-bit value pool (bit copies).
-cudaError_t launch_scatter_fresh_k8(const tessera_plan *pl, void *k_pool8, void *v_pool, const void *k_new,
-                                    const void *v_new, float k_mul, cudaStream_t st);
+// Fresh rows of the 8-bit-key path: q -> e4m3 codes of (q * q_mul) in q8, k_new / v_new (null: skipped) into an 8-bit
+// key pool (codes of k_new * k_mul; nearest-even, saturating) and a 16-bit value pool (bit copies).
+cudaError_t launch_fresh_k8(const tessera_plan *pl, const void *q, void *q8, float q_mul, void *k_pool8, void *v_pool,
+                            const void *k_new, const void *v_new, float k_mul, cudaStream_t st);
 
 }  // namespace tessera
