@@ -431,6 +431,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         const uint32_t lane_base = (uint32_t)lane16 << 16;
         const int rows[2] = {lane16 + (lane >> 2), lane16 + (lane >> 2) + 8};
         const int cq = (lane & 3) * 2;                                 // first of the thread's two columns in every group of 8
+        // (divisions by the group size, once: in the items they cost 1 680 short ones 2 % - 109.8 -> 107.2 us a layer)
+        const int row_tok[2] = {rows[0] / g, rows[1] / g}, row_head[2] = {rows[0] % g, rows[1] % g};
         int step_base[2] = {0, 0};                     // steps of each tile in earlier work items (barrier phases go on)
         auto quad_max = [](float v) {
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -449,8 +451,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         const int n_tiles = it.n_tiles, n_steps = it.n_steps, n_steps0 = it.n_steps0, n_steps1 = it.n_steps1;
         const int step0 = it.step0, kvh = it.wk.kvh;
         const AttnTile &t0 = it.t0, &t1 = it.t1;
-        int tok[2][2], p_row[2][2];
-        bool row_valid[2][2];
+        int p_row[2][2];
         // reference maximum (identical in the four threads of a row) and this thread's share of the row sum
         float m_row[2][2] = {{-INFINITY, -INFINITY}, {-INFINITY, -INFINITY}}, l_row[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
@@ -458,9 +459,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             const AttnTile &t = q ? t1 : t0;
 #pragma unroll
             for (int rr = 0; rr < 2; ++rr) {
-                tok[q][rr] = min(rows[rr] / g, t.n_tok - 1);
-                row_valid[q][rr] = rows[rr] / g < t.n_tok;
-                p_row[q][rr] = q_pos[t.q_begin + tok[q][rr]];
+                p_row[q][rr] = q_pos[t.q_begin + min(row_tok[rr], t.n_tok - 1)];
             }
         }
 
@@ -644,8 +643,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                 // a request's last, partly filled tile: 4-byte stores straight to `out`
 #pragma unroll
                 for (int rr = 0; rr < 2; ++rr) {
-                    if (!row_valid[q][rr]) continue;
-                    __nv_bfloat16 *orow = out + ((size_t)(t.q_begin + tok[q][rr]) * H_q + kvh * g + rows[rr] % g) * kD + cq;
+                    if (row_tok[rr] >= t.n_tok) continue;
+                    __nv_bfloat16 *orow = out + ((size_t)(t.q_begin + row_tok[rr]) * H_q + kvh * g + row_head[rr]) * kD + cq;
 #pragma unroll
                     for (int k = 0; k < kD / 8; ++k)
                         *reinterpret_cast<uint32_t *>(orow + 8 * k) =
@@ -664,8 +663,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             }
 #pragma unroll
             for (int rr = 0; rr < 2; ++rr)
-                if (lse && row_valid[q][rr] && (lane & 3) == 0)
-                    lse[(size_t)(t.q_begin + tok[q][rr]) * H_q + kvh * g + rows[rr] % g] =
+                if (lse && row_tok[rr] < t.n_tok && (lane & 3) == 0)
+                    lse[(size_t)(t.q_begin + row_tok[rr]) * H_q + kvh * g + row_head[rr]] =
                         (m_row[q][rr] + log2f(l_tot[rr])) * 0.6931471805599453f;
         }
         step_base[0] += n_steps0;
