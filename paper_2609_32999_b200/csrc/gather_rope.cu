@@ -180,8 +180,7 @@ gather_runs_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 
     const int tasks_per_row = H_kv * CPH, row_chunks = H_kv * (D / 8);
     for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
         const GatherRun rn = runs[run];
-        const GatherItem src = items[rn.first_item];
-        const int n_tasks = src.count * tasks_per_row;
+        const int n_tasks = rn.count * tasks_per_row;
         for (int t0 = threadIdx.x; t0 < n_tasks; t0 += U * kThreads) {
             uint4 klo[U], khi[U], vlo[U], vhi[U];
 #pragma unroll
@@ -189,7 +188,7 @@ gather_runs_kernel(const uint4 *k_src, const uint4 *v_src, uint4 *k_pool, uint4 
                 const int t = t0 + u * kThreads;
                 if (t >= n_tasks) continue;
                 const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
-                const size_t so = (size_t)g_src[src.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
+                const size_t so = (size_t)g_src[rn.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
                 klo[u] = ldg_stream(k_src + so);
                 khi[u] = ldg_stream(k_src + so + HALF);
                 vlo[u] = ldg_stream(v_src + so);

@@ -207,8 +207,7 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
     const int tasks_per_row = H_kv * CPH, row_chunks = H_kv * (D / 8);
     for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
         const GatherRun rn = runs[run];
-        const GatherItem src = items[rn.first_item];
-        const int n_tasks = src.count * tasks_per_row;
+        const int n_tasks = rn.count * tasks_per_row;
         for (int t0 = threadIdx.x; t0 < n_tasks; t0 += U * kThreads) {
             uint2 rk[U][2], rv[U][2];
 #pragma unroll
@@ -216,7 +215,7 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
                 const int t = t0 + u * kThreads;
                 if (t >= n_tasks) continue;
                 const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
-                const size_t so = (size_t)g_src[src.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
+                const size_t so = (size_t)g_src[rn.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
                 rk[u][0] = ldg_stream(k_src + so);
                 rk[u][1] = ldg_stream(k_src + so + HALF);
                 rv[u][0] = ldg_stream(v_src + so);

@@ -295,7 +295,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         const int len = d->unit_len[users[0].unit];
         for (int i0 = 0; i0 < len; i0 += item_tokens) {
             const int cnt = std::min(item_tokens, len - i0);
-            pl->runs.push_back({(int32_t)pl->items.size(), (int32_t)users.size()});
+            pl->runs.push_back({(int32_t)pl->items.size(), (int32_t)users.size(), (int32_t)pl->g_src.size(), cnt});
             for (const UnitUse &use : users) {
                 const int u = use.unit, tp = d->unit_target_pos[u];
                 const int64_t d0 = (int64_t)tp - d->unit_cached_pos[u];

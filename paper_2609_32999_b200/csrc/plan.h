@@ -32,6 +32,7 @@ struct GatherItem {
 // rows of the same cached unit (one item per request that uses it) and differ only in slots and shifts.
 struct GatherRun {
     int32_t first_item, n_items;
+    int32_t begin, count;      // of the first item: its source rows are everyone's
 };
 
 // One query tile of the attention kernel: `n_tok` consecutive recompute rows [q_begin, q_begin+n_tok)
