@@ -25,7 +25,7 @@ std::string fmt(const char *f, long a = 0, long b = 0, long c = 0) {
 
 // Merge of a split list in SM cycles: the launch and its first loads, and 65 KB of partial results per slot
 // written and read back through L2.
-constexpr int64_t kMergeCycles = 9000, kMergeCyclesPerSlot = 30;
+constexpr int64_t kMergeCycles = 9000, kMergeCyclesOneRound = 4500, kMergeCyclesPerSlot = 20;
 
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
@@ -358,12 +358,14 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         //                      limit, not a common part count: short tiles are not cut as often as long ones
         //                      (5 312 tokens, 48 items: parts of at most 14 steps before, 9 now; attention
         //                      39.4 -> 35.7 us; 5 requests of 2 048 tokens, 2 KV heads of 64: the whole layer
-        //                      41.0 -> 28.6 us).
+        //                      41.0 -> 28.6 us), unless the merge eats what that gains (448 tokens, 56 items of
+        //                      four steps: 54.2 us in the host-tier path, cut in 80 58.0).
         //   items <= kSplitMaxRounds x SMs : the limit with the least modelled time, if that is at least 10 %
         //                      below the uncut list's (168 items of 260 steps take two rounds on 148 SMs; cut in
         //                      parts they fill all rounds).  Attention of n requests of two tiles each, 12 288
-        //                      keys: 80 items 185 -> 150 us, 96 items 195 -> 162, 152 items 368 -> 310; 4 096 keys:
-        //                      left alone, a cut gains nothing (152 items 140 us, cut in 456 130-146).  128 items of
+        //                      keys: 80 items 185 -> 141 us, 96 items 195 -> 153, 152 items 368 -> 282 (in 760 parts;
+        //                      in at most 592, 296); 4 096 keys:
+        //                      left alone, a cut gains nothing (152 items 126-140 us, cut in 456 130-146).  128 items of
         //                      77 to 224 steps: layer 570 -> 502 us.
         //   more             : never; the rounds are even enough and the merge only costs.
         auto parts_of = [&](int steps, int limit) {
@@ -398,12 +400,15 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 end = std::max(end, load.back() += c);
                 std::push_heap(load.begin(), load.end(), std::greater<int64_t>());
             }
-            return end + (slots ? kMergeCycles + slots * kMergeCyclesPerSlot : 0);
+            const int64_t merge = cost.size() <= (size_t)num_sms ? kMergeCyclesOneRound : kMergeCycles;
+            return end + (slots ? merge + slots * kMergeCyclesPerSlot : 0);
         };
         int limit = longest;
         const int64_t uncut = (int64_t)pairs.size() * Hkv;
         if (uncut > 0 && 2 * uncut <= num_sms) {
-            while (limit > kSplitMinSteps && items_at(limit - 1) <= num_sms) --limit;
+            int l = longest;
+            while (l > kSplitMinSteps && items_at(l - 1) <= num_sms) --l;
+            if (modelled(l) < modelled(longest) * 90 / 100) limit = l;
         } else if (uncut > 0 && uncut <= (int64_t)kSplitMaxRounds * num_sms) {
             int64_t all = 0;
             for (auto &pr : pairs)
