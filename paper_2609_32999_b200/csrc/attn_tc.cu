@@ -718,15 +718,16 @@ attn_combine_kernel(const CombineItem *__restrict__ items, const float *__restri
             float mb = m[i];
 #pragma unroll
             for (int p = 0; p < kBatch; ++p) mb = fmaxf(mb, ml[i][p].x);
-            // the first part holds the key at position 0, which every row sees: mb is finite from the first batch on
-            // (a padding row's values are never stored)
-            const float w0 = exp2f(m[i] - mb);
+            // A row whose scores so far are all -inf (overflowed products; every row sees the key at position 0, so not
+            // for want of keys) has m = -inf, sum 0: the reference stays at 0, as in the attention kernel.
+            const float ref = mb == -INFINITY ? 0.f : mb;
+            const float w0 = exp2f(m[i] - ref);
             m[i] = mb;
             l[i] *= w0;
             acc[i].x *= w0; acc[i].y *= w0; acc[i].z *= w0; acc[i].w *= w0;
 #pragma unroll
             for (int p = 0; p < kBatch; ++p) {
-                const float w = exp2f(ml[i][p].x - mb);
+                const float w = exp2f(ml[i][p].x - ref);
                 l[i] += ml[i][p].y * w;
                 acc[i].x = fmaf(o[i][p].x, w, acc[i].x); acc[i].y = fmaf(o[i][p].y, w, acc[i].y);
                 acc[i].z = fmaf(o[i][p].z, w, acc[i].z); acc[i].w = fmaf(o[i][p].w, w, acc[i].w);

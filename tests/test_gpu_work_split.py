@@ -3,6 +3,7 @@ batch of the merge holds, lists that fit the SMs once, lists of one to four roun
 faster), lists left alone."""
 import numpy as np
 import pytest
+import torch
 
 from paper_2609_32999_b200 import binding as tb
 from paper_2609_32999_b200 import workloads as wl
@@ -35,3 +36,39 @@ def test_parity_where_the_work_list_changes(shape, requests, unit, units, tail, 
     asm, _, _ = gu.check_assembled(g)
     gu.check_untouched(g)
     gu.check_attention(g, asm)
+
+
+@pytest.mark.parametrize("masked_steps", [2, 9, 20])
+def test_parts_whose_scores_all_overflow_count_for_nothing(masked_steps):
+    """Scores of -inf in whole parts of a cut key range - more parts than the merge reads at once, too - leave the
+    later parts their weight: with equal finite scores the output is the mean of the visible finite keys' values."""
+    w = wl.build_workload("overflow", SHAPE_1, [[3] + [wl.unit(3000, ("u", i), recompute=(0, 5, 1500)) for i in range(2)] + [9]],
+                          np.random.default_rng(3))
+    plan = tb.Plan(w)
+    assert plan.info.n_attn_items == 16                    # 47 steps in parts of three
+    t = wl.make_tensors(w, device="cuda:0", seed=4)
+    page_off, pages, _ = plan.block_table()
+    T, B, dead = int(w.seq_len[0]), SHAPE_1.page_size, 128 * masked_steps
+    at = torch.from_numpy(pages[np.arange(T) // B].astype(np.int64) * B + np.arange(T) % B).to("cuda:0")
+    # q k = -1e40 a pair in the first `dead` keys, about 1 (the same everywhere) in the others
+    t.q.fill_(1e20)
+    k = t.k_pool.flatten(0, 1)
+    k[at[:dead]], k[at[dead:]] = -1e20, 1e-20
+    pos = torch.from_numpy(w.recompute_pos.astype(np.int64)).to("cuda:0")
+    v = t.v_pool.flatten(0, 1)
+    v[at] = torch.randn(T, *v.shape[1:], device="cuda:0", generator=torch.Generator("cuda:0").manual_seed(1)).to(torch.bfloat16)
+    out, lse = torch.zeros_like(t.q), torch.zeros(w.n_q, SHAPE_1.num_q_heads, device="cuda:0")
+    plan.partial_prefill_attn(t.k_pool, t.v_pool, t.q, None, None, out, lse)
+    assert plan.status() == 0
+    score = 128 * float(t.q[0, 0, 0]) * float(k[at[dead], 0, 0]) / 128 ** 0.5
+    seen = 0
+    for j, p in enumerate(pos.tolist()):
+        if p < dead:
+            continue
+        want = v[at[dead:p + 1]].double().mean(0)           # one KV head: the same for all query heads
+        # probabilities are 2^x of one common x: each rounded to bf16 alike, outputs rounded once (2^-9)
+        assert torch.allclose(out[j].double(), want.expand(SHAPE_1.num_q_heads, -1), rtol=2 ** -7, atol=1e-4), (j, p)
+        assert torch.allclose(lse[j].double(), torch.full_like(lse[j].double(), score + np.log(p + 1 - dead)), rtol=1e-4), (j, p)
+        seen += 1
+    assert seen >= 9
+    plan.destroy()
