@@ -16,7 +16,7 @@
  *   - "host" / "device" beside a pointer says where the memory lives.  The caller owns every
  *     buffer it passes; host arrays may be freed as soon as the call returns.  The library owns
  *     only the opaque plan (its host tables, device tables and staging buffers) and at most 64 MB of
- *     device memory of destroyed plans, kept for later ones.
+ *     device memory of destroyed plans per device, kept for later ones.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Device
  *     work is enqueued on it and the call returns without waiting, unless stated otherwise.
  *   - One plan serves every layer of its batch, one call after the other.  Calls on the SAME plan

@@ -99,9 +99,9 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     put(o_workc, pl->work_chunked.data(), pl->work_chunked.size() * sizeof(AttnWork));
     put(o_comb, pl->combine.data(), pl->combine.size() * sizeof(CombineItem));
     put(o_invf, pl->inv_freq.data(), pl->inv_freq.size() * sizeof(double));
-    TS_CUDA(blob_acquire(&d.blob, off, &d.blob_bytes, st));
-    TS_CUDA(cudaMemcpyAsync(d.blob, hb, table_bytes, cudaMemcpyHostToDevice, st));
-    char *db = static_cast<char *>(d.blob);
+    TS_CUDA(blob_acquire(&d.blob, off, st));
+    TS_CUDA(cudaMemcpyAsync(d.blob.p, hb, table_bytes, cudaMemcpyHostToDevice, st));
+    char *db = static_cast<char *>(d.blob.p);
     d.g_src = reinterpret_cast<int32_t *>(db + o_src);
     d.g_dst = reinterpret_cast<int32_t *>(db + o_dst);
     d.items = reinterpret_cast<GatherItem *>(db + o_items);
@@ -205,7 +205,7 @@ int32_t tessera_plan_create(const tessera_model_cfg *cfg, const tessera_compose_
     if (!pl->host_only) {
         st = upload(pl, static_cast<cudaStream_t>(stream));
         if (st != TESSERA_OK) {
-            if (pl->dev.blob) blob_release(pl->dev.blob, pl->dev.blob_bytes, pl->device);
+            if (pl->dev.blob.p) blob_release(pl->dev.blob);
             delete pl;
             return st;
         }
@@ -224,8 +224,8 @@ int32_t tessera_plan_destroy(tessera_plan *pl) {
         if (pl->ev_out) cudaEventDestroy(pl->ev_out);
         if (pl->s_in) cudaStreamDestroy(pl->s_in);
         if (pl->s_out) cudaStreamDestroy(pl->s_out);
-        if (pl->dev.blob) {
-            cudaError_t e = blob_release(pl->dev.blob, pl->dev.blob_bytes, pl->device);
+        if (pl->dev.blob.p) {
+            cudaError_t e = blob_release(pl->dev.blob);
             if (e != cudaSuccess) rc = cuda_fail(e, "release of the plan's device memory");
         }
         void *bufs[] = {pl->dev.st_q, pl->dev.st_k, pl->dev.st_v, pl->dev.st_o, pl->dev.st_lse, pl->dev.q8};

@@ -8,47 +8,69 @@ namespace tessera {
 
 namespace {
 
-struct Block {
-    void *p;
-    size_t bytes;
-    int device;
-    unsigned long long context;   // id of the context the block belongs to: a block does not outlive a device reset
-};
+constexpr int kMaxDevices = 64;
 
 // A fixed array: nothing here allocates host memory, so nothing throws through the C entry points.
 struct Pool {
     std::mutex mutex;
-    Block blocks[kBlobPoolBlocks];     // oldest first
+    unsigned long long context = 0;    // id of the primary context the blocks belong to
+    DeviceBlob blocks[kBlobPoolBlocks];     // oldest first
     int count = 0;
     size_t held = 0;
-};
-Pool g_pool;
 
-// Id of the current context, 0 when it cannot be asked for (then nothing is pooled).
-unsigned long long context_id() {
-    using Fn = CUresult (*)(CUcontext, unsigned long long *);
-    static const Fn fn = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) p = nullptr;
-        return reinterpret_cast<Fn>(p);
-    }();
-    unsigned long long id = 0;
-    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+    DeviceBlob take(int i) {
+        const DeviceBlob b = blocks[i];
+        for (int k = i; k + 1 < count; ++k) blocks[k] = blocks[k + 1];
+        --count;
+        held -= b.bytes;
+        return b;
+    }
+    // A device has one primary context at a time: blocks of an earlier one went with the reset that ended it.
+    void enter(unsigned long long id) {
+        if (context == id) return;
+        context = id;
+        count = 0;
+        held = 0;
+    }
+};
+Pool g_pools[kMaxDevices];
+
+template <class Fn>
+Fn driver_fn(const char *name) {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) p = nullptr;
+    return reinterpret_cast<Fn>(p);
 }
 
-// Takes block i out of the pool.
-Block take(Pool &pl, int i) {
-    const Block b = pl.blocks[i];
-    for (int k = i; k + 1 < pl.count; ++k) pl.blocks[k] = pl.blocks[k + 1];
-    --pl.count;
-    pl.held -= b.bytes;
-    return b;
+// Id of a context (null: the current one; ids are never used twice in a process), 0 when there is none.
+unsigned long long context_id(CUcontext c = nullptr) {
+    static const auto get_id = driver_fn<CUresult (*)(CUcontext, unsigned long long *)>("cuCtxGetId");
+    unsigned long long id = 0;
+    return get_id && get_id(c, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// Id of the primary context of `device`, 0 when it has none (and none is made).
+unsigned long long primary_context_id(int device) {
+    static const auto get_device = driver_fn<CUresult (*)(CUdevice *, int)>("cuDeviceGet");
+    static const auto get_state = driver_fn<CUresult (*)(CUdevice, unsigned *, int *)>("cuDevicePrimaryCtxGetState");
+    static const auto retain = driver_fn<CUresult (*)(CUcontext *, CUdevice)>("cuDevicePrimaryCtxRetain");
+    static const auto release = driver_fn<CUresult (*)(CUdevice)>("cuDevicePrimaryCtxRelease");
+    CUdevice dev;
+    CUcontext primary = nullptr;
+    unsigned flags = 0;
+    int active = 0;
+    if (device < 0 || device >= kMaxDevices || !get_device || !get_state || !retain || !release) return 0;
+    if (get_device(&dev, device) != CUDA_SUCCESS || get_state(dev, &flags, &active) != CUDA_SUCCESS || !active) return 0;
+    if (retain(&primary, dev) != CUDA_SUCCESS) return 0;
+    const unsigned long long id = context_id(primary);
+    release(dev);
+    return id;
 }
 
 }  // namespace
 
-cudaError_t blob_acquire(void **p, size_t bytes, size_t *granted, cudaStream_t stream) {
+cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(stream, &capturing);
     if (e != cudaSuccess) return e;
@@ -58,66 +80,56 @@ cudaError_t blob_acquire(void **p, size_t bytes, size_t *granted, cudaStream_t s
     size_t step = 4096;
     while (step * 8 < bytes) step *= 2;
     bytes = (bytes + step - 1) / step * step;
-    const unsigned long long context = context_id();
-    Pool &pl = g_pool;
-    std::lock_guard<std::mutex> lock(pl.mutex);
-    if (capturing == cudaStreamCaptureStatusNone) {
+    unsigned long long context = primary_context_id(device);
+    if (context != context_id()) context = 0;
+    if (context != 0 && capturing == cudaStreamCaptureStatusNone) {
+        Pool &pl = g_pools[device];
+        std::lock_guard<std::mutex> lock(pl.mutex);
+        pl.enter(context);
         int best = -1;
         for (int i = 0; i < pl.count; ++i) {
-            const Block &b = pl.blocks[i];
-            if (b.device != device || b.context != context || b.bytes < bytes || b.bytes > 2 * bytes) continue;
-            if (best < 0 || b.bytes < pl.blocks[best].bytes) best = i;
+            if (pl.blocks[i].bytes < bytes || pl.blocks[i].bytes > 2 * bytes) continue;
+            if (best < 0 || pl.blocks[i].bytes < pl.blocks[best].bytes) best = i;
         }
         if (best >= 0) {
-            const Block b = take(pl, best);
-            *p = b.p;
-            *granted = b.bytes;
+            *b = pl.take(best);
             return cudaSuccess;
         }
     }
-    e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation) {
+    void *p = nullptr;
+    e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && context != 0) {
+        Pool &pl = g_pools[device];
+        std::lock_guard<std::mutex> lock(pl.mutex);
+        pl.enter(context);
         bool any = false;
-        for (int i = pl.count; i-- > 0;)
-            if (pl.blocks[i].device == device) {
-                const Block b = take(pl, i);
-                if (b.context == context) any |= cudaFree(b.p) == cudaSuccess;
-            }
+        while (pl.count > 0) any |= cudaFree(pl.take(0).p) == cudaSuccess;
         if (any) {
             cudaGetLastError();
-            e = cudaMalloc(p, bytes);
+            e = cudaMalloc(&p, bytes);
         }
     }
-    *granted = bytes;
+    if (e == cudaSuccess) *b = {p, bytes, device, context};
     return e;
 }
 
-cudaError_t blob_release(void *p, size_t bytes, int device) {
-    int current = 0;
-    cudaError_t e = cudaGetDevice(&current);
-    if (e == cudaSuccess && current != device) e = cudaSetDevice(device);
-    if (e != cudaSuccess) return e;
-    const unsigned long long context = context_id();
-    if (context == 0 || bytes > kBlobPoolBytes / 2) {
-        e = cudaFree(p);
-    } else if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
-        cudaFree(p);
-    } else {
-        Pool &pl = g_pool;
-        std::lock_guard<std::mutex> lock(pl.mutex);
-        while (pl.count == kBlobPoolBlocks || (pl.count > 0 && pl.held + bytes > kBlobPoolBytes)) {
-            const Block b = take(pl, 0);
-            if (b.device != device) cudaSetDevice(b.device);
-            if (context_id() == b.context) {
-                const cudaError_t f = cudaFree(b.p);
-                if (e == cudaSuccess) e = f;
-            }
-            if (b.device != device) cudaSetDevice(device);
-        }
-        pl.blocks[pl.count++] = {p, bytes, device, context};
-        pl.held += bytes;
+cudaError_t blob_release(const DeviceBlob &b) {
+    if (b.context != 0 && primary_context_id(b.device) != b.context) return cudaErrorContextIsDestroyed;   // freed by a reset
+    if (b.context == 0 || b.context != context_id() || b.bytes > kBlobPoolBytes / 2) return cudaFree(b.p);
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+        cudaFree(b.p);
+        return e;
     }
-    if (current != device) cudaSetDevice(current);
+    Pool &pl = g_pools[b.device];
+    std::lock_guard<std::mutex> lock(pl.mutex);
+    pl.enter(b.context);
+    while (pl.count == kBlobPoolBlocks || (pl.count > 0 && pl.held + b.bytes > kBlobPoolBytes)) {
+        const cudaError_t f = cudaFree(pl.take(0).p);
+        if (e == cudaSuccess) e = f;
+    }
+    pl.blocks[pl.count++] = b;
+    pl.held += b.bytes;
     return e;
 }
 

@@ -8,15 +8,24 @@
 
 namespace tessera {
 
-constexpr size_t kBlobPoolBytes = size_t(64) << 20;
+constexpr size_t kBlobPoolBytes = size_t(64) << 20;   // per device
 constexpr int kBlobPoolBlocks = 16;
 
-// A block of at least `bytes` on the current device (`*granted`: its size).  Refused, like cudaMalloc, while
-// `stream` is being captured.  Thread-safe.
-cudaError_t blob_acquire(void **p, size_t bytes, size_t *granted, cudaStream_t stream);
+struct DeviceBlob {
+    void *p = nullptr;
+    size_t bytes = 0;
+    int device = -1;
+    unsigned long long context = 0;    // id of the context it was allocated in; 0: never pooled
+};
 
-// Returns a block of `device` after waiting, as cudaFree does, for all work of that device.  At most kBlobPoolBytes
-// in kBlobPoolBlocks blocks stay in the pool over all devices (the oldest go first); when an allocation fails everything is given back.
-cudaError_t blob_release(void *p, size_t bytes, int device);
+// A block of at least `bytes` on the current device.  Refused, like cudaMalloc, while `stream` is being captured.
+// Thread-safe.
+cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream);
+
+// Returns a block after waiting, as cudaFree does, for all work of its device.  At most kBlobPoolBytes in
+// kBlobPoolBlocks blocks stay in a device's pool (the oldest go first); when an allocation fails all are given back.
+// Only blocks of a device's primary context are kept, and only while that context is the current one; anything else
+// is a plain cudaFree.
+cudaError_t blob_release(const DeviceBlob &b);
 
 }  // namespace tessera

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <vector_types.h>
 
+#include "blob_pool.h"
 #include "tessera.h"
 
 namespace tessera {
@@ -62,8 +63,7 @@ struct CombineItem {
 };
 
 struct DeviceTables {
-    void *blob = nullptr;          // one allocation holding everything below
-    size_t blob_bytes = 0;
+    DeviceBlob blob;               // one allocation holding everything below
     int32_t *g_src = nullptr, *g_dst = nullptr;
     GatherItem *items = nullptr;
     GatherRun *runs = nullptr;

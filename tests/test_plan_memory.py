@@ -1,0 +1,124 @@
+"""What creating and destroying plans does with device memory, on the CPU: the library's host sources linked with a
+stand-in for the CUDA runtime (fake_cuda.cpp)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2609_32999_b200 import binding as tb
+from paper_2609_32999_b200 import workloads as wl
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2609_32999_b200", "csrc")
+SHAPE = wl.ModelShape(32, 8, 128, 64, 500000.0)
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    """libtessera's host half over the stand-in, behind the binding's Plan."""
+    so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    sources = [os.path.join(CSRC, f) for f in ("api.cu", "plan.cu", "blob_pool.cu")]
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-fvisibility=hidden", "-Wl,-Bsymbolic", "-Wl,--no-undefined",
+                           "-I", os.path.join(cuda, "include"), "-I", CSRC, "-I", os.path.join(os.path.dirname(HERE), "include"),
+                           "-x", "c++", *sources, os.path.join(HERE, "fake_cuda.cpp"), "-o", so])
+    fake = ctypes.CDLL(so)
+    fake.fake_reset.argtypes = fake.fake_limit.argtypes = [ctypes.c_size_t]
+    fake.fake_count.argtypes, fake.fake_count.restype = [ctypes.c_char_p], ctypes.c_long
+    for n in ("tessera_plan_create", "tessera_plan_destroy", "tessera_plan_get_info", "tessera_plan_status", "tessera_last_error"):
+        getattr(fake, n).argtypes = getattr(tb._lib, n).argtypes
+        getattr(fake, n).restype = ctypes.c_int32
+    real, tb._lib = tb._lib, fake
+    yield fake
+    tb._lib = real
+
+
+@pytest.fixture
+def cuda(lib):
+    lib.fake_reset(4096 * MB)
+    yield lib
+
+
+def _count(lib, what):
+    return lib.fake_count(what.encode())
+
+
+def _workload(requests, tokens, tail=64, shape=SHAPE):
+    reqs = [[wl.unit(512, (r, i), recompute=()) for i in range(tokens // 512)] + [tail] for r in range(requests)]
+    return wl.build_workload("memory", shape, reqs, np.random.default_rng(0))
+
+
+def _plan(w):
+    return tb.Plan(w, stream=0)
+
+
+def test_a_block_is_used_again(cuda):
+    w = _workload(1, 5120)
+    _plan(w).destroy()
+    n = _count(cuda, "live_bytes")
+    assert 0 < n <= 64 * MB + 4 * MB
+    for _ in range(5):
+        _plan(w).destroy()
+        assert _count(cuda, "live_bytes") == n
+    assert _count(cuda, "foreign_frees") == _count(cuda, "foreign_writes") == 0
+
+
+def test_a_block_stays_with_the_context_it_came_from(cuda):
+    """Made in the primary context, destroyed while another one of the same device is current: the next plan there
+    must not write to it, and nothing of a live context is forgotten."""
+    w = _workload(1, 5120)
+    plans = [_plan(w) for _ in range(3)]
+    cuda.fake_push_other_context()
+    for p in plans:
+        p.destroy()
+    _plan(w).destroy()
+    _plan(w).destroy()
+    assert _count(cuda, "foreign_writes") == 0
+    cuda.fake_pop_context()
+    _plan(w).destroy()
+    assert _count(cuda, "foreign_writes") == _count(cuda, "foreign_frees") == 0
+    assert _count(cuda, "live_bytes") <= 64 * MB
+
+
+def test_blocks_do_not_outlive_a_device_reset(cuda):
+    w = _workload(1, 5120)
+    _plan(w).destroy()
+    old = _plan(w)
+    cuda.fake_device_reset()
+    p = _plan(w)
+    assert _count(cuda, "foreign_writes") == 0
+    with pytest.raises(tb.TesseraError):    # its memory went with the reset, and may be another plan's by now
+        old.destroy()
+    old._h = ctypes.c_void_p()
+    p.destroy()
+    _plan(w).destroy()
+    assert _count(cuda, "foreign_writes") == 0
+
+
+def test_many_sizes_stay_within_the_bound(cuda):
+    """More than sixteen blocks of different sizes: the oldest are given back."""
+    plans = [_plan(_workload(1 + i, 512 * (1 + 3 * i), tail=16)) for i in range(24)]
+    made = _count(cuda, "live_bytes")
+    for p in plans:
+        p.destroy()
+    assert _count(cuda, "live_bytes") <= 64 * MB < made + 64 * MB
+    assert _count(cuda, "live") <= 16 + 2
+    assert _count(cuda, "foreign_frees") == 0
+
+
+def test_kept_blocks_are_given_back_when_memory_runs_out(cuda):
+    small, large = _workload(1, 512), _workload(4, 33000 // 512 * 512, tail=256)
+    p = _plan(large)
+    need = _count(cuda, "live_bytes")
+    p.destroy()
+    cuda.fake_reset(4096 * MB)
+    alive = [_plan(small) for _ in range(12)]
+    for q in alive:
+        q.destroy()
+    assert _count(cuda, "live_bytes") > 0
+    cuda.fake_limit(need + MB // 8)
+    _plan(large).destroy()                 # fits only without the kept blocks
+    assert _count(cuda, "last_error") == 0
