@@ -252,8 +252,8 @@ class Plan:
 
     def destroy(self) -> None:
         if self._h:
-            _check(_lib.tessera_plan_destroy(self._h))
-            self._h = _vp()
+            h, self._h = self._h, _vp()        # the plan is gone even when its memory could not be released
+            _check(_lib.tessera_plan_destroy(h))
 
     def __del__(self):
         try:

@@ -92,7 +92,7 @@ def test_blocks_do_not_outlive_a_device_reset(cuda):
     assert _count(cuda, "foreign_writes") == 0
     with pytest.raises(tb.TesseraError):    # its memory went with the reset, and may be another plan's by now
         old.destroy()
-    old._h = ctypes.c_void_p()
+    assert not old._h                       # it is gone all the same: nothing may free it a second time
     p.destroy()
     _plan(w).destroy()
     assert _count(cuda, "foreign_writes") == 0
