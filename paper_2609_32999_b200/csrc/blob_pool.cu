@@ -9,11 +9,14 @@ namespace tessera {
 namespace {
 
 constexpr int kMaxDevices = 64;
+constexpr size_t kGuardBytes = 256;
 
 // A fixed array: nothing here allocates host memory, so nothing throws through the C entry points.
 struct Pool {
     std::mutex mutex;
     unsigned long long context = 0;    // id of the primary context the blocks belong to
+    void *anchor = nullptr;            // keeps the driver's slab of small allocations mapped: beside it a guard's cudaMalloc
+                                       // and cudaFree take 2.1 + 3.4 us, alone in its slab 700 + 570 and more
     DeviceBlob blocks[kBlobPoolBlocks];     // oldest first
     int count = 0;
     size_t held = 0;
@@ -29,6 +32,7 @@ struct Pool {
     void enter(unsigned long long id) {
         if (context == id) return;
         context = id;
+        anchor = nullptr;
         count = 0;
         held = 0;
     }
@@ -71,55 +75,69 @@ unsigned long long primary_context_id(int device) {
 }  // namespace
 
 cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream) {
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(stream, &capturing);
-    if (e != cudaSuccess) return e;
     int device = 0;
-    if ((e = cudaGetDevice(&device)) != cudaSuccess) return e;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
     // sizes in steps of an eighth: plans of about the same size fit each other's blocks
     size_t step = 4096;
     while (step * 8 < bytes) step *= 2;
     bytes = (bytes + step - 1) / step * step;
-    unsigned long long context = primary_context_id(device);
-    if (context != context_id()) context = 0;
-    if (context != 0 && capturing == cudaStreamCaptureStatusNone) {
-        Pool &pl = g_pools[device];
-        std::lock_guard<std::mutex> lock(pl.mutex);
-        pl.enter(context);
-        int best = -1;
-        for (int i = 0; i < pl.count; ++i) {
-            if (pl.blocks[i].bytes < bytes || pl.blocks[i].bytes > 2 * bytes) continue;
-            if (best < 0 || pl.blocks[i].bytes < pl.blocks[best].bytes) best = i;
+    if (context_id() == 0) cudaFree(nullptr);          // the first call of the process: makes the primary context
+    const unsigned long long context = context_id();
+    Pool &pl = g_pools[device < kMaxDevices ? device : 0];
+    std::unique_lock<std::mutex> lock(pl.mutex);
+    // (a context that was the primary one stays it while it lives: asked once per context)
+    if (context == 0 || device >= kMaxDevices || (context != pl.context && context != primary_context_id(device))) {
+        lock.unlock();
+        void *p = nullptr;
+        if ((e = cudaMalloc(&p, bytes)) == cudaSuccess) *b = {p, bytes, device, 0, nullptr};
+        return e;
+    }
+    pl.enter(context);
+    auto allocate = [&pl](void **p, size_t n) {
+        cudaError_t r = cudaMalloc(p, n);
+        while (r == cudaErrorMemoryAllocation && pl.count > 0) {
+            if (cudaFree(pl.take(0).p) != cudaSuccess) continue;
+            cudaGetLastError();
+            r = cudaMalloc(p, n);
         }
-        if (best >= 0) {
-            *b = pl.take(best);
-            return cudaSuccess;
-        }
+        return r;
+    };
+    if (!pl.anchor && (e = allocate(&pl.anchor, kGuardBytes)) != cudaSuccess) return e;
+    void *guard = nullptr;
+    if ((e = allocate(&guard, kGuardBytes)) != cudaSuccess) return e;
+    // A captured upload belongs to a graph that may run after the plan is gone: it gets memory of its own.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) {
+        cudaGetLastError();
+        capturing = cudaStreamCaptureStatusActive;
+    }
+    int best = -1;
+    for (int i = 0; i < pl.count && capturing == cudaStreamCaptureStatusNone; ++i) {
+        if (pl.blocks[i].bytes < bytes || pl.blocks[i].bytes > 2 * bytes) continue;
+        if (best < 0 || pl.blocks[i].bytes < pl.blocks[best].bytes) best = i;
     }
     void *p = nullptr;
-    e = cudaMalloc(&p, bytes);
-    if (e == cudaErrorMemoryAllocation && context != 0) {
-        Pool &pl = g_pools[device];
-        std::lock_guard<std::mutex> lock(pl.mutex);
-        pl.enter(context);
-        bool any = false;
-        while (pl.count > 0) any |= cudaFree(pl.take(0).p) == cudaSuccess;
-        if (any) {
-            cudaGetLastError();
-            e = cudaMalloc(&p, bytes);
-        }
+    if (best >= 0) {
+        *b = pl.take(best);
+    } else if ((e = allocate(&p, bytes)) == cudaSuccess) {
+        *b = {p, bytes, device, context, nullptr};
+    } else {
+        cudaFree(guard);
+        return e;
     }
-    if (e == cudaSuccess) *b = {p, bytes, device, context};
-    return e;
+    b->guard = guard;
+    return cudaSuccess;
 }
 
 cudaError_t blob_release(const DeviceBlob &b) {
-    if (b.context != 0 && primary_context_id(b.device) != b.context) return cudaErrorContextIsDestroyed;   // freed by a reset
-    if (b.context == 0 || b.context != context_id() || b.bytes > kBlobPoolBytes / 2) return cudaFree(b.p);
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) {
-        cudaFree(b.p);
-        return e;
+    if (b.context == 0) return cudaFree(b.p);
+    const bool current = context_id() == b.context;
+    if (!current && primary_context_id(b.device) != b.context) return cudaErrorContextIsDestroyed;   // freed by a reset
+    cudaError_t e = cudaFree(b.guard);                  // waits for the device
+    if (e != cudaSuccess || !current || b.bytes > kBlobPoolBytes / 2) {
+        const cudaError_t f = cudaFree(b.p);
+        return e != cudaSuccess ? e : f;
     }
     Pool &pl = g_pools[b.device];
     std::lock_guard<std::mutex> lock(pl.mutex);

@@ -16,13 +16,16 @@ struct DeviceBlob {
     size_t bytes = 0;
     int device = -1;
     unsigned long long context = 0;    // id of the context it was allocated in; 0: never pooled
+    void *guard = nullptr;             // of a block that may be pooled: a few bytes allocated and freed with every plan
 };
 
-// A block of at least `bytes` on the current device.  Refused, like cudaMalloc, while `stream` is being captured.
-// Thread-safe.
+// A block of at least `bytes` on the current device.  Refused whenever cudaMalloc is (a capture that forbids it on
+// any stream), also when a kept block would do.  Thread-safe.
 cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream);
 
-// Returns a block after waiting, as cudaFree does, for all work of its device.  At most kBlobPoolBytes in
+// Returns a block once all work of its device has ended: the guard's cudaFree waits for it, and is allowed wherever
+// the plan's own cudaFree would be (cudaDeviceSynchronize is not: it breaks every capture of the context, thread-local
+// and relaxed ones on other threads too).  At most kBlobPoolBytes in
 // kBlobPoolBlocks blocks stay in a device's pool (the oldest go first); when an allocation fails all are given back.
 // Only blocks of a device's primary context are kept, and only while that context is the current one; anything else
 // is a plain cudaFree.

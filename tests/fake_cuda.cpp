@@ -22,7 +22,7 @@ size_t g_live_bytes, g_limit;
 long g_mallocs, g_frees, g_foreign_frees, g_foreign_writes, g_writes_while_busy;
 unsigned long long g_primary, g_current;      // context ids; the primary one is current unless another was pushed
 unsigned long long g_next_id = 1;
-bool g_busy, g_capture_elsewhere, g_capture_broken;
+bool g_busy, g_forbid_malloc, g_capture_elsewhere, g_capture_broken;
 cudaError_t g_last;
 
 cudaError_t ret(cudaError_t e) { return e == cudaSuccess ? e : (g_last = e); }
@@ -44,7 +44,7 @@ __attribute__((visibility("default"))) void fake_reset(size_t limit) {
     g_live_bytes = 0;
     g_limit = limit;
     g_mallocs = g_frees = g_foreign_frees = g_foreign_writes = g_writes_while_busy = 0;
-    g_busy = g_capture_elsewhere = g_capture_broken = false;
+    g_busy = g_forbid_malloc = g_capture_elsewhere = g_capture_broken = false;
     g_last = cudaSuccess;
     g_primary = g_current = g_next_id++;
 }
@@ -64,6 +64,8 @@ __attribute__((visibility("default"))) void fake_device_reset() {
     g_primary = g_current = g_next_id++;
 }
 __attribute__((visibility("default"))) void fake_busy(int on) { g_busy = on != 0; }
+// a capture that forbids allocation calls on every thread
+__attribute__((visibility("default"))) void fake_forbid_malloc(int on) { g_forbid_malloc = on != 0; }
 // a thread-local or relaxed capture on another thread: allocation calls are allowed, waiting for the device is not
 __attribute__((visibility("default"))) void fake_capture_elsewhere(int on) { g_capture_elsewhere = on != 0; }
 __attribute__((visibility("default"))) long fake_count(const char *what) {
@@ -83,6 +85,7 @@ __attribute__((visibility("default"))) long fake_count(const char *what) {
 // ---- the runtime's side
 cudaError_t cudaMalloc(void **p, size_t n) {
     *p = nullptr;
+    if (g_forbid_malloc) return ret(cudaErrorStreamCaptureUnsupported);
     if (g_live_bytes + n > g_limit) return ret(cudaErrorMemoryAllocation);
     *p = malloc(n);
     g_live[*p] = {n, g_current};
@@ -91,6 +94,7 @@ cudaError_t cudaMalloc(void **p, size_t n) {
     return cudaSuccess;
 }
 cudaError_t cudaFree(void *p) {
+    if (!p) return cudaSuccess;
     auto it = g_live.find(p);
     if (it == g_live.end()) return ++g_foreign_frees, ret(cudaErrorInvalidValue);
     g_busy = false;               // waits for the device

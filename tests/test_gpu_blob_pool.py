@@ -70,3 +70,36 @@ def test_plans_on_several_threads():
     assert not errors
     for o in outs[1:]:
         assert torch.equal(outs[0], o)
+
+
+def test_plans_come_and_go_while_another_thread_captures():
+    """A thread-local capture stays valid while another thread destroys an idle plan, makes one, runs it and destroys it."""
+    w = wl.config(2)
+    t, t2 = wl.make_tensors(w, device="cuda:0", seed=3), wl.make_tensors(w, device="cuda:0", seed=3)
+    ref, out, out2 = (torch.zeros_like(t.q) for _ in range(3))
+    plan, idle = _layer(w, t, ref), tb.Plan(w)
+    side, errors, graph = torch.cuda.Stream(), [], torch.cuda.CUDAGraph()
+
+    def other():
+        try:
+            with torch.cuda.stream(side):
+                idle.destroy()
+                p = _layer(w, t2, out2)
+                assert p.status() == 0
+                p.destroy()
+        except Exception as e:       # noqa: BLE001
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        plan.kv_compose(t.k_pool, t.v_pool)
+        th = threading.Thread(target=other)
+        th.start()
+        th.join()
+        plan.partial_prefill_attn(t.k_pool, t.v_pool, t.q, t.k_new, t.v_new, out, None)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert torch.equal(out, ref) and torch.equal(out2, ref)
+    assert plan.status() == 0
+    plan.destroy()

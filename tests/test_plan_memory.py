@@ -105,7 +105,7 @@ def test_many_sizes_stay_within_the_bound(cuda):
     for p in plans:
         p.destroy()
     assert _count(cuda, "live_bytes") <= 64 * MB < made + 64 * MB
-    assert _count(cuda, "live") <= 16 + 2
+    assert _count(cuda, "live") <= 16 + 1
     assert _count(cuda, "foreign_frees") == 0
 
 
@@ -122,3 +122,36 @@ def test_kept_blocks_are_given_back_when_memory_runs_out(cuda):
     cuda.fake_limit(need + MB // 8)
     _plan(large).destroy()                 # fits only without the kept blocks
     assert _count(cuda, "last_error") == 0
+
+
+def test_destroying_a_plan_leaves_captures_of_other_threads_alone(cuda):
+    """A thread-local or relaxed capture forbids waiting for the device, on any thread; freeing memory it allows."""
+    w = _workload(1, 5120)
+    plans = [_plan(w) for _ in range(2)]
+    cuda.fake_capture_elsewhere(1)
+    for p in plans:
+        p.destroy()
+    _plan(w).destroy()
+    assert not _count(cuda, "capture_broken") and _count(cuda, "last_error") == 0
+
+
+def test_a_block_is_used_again_only_when_the_device_is_idle(cuda):
+    w = _workload(1, 5120)
+    for _ in range(4):
+        p = _plan(w)
+        cuda.fake_busy(1)                  # the plan's kernels are still queued
+        p.destroy()
+    _plan(w).destroy()
+    assert _count(cuda, "writes_while_busy") == 0
+
+
+def test_a_refused_allocation_refuses_the_plan_also_beside_kept_blocks(cuda):
+    w = _workload(1, 5120)
+    _plan(w).destroy()
+    cuda.fake_forbid_malloc(1)             # what a global capture does
+    with pytest.raises(tb.TesseraError):
+        _plan(w)
+    cuda.fake_forbid_malloc(0)
+    n = _count(cuda, "live_bytes")
+    _plan(w).destroy()
+    assert _count(cuda, "live_bytes") == n and _count(cuda, "foreign_frees") == 0
