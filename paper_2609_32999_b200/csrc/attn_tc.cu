@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 
 #include "device_mem.cuh"
 #include "launch.h"
@@ -698,7 +699,9 @@ attn_combine_kernel(const CombineItem *__restrict__ items, const float *__restri
     grid_release();
     if (row0 >= it.n_tok * g) return;
     constexpr int kBatch = 4;          // one batch holds all parts as a rule
-    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+    // The running maximum starts at the lowest finite value: a part whose scores are all -inf (overflowed products;
+    // every row sees the key at position 0, so not for want of keys) then has weight 2^-inf = 0, not 2^(-inf + inf).
+    float m[2] = {-FLT_MAX, -FLT_MAX}, l[2] = {0.f, 0.f};
     float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
     for (int p0 = 0; p0 < it.n_parts; p0 += kBatch) {
         float2 ml[2][kBatch];
@@ -718,16 +721,13 @@ attn_combine_kernel(const CombineItem *__restrict__ items, const float *__restri
             float mb = m[i];
 #pragma unroll
             for (int p = 0; p < kBatch; ++p) mb = fmaxf(mb, ml[i][p].x);
-            // A row whose scores so far are all -inf (overflowed products; every row sees the key at position 0, so not
-            // for want of keys) has m = -inf, sum 0: the reference stays at 0, as in the attention kernel.
-            const float ref = mb == -INFINITY ? 0.f : mb;
-            const float w0 = exp2f(m[i] - ref);
+            const float w0 = exp2f(m[i] - mb);
             m[i] = mb;
             l[i] *= w0;
             acc[i].x *= w0; acc[i].y *= w0; acc[i].z *= w0; acc[i].w *= w0;
 #pragma unroll
             for (int p = 0; p < kBatch; ++p) {
-                const float w = exp2f(ml[i][p].x - ref);
+                const float w = exp2f(ml[i][p].x - mb);
                 l[i] += ml[i][p].y * w;
                 acc[i].x = fmaf(o[i][p].x, w, acc[i].x); acc[i].y = fmaf(o[i][p].y, w, acc[i].y);
                 acc[i].z = fmaf(o[i][p].z, w, acc[i].z); acc[i].w = fmaf(o[i][p].w, w, acc[i].w);
