@@ -15,7 +15,7 @@
  *     of the calling thread's last failure.  Nothing throws, aborts or traps.
  *   - "host" / "device" beside a pointer says where the memory lives.  The caller owns every
  *     buffer it passes; host arrays may be freed as soon as the call returns.  The library owns
- *     only the opaque plan (its host tables, device tables and staging buffers) and at most 64 MB of
+ *     only the opaque plan (its host tables, device tables and staging buffers) and at most 192 MB of
  *     device memory of destroyed plans per device, kept for later ones.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Device
  *     work is enqueued on it and the call returns without waiting, unless stated otherwise.
@@ -148,7 +148,10 @@ typedef struct tessera_plan_info {
  * Validates the batch, hands request r the next ceil(T_r/page_size) ids of free_pages, derives the
  * per-position source slot, the copy list, the table of shift amounts (cos/sin evaluated in fp64,
  * stored fp32) and the attention work list, and uploads them on `stream`.  The plan depends on the
- * layout only, so one plan serves every layer of the batch.
+ * layout only, so one plan serves every layer of the batch.  Beside its tables a plan holds the
+ * workspace of split key ranges: 66 560 bytes (head_dim 64: 33 792) for each of at most 16 slots per
+ * multiprocessor, 158 MB on a B200 for batches of one to four attention items per multiprocessor and
+ * long keys, nothing for larger batches.  Where that much is not to be had, nothing is split.
  *   num_pool_pages: pages in each pool tensor.   flags: 0 or TESSERA_PLAN_HOST_ONLY.
  * Returns the plan in *out; errors: every code above except DEVICE_TIMEOUT.
  */

@@ -57,7 +57,8 @@ size_t place(size_t &off, size_t n) {
     return o;
 }
 
-int32_t upload(tessera_plan *pl, cudaStream_t st) {
+// `no_memory`: set when the device has no room for the tables and the split-KV workspace.
+int32_t upload(tessera_plan *pl, cudaStream_t st, bool *no_memory) {
     using namespace tessera;
     DeviceTables &d = pl->dev;
     TS_CUDA(cudaGetDevice(&pl->device));
@@ -99,7 +100,9 @@ int32_t upload(tessera_plan *pl, cudaStream_t st) {
     put(o_workc, pl->work_chunked.data(), pl->work_chunked.size() * sizeof(AttnWork));
     put(o_comb, pl->combine.data(), pl->combine.size() * sizeof(CombineItem));
     put(o_invf, pl->inv_freq.data(), pl->inv_freq.size() * sizeof(double));
-    TS_CUDA(blob_acquire(&d.blob, off, st));
+    const cudaError_t e = blob_acquire(&d.blob, off, st);
+    *no_memory = e == cudaErrorMemoryAllocation;
+    if (e != cudaSuccess) return cuda_fail(e, "allocation of the plan's device memory");
     TS_CUDA(cudaMemcpyAsync(d.blob.p, hb, table_bytes, cudaMemcpyHostToDevice, st));
     char *db = static_cast<char *>(d.blob.p);
     d.g_src = reinterpret_cast<int32_t *>(db + o_src);
@@ -181,37 +184,40 @@ int32_t tessera_plan_create(const tessera_model_cfg *cfg, const tessera_compose_
     if (!out) return set_error(TESSERA_INVALID_ARG, "null out pointer");
     *out = nullptr;
     if (flags & ~uint32_t(TESSERA_PLAN_HOST_ONLY)) return set_error(TESSERA_INVALID_ARG, "unknown plan flag");
-    tessera_plan *pl = new (std::nothrow) tessera_plan();
-    if (!pl) return set_error(TESSERA_INVALID_ARG, "out of host memory");
     std::string err;
     int32_t st = TESSERA_INVALID_ARG;
     int num_sms = kDefaultSMs;               // a host-only plan touches no device and is sized for a B200
-    if (!(flags & TESSERA_PLAN_HOST_ONLY)) {
-        if (int32_t rc = device_sm_count(&num_sms)) {
-            delete pl;
-            return rc;
+    const bool host_only = (flags & TESSERA_PLAN_HOST_ONLY) != 0;
+    if (!host_only)
+        if (int32_t rc = device_sm_count(&num_sms)) return rc;
+    // Without room for the workspace of a cut list on the device the plan is made again with nothing cut.
+    for (const bool cut : {true, false}) {
+        tessera_plan *pl = new (std::nothrow) tessera_plan();
+        if (!pl) return set_error(TESSERA_INVALID_ARG, "out of host memory");
+        try {
+            st = build_plan_host(cfg, desc, num_pool_pages, num_sms, cut, pl, &err);
+        } catch (const std::bad_alloc &) {
+            st = TESSERA_INVALID_ARG;
+            err = "out of host memory while building the plan";
         }
-    }
-    try {
-        st = build_plan_host(cfg, desc, num_pool_pages, num_sms, pl, &err);
-    } catch (const std::bad_alloc &) {
-        err = "out of host memory while building the plan";
-    }
-    if (st != TESSERA_OK) {
-        delete pl;
-        return set_error(st, err);
-    }
-    pl->host_only = (flags & TESSERA_PLAN_HOST_ONLY) != 0;
-    if (!pl->host_only) {
-        st = upload(pl, static_cast<cudaStream_t>(stream));
         if (st != TESSERA_OK) {
-            if (pl->dev.blob.p) blob_release(pl->dev.blob);
             delete pl;
-            return st;
+            return set_error(st, err);
         }
+        pl->host_only = host_only;
+        bool no_memory = false;
+        if (!host_only) st = upload(pl, static_cast<cudaStream_t>(stream), &no_memory);
+        if (st == TESSERA_OK) {
+            *out = pl;
+            break;
+        }
+        const bool again = cut && no_memory && pl->n_slots > 0;
+        if (pl->dev.blob.p) blob_release(pl->dev.blob);
+        delete pl;
+        if (!again) break;
+        cudaGetLastError();
     }
-    *out = pl;
-    return TESSERA_OK;
+    return st;
 }
 
 int32_t tessera_plan_destroy(tessera_plan *pl) {

@@ -135,7 +135,7 @@ cudaError_t blob_release(const DeviceBlob &b) {
     const bool current = context_id() == b.context;
     if (!current && primary_context_id(b.device) != b.context) return cudaErrorContextIsDestroyed;   // freed by a reset
     cudaError_t e = cudaFree(b.guard);                  // waits for the device
-    if (e != cudaSuccess || !current || b.bytes > kBlobPoolBytes / 2) {
+    if (e != cudaSuccess || !current || b.bytes > kBlobPoolBytes) {
         const cudaError_t f = cudaFree(b.p);
         return e != cudaSuccess ? e : f;
     }

