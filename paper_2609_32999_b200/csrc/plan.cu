@@ -6,8 +6,8 @@
 #include <cstdio>
 #include <functional>
 #include <numeric>
+#include <queue>
 #include <tuple>
-#include <unordered_map>
 
 #include <vector_types.h>
 
@@ -261,52 +261,68 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
     // Requests may use the same cached unit (equal source pages, offset and length).  The items of its users
     // are emitted side by side, so that blocks running together read the same rows out of L2 (and the
     // host-tier reader fetches a row once for all of them): 81 550 cached rows, 47 846 distinct, 106 -> 91 us.
-    struct UnitUse { int32_t req, unit; };
-    std::vector<std::vector<UnitUse>> shared;              // users of each distinct unit, in order of first use
+    // (Flat lists and hash chains: a vector per distinct unit and a multimap made plans of many units up to 40 % longer.)
+    struct Use { int32_t req, unit, next; };           // users of a distinct unit, in order
+    struct Distinct { int32_t first, last, n, next; }; // next: of the same hash
+    std::vector<Use> uses;
+    std::vector<Distinct> distinct;                    // in order of first use
+    uses.reserve(n_units);
+    distinct.reserve(n_units);
     {
-        std::unordered_multimap<int64_t, int32_t> by_page;   // first source page -> index into `shared`
-        by_page.reserve(n_units);
+        size_t slots = 16;
+        while (slots < 2 * (size_t)n_units) slots *= 2;
+        std::vector<int32_t> head(slots, -1);
+        auto src_off = [&](int u) { return d->unit_src_offset ? d->unit_src_offset[u] : 0; };
         for (int r = 0; r < batch; ++r)
             for (int u = d->unit_off[r]; u < d->unit_off[r + 1]; ++u) {
                 const int p0 = d->unit_page_off[u], np = d->unit_page_off[u + 1] - p0;
                 if (np <= 0) continue;
-                int found = -1;
-                auto range = by_page.equal_range(d->unit_pages[p0]);
-                for (auto it = range.first; it != range.second && found < 0; ++it) {
-                    const int v = shared[it->second][0].unit;
-                    const bool same_off = !d->unit_src_offset || d->unit_src_offset[u] == d->unit_src_offset[v];
-                    if (d->unit_len[u] == d->unit_len[v] && same_off && d->unit_page_off[v + 1] - d->unit_page_off[v] == np &&
-                        std::equal(d->unit_pages + p0, d->unit_pages + p0 + np, d->unit_pages + d->unit_page_off[v]))
-                        found = it->second;
+                const uint64_t key = (((uint64_t)(uint32_t)d->unit_pages[p0] << 32) | (uint32_t)d->unit_len[u]) * 128 + (uint32_t)src_off(u);
+                int32_t &chain = head[((key * 0x9E3779B97F4A7C15ull) >> 32) & (slots - 1)];
+                int32_t k = chain;
+                for (; k >= 0; k = distinct[k].next) {
+                    const int v = uses[distinct[k].first].unit, v0 = d->unit_page_off[v];
+                    if (d->unit_len[u] == d->unit_len[v] && src_off(u) == src_off(v) && d->unit_page_off[v + 1] - v0 == np &&
+                        std::equal(d->unit_pages + p0, d->unit_pages + p0 + np, d->unit_pages + v0))
+                        break;
                 }
-                if (found < 0) {
-                    found = (int)shared.size();
-                    shared.emplace_back();
-                    by_page.emplace(d->unit_pages[p0], found);
+                const int32_t use = (int32_t)uses.size();
+                uses.push_back({r, u, -1});
+                if (k < 0) {
+                    distinct.push_back({use, use, 1, chain});
+                    chain = (int32_t)distinct.size() - 1;
+                } else {
+                    uses[distinct[k].last].next = use;
+                    distinct[k].last = use;
+                    ++distinct[k].n;
                 }
-                shared[found].push_back({r, u});
                 pl->cached_tokens += d->unit_len[u];
             }
     }
     std::vector<int32_t> req_run_off(batch + 1, -1);       // first run whose first user is the request (or a later one)
     pl->runs.clear();
-    for (const auto &users : shared) {
-        if (req_run_off[users[0].req] < 0) req_run_off[users[0].req] = (int32_t)pl->runs.size();
-        const int len = d->unit_len[users[0].unit];
+    pl->g_src.resize((size_t)pl->cached_tokens);
+    pl->g_dst.resize((size_t)pl->cached_tokens);
+    int page_shift = 0;
+    while ((1 << page_shift) < B) ++page_shift;
+    int32_t listed = 0;
+    for (const Distinct &unit : distinct) {
+        const int32_t first_req = uses[unit.first].req;
+        if (req_run_off[first_req] < 0) req_run_off[first_req] = (int32_t)pl->runs.size();
+        const int len = d->unit_len[uses[unit.first].unit];
         for (int i0 = 0; i0 < len; i0 += item_tokens) {
             const int cnt = std::min(item_tokens, len - i0);
-            pl->runs.push_back({(int32_t)pl->items.size(), (int32_t)users.size(), (int32_t)pl->g_src.size(), cnt});
-            for (const UnitUse &use : users) {
-                const int u = use.unit, tp = d->unit_target_pos[u];
+            pl->runs.push_back({(int32_t)pl->items.size(), unit.n, listed, cnt});
+            for (int32_t k = unit.first; k >= 0; k = uses[k].next) {
+                const int u = uses[k].unit, r = uses[k].req, tp = d->unit_target_pos[u];
                 const int64_t d0 = (int64_t)tp - d->unit_cached_pos[u];
                 const int step = (d->unit_target_stride ? d->unit_target_stride[u] : 1) - d->unit_cached_stride[u];
-                const int32_t row0 = row_of(d0);       // step +-1: consecutive integers are consecutive rows
-                pl->items.push_back({(int32_t)pl->g_src.size(), cnt, row0 + i0 * step, step});
-                for (int i = i0; i < i0 + cnt; ++i) {
-                    const int p = tp + i;
-                    pl->g_src.push_back(pl->src_slot[pl->tok_off[use.req] + p]);
-                    pl->g_dst.push_back(pl->pages[pl->page_off[use.req] + p / B] * B + p % B);
-                }
+                pl->items.push_back({listed, cnt, row_of(d0) + i0 * step, step});   // step +-1: consecutive integers are consecutive rows
+                const int32_t *src = pl->src_slot.data() + pl->tok_off[r] + tp + i0;
+                std::copy(src, src + cnt, pl->g_src.data() + listed);
+                const int32_t *table = pl->pages.data() + pl->page_off[r];
+                for (int i = 0, p = tp + i0; i < cnt; ++i, ++p) pl->g_dst[listed + i] = (table[p >> page_shift] << page_shift) + (p & (B - 1));
+                listed += cnt;
             }
         }
     }
@@ -379,44 +395,59 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             for (auto &pr : pairs) n += parts_of(long_steps(pr), limit);
             return n * Hkv;
         };
-        // time of the list cut at `limit`: longest-first assignment to the least-loaded SM, plus the merge
-        auto modelled = [&](int limit) -> int64_t {
-            std::vector<int64_t> cost;
-            int64_t slots = 0;
+        // Time of the list cut at `limit`: longest-first assignment to the least-loaded SM, plus the merge.  Returns at
+        // once - with no more than that time - where even a perfectly even assignment reaches `enough`.
+        std::vector<int64_t> part_cost, load;
+        auto modelled = [&](int limit, int64_t enough) -> int64_t {
+            part_cost.clear();          // of the parts of one head; every head has the same
+            int64_t slots = 0, sum = 0, top = 0;
             for (auto &pr : pairs) {
                 const int sl = long_steps(pr), sa = pr.second >= 0 ? steps_of(pr.first) : 0, parts = parts_of(sl, limit);
                 const int len = (sl + parts - 1) / parts;
                 for (int b0 = 0; b0 < sl; b0 += len) {
                     const int n_b = std::min(sl, b0 + len) - b0, n_a = std::max(0, std::min(sa, b0 + len) - b0);
-                    cost.insert(cost.end(), Hkv, model_cycles(n_a, n_b, n_a > 0 ? 2 : 1));
+                    part_cost.push_back(model_cycles(n_a, n_b, n_a > 0 ? 2 : 1));
+                    sum += part_cost.back() * Hkv;
+                    top = std::max(top, part_cost.back());
                     if (parts > 1) slots += (n_a > 0 ? 2 : 1) * Hkv;
                 }
             }
-            std::sort(cost.begin(), cost.end(), std::greater<int64_t>());
-            std::vector<int64_t> load(num_sms, 0);      // a heap, least-loaded SM first
+            const bool one_round = (int64_t)part_cost.size() * Hkv <= num_sms;
+            const int64_t merge = slots ? (one_round ? kMergeCyclesOneRound : kMergeCycles) + slots * kMergeCyclesPerSlot : 0;
+            if (one_round) return top + merge;
+            const int64_t even = std::max(top, sum / num_sms) + merge;
+            if (even >= enough) return even;
+            std::sort(part_cost.begin(), part_cost.end(), std::greater<int64_t>());
+            load.assign(num_sms, 0);                    // a heap, least-loaded SM first
             int64_t end = 0;
-            for (int64_t c : cost) {
-                std::pop_heap(load.begin(), load.end(), std::greater<int64_t>());
-                end = std::max(end, load.back() += c);
-                std::push_heap(load.begin(), load.end(), std::greater<int64_t>());
-            }
-            const int64_t merge = cost.size() <= (size_t)num_sms ? kMergeCyclesOneRound : kMergeCycles;
-            return end + (slots ? merge + slots * kMergeCyclesPerSlot : 0);
+            for (int64_t c : part_cost)
+                for (int h = 0; h < Hkv; ++h) {
+                    const int64_t l = load[0] + c;
+                    end = std::max(end, l);
+                    size_t i = 0;
+                    for (size_t k = 1; k < load.size(); i = k, k = 2 * i + 1) {
+                        if (k + 1 < load.size() && load[k + 1] < load[k]) ++k;
+                        if (load[k] >= l) break;
+                        load[i] = load[k];
+                    }
+                    load[i] = l;
+                }
+            return end + merge;
         };
         int limit = longest;
         const int64_t uncut = may_cut ? (int64_t)pairs.size() * Hkv : 0;
         if (uncut > 0 && 2 * uncut <= num_sms) {
             int l = longest;
             while (l > kSplitMinSteps && items_at(l - 1) <= num_sms) --l;
-            if (modelled(l) < modelled(longest) * 90 / 100) limit = l;
+            if (modelled(l, INT64_MAX) < modelled(longest, INT64_MAX) * 90 / 100) limit = l;
         } else if (uncut > 0 && uncut <= (int64_t)kSplitMaxRounds * num_sms) {
             int64_t all = 0;
             for (auto &pr : pairs)
                 all += Hkv * model_cycles(pr.second >= 0 ? steps_of(pr.first) : 0, long_steps(pr), pr.second >= 0 ? 2 : 1);
-            int64_t best = modelled(longest) * 90 / 100;
+            int64_t best = modelled(longest, INT64_MAX) * 90 / 100;
             if (best > all / num_sms)           // otherwise no cut can reach it
                 for (int l = longest * 3 / 4; l >= 2 * kSplitMinSteps && items_at(l) <= 2 * kSplitMaxRounds * num_sms; l = l * 5 / 6) {
-                    const int64_t m = modelled(l);
+                    const int64_t m = modelled(l, best);
                     if (m < best) best = m, limit = l;
                 }
         }
@@ -540,15 +571,20 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         auto lpt_layout = [&](std::vector<AttnWork> &list) {
             const int G = num_sms;
             if ((int)list.size() <= G || (int)list.size() > kLptMaxItemsPerBlock * G) return;
+            std::vector<int64_t> cycles(list.size());
+            for (size_t i = 0; i < list.size(); ++i) cycles[i] = cycles_of(list[i]);
             std::vector<int> order(list.size());
             std::iota(order.begin(), order.end(), 0);
-            std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cycles_of(list[a]) > cycles_of(list[b]); });
-            std::vector<int64_t> load(G, 0);
+            std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cycles[a] > cycles[b]; });
+            using Block = std::pair<int64_t, int>;         // (load, block): the lowest block of the least load comes first
+            std::priority_queue<Block, std::vector<Block>, std::greater<Block>> blocks;
+            for (int b = 0; b < G; ++b) blocks.push({0, b});
             std::vector<std::vector<int>> mine(G);
             for (int i : order) {
-                const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-                load[b] += cycles_of(list[i]);
-                mine[b].push_back(i);
+                const Block least = blocks.top();
+                blocks.pop();
+                blocks.push({least.first + cycles[i], least.second});
+                mine[least.second].push_back(i);
             }
             size_t rounds = 0;
             for (auto &m : mine) rounds = std::max(rounds, m.size());
