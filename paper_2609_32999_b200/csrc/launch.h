@@ -35,6 +35,7 @@ cudaError_t launch_clusters(void (*kernel)(P...), unsigned grid, unsigned block,
     }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     if (e == cudaSuccess) count_launch();
+    else cudaGetLastError();          // returned here, not left for a later call's own check
     return e;
 }
 template <class... P, class... A>
