@@ -143,19 +143,23 @@ int32_t attention(const tessera_plan *pl, void *k_pool, void *v_pool, const void
     return TESSERA_OK;
 }
 
-// Streams and events of the host-buffer entry point, created once per plan.
+// Streams and events of the host-buffer entry point, created once per plan (a call that failed half way is made up for
+// by the next).
 int32_t ensure_pipeline(tessera_plan *pl) {
-    if (pl->s_in) return TESSERA_OK;
     const size_t n = pl->chunk_row_off.size() - 1;
-    TS_CUDA(cudaStreamCreateWithFlags(&pl->s_in, cudaStreamNonBlocking));
-    TS_CUDA(cudaStreamCreateWithFlags(&pl->s_out, cudaStreamNonBlocking));
-    TS_CUDA(cudaEventCreateWithFlags(&pl->ev_start, cudaEventDisableTiming));
-    TS_CUDA(cudaEventCreateWithFlags(&pl->ev_out, cudaEventDisableTiming));
-    pl->ev_in.assign(n, nullptr);
-    pl->ev_comp.assign(n, nullptr);
+    try {
+        pl->ev_in.resize(n, nullptr);
+        pl->ev_comp.resize(n, nullptr);
+    } catch (const std::bad_alloc &) {
+        return set_error(TESSERA_INVALID_ARG, "out of host memory");
+    }
+    if (!pl->s_in) TS_CUDA(cudaStreamCreateWithFlags(&pl->s_in, cudaStreamNonBlocking));
+    if (!pl->s_out) TS_CUDA(cudaStreamCreateWithFlags(&pl->s_out, cudaStreamNonBlocking));
+    if (!pl->ev_start) TS_CUDA(cudaEventCreateWithFlags(&pl->ev_start, cudaEventDisableTiming));
+    if (!pl->ev_out) TS_CUDA(cudaEventCreateWithFlags(&pl->ev_out, cudaEventDisableTiming));
     for (size_t c = 0; c < n; ++c) {
-        TS_CUDA(cudaEventCreateWithFlags(&pl->ev_in[c], cudaEventDisableTiming));
-        TS_CUDA(cudaEventCreateWithFlags(&pl->ev_comp[c], cudaEventDisableTiming));
+        if (!pl->ev_in[c]) TS_CUDA(cudaEventCreateWithFlags(&pl->ev_in[c], cudaEventDisableTiming));
+        if (!pl->ev_comp[c]) TS_CUDA(cudaEventCreateWithFlags(&pl->ev_comp[c], cudaEventDisableTiming));
     }
     return TESSERA_OK;
 }
@@ -194,19 +198,15 @@ int32_t tessera_plan_create(const tessera_model_cfg *cfg, const tessera_compose_
     for (const bool cut : {true, false}) {
         tessera_plan *pl = new (std::nothrow) tessera_plan();
         if (!pl) return set_error(TESSERA_INVALID_ARG, "out of host memory");
+        bool no_memory = false;
         try {
             st = build_plan_host(cfg, desc, num_pool_pages, num_sms, cut, pl, &err);
+            if (st != TESSERA_OK) set_error(st, err);
+            pl->host_only = host_only;
+            if (st == TESSERA_OK && !host_only) st = upload(pl, static_cast<cudaStream_t>(stream), &no_memory);
         } catch (const std::bad_alloc &) {
-            st = TESSERA_INVALID_ARG;
-            err = "out of host memory while building the plan";
+            st = set_error(TESSERA_INVALID_ARG, "out of host memory while building the plan");
         }
-        if (st != TESSERA_OK) {
-            delete pl;
-            return set_error(st, err);
-        }
-        pl->host_only = host_only;
-        bool no_memory = false;
-        if (!host_only) st = upload(pl, static_cast<cudaStream_t>(stream), &no_memory);
         if (st == TESSERA_OK) {
             *out = pl;
             break;

@@ -1,9 +1,11 @@
 // A host-memory stand-in for the CUDA calls that creating and destroying a plan makes, so that what they do with
 // device memory is tested without a device: two contexts, an out-of-memory limit, work in flight, captures.
 // Linked with the library's host sources; the launches are never reached.
+#include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
 
 #include <cuda.h>
@@ -33,11 +35,24 @@ CUresult retain(CUcontext *c, CUdevice) { return *c = reinterpret_cast<CUcontext
 CUresult release(CUdevice) { return CUDA_SUCCESS; }
 CUresult get_device(CUdevice *d, int i) { return *d = i, CUDA_SUCCESS; }
 
+size_t g_host_limit = SIZE_MAX;
+
 }  // namespace
+
+// of the library's sources alone (hidden): one allocation of more than the limit fails
+void *operator new(size_t n) {
+    void *p = n > g_host_limit ? nullptr : malloc(n);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void *operator new(size_t n, const std::nothrow_t &) noexcept { return n > g_host_limit ? nullptr : malloc(n); }
+void operator delete(void *p) noexcept { free(p); }
+void operator delete(void *p, size_t) noexcept { free(p); }
 
 extern "C" {
 
 // ---- the test's side
+__attribute__((visibility("default"))) void fake_host_limit(size_t limit) { g_host_limit = limit; }
 __attribute__((visibility("default"))) void fake_reset(size_t limit) {
     for (auto &b : g_live) free(b.first);
     g_live.clear();

@@ -26,7 +26,7 @@ def lib(tmp_path_factory):
                            "-I", os.path.join(cuda, "include"), "-I", CSRC, "-I", os.path.join(os.path.dirname(HERE), "include"),
                            "-x", "c++", *sources, os.path.join(HERE, "fake_cuda.cpp"), "-o", so])
     fake = ctypes.CDLL(so)
-    fake.fake_reset.argtypes = fake.fake_limit.argtypes = [ctypes.c_size_t]
+    fake.fake_reset.argtypes = fake.fake_limit.argtypes = fake.fake_host_limit.argtypes = [ctypes.c_size_t]
     fake.fake_count.argtypes, fake.fake_count.restype = [ctypes.c_char_p], ctypes.c_long
     for n in ("tessera_plan_create", "tessera_plan_destroy", "tessera_plan_get_info", "tessera_plan_status", "tessera_last_error"):
         getattr(fake, n).argtypes = getattr(tb._lib, n).argtypes
@@ -186,3 +186,23 @@ def test_nothing_is_cut_where_the_workspace_does_not_fit(cuda):
     with pytest.raises(tb.TesseraError) as e:
         _plan(w)
     assert e.value.status == tb.CUDA_ERROR
+
+
+def test_host_memory_running_out_is_an_error(cuda):
+    """Whichever of the plan's host allocations fails - the image of the device tables is the largest - nothing throws
+    through the C call, and the device keeps nothing of the plan."""
+    w = _workload(2, 5120)
+    _plan(w).destroy()
+    live = _count(cuda, "live_bytes")
+    refused = 0
+    for limit in np.geomspace(64, 4 * MB, 120).astype(int).tolist():
+        cuda.fake_host_limit(limit)
+        try:
+            _plan(w).destroy()
+        except tb.TesseraError as e:
+            refused += 1
+            assert e.status == tb.INVALID_ARG
+        finally:
+            cuda.fake_host_limit(ctypes.c_size_t(-1).value)
+    assert 10 < refused < 120
+    assert _count(cuda, "live_bytes") == live
