@@ -429,13 +429,13 @@ int32_t tessera_composed_prefill_host(tessera_plan *pl, void *k_pool, void *v_po
     const size_t q_bytes = (size_t)pl->n_q * pl->cfg.num_q_heads * pl->cfg.head_dim * 2;
     const size_t kv_bytes = (size_t)pl->n_q * pl->cfg.num_kv_heads * pl->cfg.head_dim * 2;
     const size_t lse_bytes = (size_t)pl->n_q * pl->cfg.num_q_heads * sizeof(float);
-    if (!d.st_q && pl->n_q > 0) {
-        TS_CUDA(cudaMalloc(&d.st_q, q_bytes));
-        TS_CUDA(cudaMalloc(&d.st_k, kv_bytes));
-        TS_CUDA(cudaMalloc(&d.st_v, kv_bytes));
-        TS_CUDA(cudaMalloc(&d.st_o, q_bytes));
-        TS_CUDA(cudaMalloc(reinterpret_cast<void **>(&d.st_lse), lse_bytes));
+    if (!d.st_lse && pl->n_q > 0) {             // st_lse comes last: a call that failed half way is made up for by the next
+        if (!d.st_q) TS_CUDA(cudaMalloc(&d.st_q, q_bytes));
+        if (!d.st_k) TS_CUDA(cudaMalloc(&d.st_k, kv_bytes));
+        if (!d.st_v) TS_CUDA(cudaMalloc(&d.st_v, kv_bytes));
+        if (!d.st_o) TS_CUDA(cudaMalloc(&d.st_o, q_bytes));
         TS_CUDA(cudaMemsetAsync(d.st_q, 0, q_bytes, st));   // rows of later chunks are read (and discarded) as tile padding
+        TS_CUDA(cudaMalloc(reinterpret_cast<void **>(&d.st_lse), lse_bytes));
     }
     if (pl->n_q == 0) {
         TS_CUDA(launch_gather(pl, k_pool, v_pool, k_pool, v_pool, GatherMode::kCopyRotate, st));

@@ -1,6 +1,6 @@
 // A host-memory stand-in for the CUDA calls that creating and destroying a plan makes, so that what they do with
 // device memory is tested without a device: two contexts, an out-of-memory limit, work in flight, captures.
-// Linked with the library's host sources; the launches are never reached.
+// Linked with the library's host sources; launches do nothing.
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
@@ -21,12 +21,14 @@ struct Block {
 };
 std::map<void *, Block> g_live;
 size_t g_live_bytes, g_limit;
-long g_mallocs, g_frees, g_foreign_frees, g_foreign_writes, g_writes_while_busy;
+long g_calls_left = -1, g_mallocs, g_frees, g_foreign_frees, g_foreign_writes, g_writes_while_busy;
 unsigned long long g_primary, g_current;      // context ids; the primary one is current unless another was pushed
 unsigned long long g_next_id = 1;
 bool g_busy, g_forbid_malloc, g_capture_elsewhere, g_capture_broken;
 cudaError_t g_last;
 
+// counts down the calls that make something; the one that reaches zero fails
+bool fails() { return g_calls_left > 0 && --g_calls_left == 0; }
 cudaError_t ret(cudaError_t e) { return e == cudaSuccess ? e : (g_last = e); }
 
 CUresult get_id(CUcontext c, unsigned long long *id) { return *id = c ? reinterpret_cast<unsigned long long>(c) : g_current, CUDA_SUCCESS; }
@@ -52,6 +54,7 @@ void operator delete(void *p, size_t) noexcept { free(p); }
 extern "C" {
 
 // ---- the test's side
+__attribute__((visibility("default"))) void fake_fail_call(long k) { g_calls_left = k; }
 __attribute__((visibility("default"))) void fake_host_limit(size_t limit) { g_host_limit = limit; }
 __attribute__((visibility("default"))) void fake_reset(size_t limit) {
     for (auto &b : g_live) free(b.first);
@@ -101,7 +104,7 @@ __attribute__((visibility("default"))) long fake_count(const char *what) {
 cudaError_t cudaMalloc(void **p, size_t n) {
     *p = nullptr;
     if (g_forbid_malloc) return ret(cudaErrorStreamCaptureUnsupported);
-    if (g_live_bytes + n > g_limit) return ret(cudaErrorMemoryAllocation);
+    if (fails() || g_live_bytes + n > g_limit) return ret(cudaErrorMemoryAllocation);
     *p = malloc(n);
     g_live[*p] = {n, g_current};
     g_live_bytes += n;
@@ -119,7 +122,8 @@ cudaError_t cudaFree(void *p) {
     ++g_frees;
     return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+    if (kind == cudaMemcpyDeviceToHost) return cudaSuccess;
     auto it = g_live.upper_bound(dst);
     if (it == g_live.begin()) return ++g_foreign_writes, cudaSuccess;
     --it;
@@ -128,7 +132,7 @@ cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t n, cudaMemcpyKind
     memcpy(dst, src, n);
     return cudaSuccess;
 }
-cudaError_t cudaMemsetAsync(void *, int, size_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *p, int, size_t, cudaStream_t) { return g_foreign_writes += g_live.count(p) == 0, cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() {
     if (g_capture_elsewhere) return g_capture_broken = true, ret(cudaErrorStreamCaptureUnsupported);
     g_busy = false;
@@ -157,22 +161,22 @@ cudaError_t cudaGetDriverEntryPoint(const char *name, void **fn, unsigned long l
     *q = *fn ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
     return cudaSuccess;
 }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *, unsigned) { abort(); }
-cudaError_t cudaStreamDestroy(cudaStream_t) { abort(); }
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { abort(); }
-cudaError_t cudaEventCreateWithFlags(cudaEvent_t *, unsigned) { abort(); }
-cudaError_t cudaEventDestroy(cudaEvent_t) { abort(); }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { abort(); }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return fails() ? ret(cudaErrorUnknown) : (*s = reinterpret_cast<cudaStream_t>(new char), cudaSuccess); }
+cudaError_t cudaStreamDestroy(cudaStream_t s) { return delete reinterpret_cast<char *>(s), cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t e, unsigned) { return e ? cudaSuccess : ret(cudaErrorInvalidResourceHandle); }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return fails() ? ret(cudaErrorUnknown) : (*e = reinterpret_cast<cudaEvent_t>(new char), cudaSuccess); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { return delete reinterpret_cast<char *>(e), cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { return e ? cudaSuccess : ret(cudaErrorInvalidResourceHandle); }
 
 }  // extern "C"
 
 namespace tessera {
-cudaError_t launch_gather(const tessera_plan *, const void *, const void *, void *, void *, GatherMode, cudaStream_t) { abort(); }
+cudaError_t launch_gather(const tessera_plan *, const void *, const void *, void *, void *, GatherMode, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_kv_fp8(const tessera_plan *, const void *, const void *, void *, void *, bool, bool, float, float, cudaStream_t) { abort(); }
-cudaError_t launch_scatter_fresh(const tessera_plan *, void *, void *, const void *, const void *, int, cudaStream_t) { abort(); }
+cudaError_t launch_scatter_fresh(const tessera_plan *, void *, void *, const void *, const void *, int, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_rope_fresh(const tessera_plan *, void *, void *, cudaStream_t) { abort(); }
 cudaError_t launch_extend_write(const tessera_plan *, void *, void *, void *, const void *, const void *, void *, void *, cudaStream_t) { abort(); }
-cudaError_t launch_attn_tc(const tessera_plan *, void *, void *, const void *, void *, float *, int, int, cudaStream_t, std::string *) { abort(); }
+cudaError_t launch_attn_tc(const tessera_plan *, void *, void *, const void *, void *, float *, int, int, cudaStream_t, std::string *) { return cudaSuccess; }
 cudaError_t launch_attn_tc_k8(const tessera_plan *, void *, void *, const void *, void *, float *, float, cudaStream_t, std::string *) { abort(); }
 cudaError_t launch_compose_k8(const tessera_plan *, const void *, const void *, void *, void *, bool, float, cudaStream_t) { abort(); }
 cudaError_t launch_fresh_k8(const tessera_plan *, const void *, void *, float, void *, void *, const void *, const void *, float, cudaStream_t) { abort(); }

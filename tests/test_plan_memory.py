@@ -27,8 +27,10 @@ def lib(tmp_path_factory):
                            "-x", "c++", *sources, os.path.join(HERE, "fake_cuda.cpp"), "-o", so])
     fake = ctypes.CDLL(so)
     fake.fake_reset.argtypes = fake.fake_limit.argtypes = fake.fake_host_limit.argtypes = [ctypes.c_size_t]
+    fake.fake_fail_call.argtypes = [ctypes.c_long]
     fake.fake_count.argtypes, fake.fake_count.restype = [ctypes.c_char_p], ctypes.c_long
-    for n in ("tessera_plan_create", "tessera_plan_destroy", "tessera_plan_get_info", "tessera_plan_status", "tessera_last_error"):
+    for n in ("tessera_plan_create", "tessera_plan_destroy", "tessera_plan_get_info", "tessera_plan_status", "tessera_last_error",
+              "tessera_composed_prefill_host"):
         getattr(fake, n).argtypes = getattr(tb._lib, n).argtypes
         getattr(fake, n).restype = ctypes.c_int32
     real, tb._lib = tb._lib, fake
@@ -206,3 +208,28 @@ def test_host_memory_running_out_is_an_error(cuda):
             cuda.fake_host_limit(ctypes.c_size_t(-1).value)
     assert 10 < refused < 120
     assert _count(cuda, "live_bytes") == live
+
+
+def test_a_host_call_that_failed_half_way_is_made_up_for_by_the_next(cuda):
+    """Its streams, events and staging buffers are made by the first call; whichever of them fails, that call is
+    refused and the next one finds or makes all of them."""
+    w = _workload(3, 1024)
+    buf = np.zeros(1 << 24, np.uint8)
+    pool = (buf.ctypes.data + 255) // 256 * 256
+    ptr = type("T", (), {"data_ptr": lambda self: pool})()
+    for k in range(1, 40):
+        p = _plan(w)
+        cuda.fake_fail_call(k)
+        try:
+            p.composed_prefill_host(*[ptr] * 7, stream=0)
+            done = True
+        except tb.TesseraError as e:
+            assert e.status == tb.CUDA_ERROR
+            done = False
+        cuda.fake_fail_call(-1)
+        p.composed_prefill_host(*[ptr] * 7, stream=0)
+        p.destroy()
+        assert _count(cuda, "foreign_writes") == 0
+        if done:
+            break
+    assert 10 < k < 39                     # five buffers, two streams, two events and two for each chunk
