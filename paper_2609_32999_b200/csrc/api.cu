@@ -230,15 +230,10 @@ int32_t tessera_plan_destroy(tessera_plan *pl) {
         if (pl->ev_out) cudaEventDestroy(pl->ev_out);
         if (pl->s_in) cudaStreamDestroy(pl->s_in);
         if (pl->s_out) cudaStreamDestroy(pl->s_out);
-        if (pl->dev.blob.p) {
-            cudaError_t e = blob_release(pl->dev.blob);
-            if (e != cudaSuccess) rc = cuda_fail(e, "release of the plan's device memory");
-        }
-        void *bufs[] = {pl->dev.st_q, pl->dev.st_k, pl->dev.st_v, pl->dev.st_o, pl->dev.st_lse, pl->dev.q8};
-        for (void *b : bufs)
-            if (b) {
-                cudaError_t e = cudaFree(b);
-                if (e != cudaSuccess) rc = cuda_fail(e, "cudaFree");
+        for (const DeviceBlob &b : {pl->dev.blob, pl->dev.q8, pl->dev.staging})
+            if (b.p) {
+                cudaError_t e = blob_release(b);
+                if (e != cudaSuccess) rc = cuda_fail(e, "release of the plan's device memory");
             }
     }
     delete pl;
@@ -405,11 +400,11 @@ int32_t tessera_partial_prefill_attn_k8(tessera_plan *pl, void *k_pool8, float k
     if (pl->n_q == 0) return TESSERA_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t q_elems = pl->n_q * pl->cfg.num_q_heads * pl->cfg.head_dim;
-    if (!pl->dev.q8) TS_CUDA(cudaMalloc(&pl->dev.q8, (size_t)q_elems));
+    if (!pl->dev.q8.p) TS_CUDA(blob_acquire(&pl->dev.q8, (size_t)q_elems, st));
     // the reciprocals are taken once, in fp32: every element is multiplied by it and rounded to e4m3
-    TS_CUDA(launch_fresh_k8(pl, q, pl->dev.q8, 1.0f / q_scale, k_pool8, v_pool, k_new, v_new, 1.0f / k_scale, st));
+    TS_CUDA(launch_fresh_k8(pl, q, pl->dev.q8.p, 1.0f / q_scale, k_pool8, v_pool, k_new, v_new, 1.0f / k_scale, st));
     std::string err;
-    cudaError_t e = launch_attn_tc_k8(pl, k_pool8, v_pool, pl->dev.q8, out, lse, q_scale * k_scale, st, &err);
+    cudaError_t e = launch_attn_tc_k8(pl, k_pool8, v_pool, pl->dev.q8.p, out, lse, q_scale * k_scale, st, &err);
     if (e != cudaSuccess) return set_error(TESSERA_CUDA_ERROR, "tcgen05 attention launch (8-bit keys): " + err + " / " + cudaGetErrorString(e));
     return TESSERA_OK;
 }
@@ -429,13 +424,18 @@ int32_t tessera_composed_prefill_host(tessera_plan *pl, void *k_pool, void *v_po
     const size_t q_bytes = (size_t)pl->n_q * pl->cfg.num_q_heads * pl->cfg.head_dim * 2;
     const size_t kv_bytes = (size_t)pl->n_q * pl->cfg.num_kv_heads * pl->cfg.head_dim * 2;
     const size_t lse_bytes = (size_t)pl->n_q * pl->cfg.num_q_heads * sizeof(float);
-    if (!d.st_lse && pl->n_q > 0) {             // st_lse comes last: a call that failed half way is made up for by the next
-        if (!d.st_q) TS_CUDA(cudaMalloc(&d.st_q, q_bytes));
-        if (!d.st_k) TS_CUDA(cudaMalloc(&d.st_k, kv_bytes));
-        if (!d.st_v) TS_CUDA(cudaMalloc(&d.st_v, kv_bytes));
-        if (!d.st_o) TS_CUDA(cudaMalloc(&d.st_o, q_bytes));
-        TS_CUDA(cudaMemsetAsync(d.st_q, 0, q_bytes, st));   // rows of later chunks are read (and discarded) as tile padding
-        TS_CUDA(cudaMalloc(reinterpret_cast<void **>(&d.st_lse), lse_bytes));
+    if (!d.st_q && pl->n_q > 0) {
+        size_t off = 0;
+        const size_t o_q = place<char>(off, q_bytes), o_k = place<char>(off, kv_bytes), o_v = place<char>(off, kv_bytes);
+        const size_t o_o = place<char>(off, q_bytes), o_lse = place<char>(off, lse_bytes);
+        if (!d.staging.p) TS_CUDA(blob_acquire(&d.staging, off, st));
+        char *base = static_cast<char *>(d.staging.p);
+        TS_CUDA(cudaMemsetAsync(base + o_q, 0, q_bytes, st));   // rows of later chunks are read (and discarded) as tile padding
+        d.st_q = base + o_q;
+        d.st_k = base + o_k;
+        d.st_v = base + o_v;
+        d.st_o = base + o_o;
+        d.st_lse = reinterpret_cast<float *>(base + o_lse);
     }
     if (pl->n_q == 0) {
         TS_CUDA(launch_gather(pl, k_pool, v_pool, k_pool, v_pool, GatherMode::kCopyRotate, st));

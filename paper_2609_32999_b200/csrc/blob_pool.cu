@@ -83,7 +83,13 @@ cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream) {
     while (step * 8 < bytes) step *= 2;
     bytes = (bytes + step - 1) / step * step;
     if (context_id() == 0) cudaFree(nullptr);          // the first call of the process: makes the primary context
-    const unsigned long long context = context_id();
+    // A captured copy belongs to a graph that may run after the plan is gone: it gets memory that is never pooled.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) {
+        cudaGetLastError();
+        capturing = cudaStreamCaptureStatusActive;
+    }
+    const unsigned long long context = capturing == cudaStreamCaptureStatusNone ? context_id() : 0;
     Pool &pl = g_pools[device < kMaxDevices ? device : 0];
     std::unique_lock<std::mutex> lock(pl.mutex);
     // (a context that was the primary one stays it while it lives: asked once per context)
@@ -106,14 +112,8 @@ cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream) {
     if (!pl.anchor && (e = allocate(&pl.anchor, kGuardBytes)) != cudaSuccess) return e;
     void *guard = nullptr;
     if ((e = allocate(&guard, kGuardBytes)) != cudaSuccess) return e;
-    // A captured upload belongs to a graph that may run after the plan is gone: it gets memory of its own.
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) {
-        cudaGetLastError();
-        capturing = cudaStreamCaptureStatusActive;
-    }
     int best = -1;
-    for (int i = 0; i < pl.count && capturing == cudaStreamCaptureStatusNone; ++i) {
+    for (int i = 0; i < pl.count; ++i) {
         if (pl.blocks[i].bytes < bytes || pl.blocks[i].bytes > 2 * bytes) continue;
         if (best < 0 || pl.blocks[i].bytes < pl.blocks[best].bytes) best = i;
     }

@@ -1,6 +1,7 @@
 // Device memory of plans.  A plan is created and destroyed per batch, and cudaMalloc / cudaFree of its tables and
 // split-KV workspace (0.3 MB and 11 MB for one 5 312-token request) cost several times what building the plan
-// costs, so blocks of destroyed plans are kept for the next ones.
+// costs, so blocks of destroyed plans are kept for the next ones.  So do the 8-bit copy of q and the staging buffers,
+// which a plan's first call asks for.
 #pragma once
 #include <cstddef>
 
@@ -23,7 +24,7 @@ struct DeviceBlob {
 };
 
 // A block of at least `bytes` on the current device.  Refused whenever cudaMalloc is (a capture that forbids it on
-// any stream), also when a kept block would do.  Thread-safe.
+// any stream), also when a kept block would do; not pooled when `stream` itself is being captured.  Thread-safe.
 cudaError_t blob_acquire(DeviceBlob *b, size_t bytes, cudaStream_t stream);
 
 // Returns a block once all work of its device has ended: the guard's cudaFree waits for it, and is allowed wherever

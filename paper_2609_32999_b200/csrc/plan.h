@@ -81,8 +81,8 @@ struct DeviceTables {
     float2 *ws_ml = nullptr;           // ... and [slot][128] (reference maximum in log2 units, sum)
     int32_t *status = nullptr;     // device status word(s)
     double *inv_freq = nullptr;    // [D/2] rotary frequencies
-    // staging for the host-buffer entry point (allocated on first use)
-    void *q8 = nullptr;            // 8-bit copy of q for the 8-bit-key attention entry (allocated on first use)
+    DeviceBlob q8;                 // 8-bit copy of q for the 8-bit-key attention entry (allocated on first use)
+    DeviceBlob staging;            // of the host-buffer entry point (allocated on first use), holding:
     void *st_q = nullptr, *st_k = nullptr, *st_v = nullptr, *st_o = nullptr;
     float *st_lse = nullptr;
 };

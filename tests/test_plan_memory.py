@@ -232,4 +232,20 @@ def test_a_host_call_that_failed_half_way_is_made_up_for_by_the_next(cuda):
         assert _count(cuda, "foreign_writes") == 0
         if done:
             break
-    assert 10 < k < 39                     # five buffers, two streams, two events and two for each chunk
+    assert 10 < k < 39                     # the buffers, two streams, two events and two for each chunk
+
+
+def test_staging_buffers_are_kept_for_the_next_plan(cuda):
+    """A first call through host buffers allocates its guard and nothing else once a plan like it has come and gone."""
+    w = _workload(3, 1024)
+    buf = np.zeros(1 << 24, np.uint8)
+    pool = (buf.ctypes.data + 255) // 256 * 256
+    ptr = type("T", (), {"data_ptr": lambda self: pool})()
+    mallocs = []
+    for _ in range(4):
+        p = _plan(w)
+        n = _count(cuda, "mallocs")
+        p.composed_prefill_host(*[ptr] * 7, stream=0)
+        mallocs.append(_count(cuda, "mallocs") - n)
+        p.destroy()
+    assert mallocs == [2, 1, 1, 1] and _count(cuda, "foreign_writes") == 0
