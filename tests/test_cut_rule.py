@@ -52,8 +52,8 @@ def _modelled(pairs, heads, limit):
     return max(load) + ((4500 if len(cost) <= SMS else 9000) + slots * 20 if slots else 0)
 
 
-def _items(w):
-    pairs, heads = _pairs(w), w.shape.num_kv_heads
+def _limit(pairs, heads):
+    """Most steps a part may have; the longest tile's where nothing is cut."""
     count = lambda limit: heads * sum(_parts(b, limit) for _, b in pairs)          # noqa: E731
     longest = max([b for _, b in pairs], default=1)
     limit, uncut = longest, len(pairs) * heads
@@ -71,7 +71,24 @@ def _items(w):
             if m < best:
                 best, limit = m, low
             low = low * 5 // 6
-    return heads * sum(len(_lengths(b, limit)) for _, b in pairs), limit < longest
+    return limit
+
+
+def items_and_cut(w):
+    pairs, heads = _pairs(w), w.shape.num_kv_heads
+    limit = _limit(pairs, heads)
+    return heads * sum(len(_lengths(b, limit)) for _, b in pairs), limit < max([b for _, b in pairs], default=1)
+
+
+def is_chained(w):
+    """Whether the plan's kernels are launched with programmatic serialization: its attention is modelled short."""
+    pairs, heads = _pairs(w), w.shape.num_kv_heads
+    limit, total = _limit(pairs, heads), 0
+    for a, b in pairs:
+        for lo, hi in _lengths(b, limit):
+            n_a = max(0, min(a or 0, hi) - lo)
+            total += _cycles(n_a, hi - lo, 2 if n_a else 1) * heads
+    return total // SMS <= 300000
 
 
 @pytest.mark.parametrize("seed", range(6))
@@ -86,7 +103,7 @@ def test_the_planner_cuts_as_the_rule_says(seed):
                 for r in range(max(1, int(2 ** rng.uniform(0, 4.6))))]
         w = wl.build_workload("cut", shape, reqs, np.random.default_rng(i))
         plan = tb.Plan(w, host_only=True)
-        want, was_cut = _items(w)
+        want, was_cut = items_and_cut(w)
         assert plan.info.n_attn_items == want, (i, len(reqs), units, heads, group)
         cut += was_cut
     assert 3 <= cut <= 17                  # both sides of the rule

@@ -23,7 +23,8 @@ def test_results_and_memory_over_many_plans():
     ws = [wl.config(1), wl.config(2), wl.config(3, requests_override=2)]
     ts = [wl.make_tensors(w, device="cuda:0", seed=i) for i, w in enumerate(ws)]
     ref = [torch.zeros_like(t.q) for t in ts]
-    keep = [_layer(w, t, o) for w, t, o in zip(ws, ts, ref)]
+    # five of each alive at once: as much memory as the loop below ever holds
+    keep = [_layer(w, t, o) for w, t, o in zip(ws, ts, ref) for _ in range(5)]
     torch.cuda.synchronize()
     for p in keep:
         p.destroy()
@@ -31,7 +32,7 @@ def test_results_and_memory_over_many_plans():
     rng = np.random.default_rng(0)
     out = [torch.zeros_like(t.q) for t in ts]
     alive = []
-    for _ in range(60):
+    for _ in range(150):
         i = int(rng.integers(3))
         out[i].zero_()
         alive.append(_layer(ws[i], ts[i], out[i]))
@@ -41,13 +42,18 @@ def test_results_and_memory_over_many_plans():
         assert torch.equal(out[i], ref[i])
     for p in alive:
         p.destroy()
-    assert free0 - torch.cuda.mem_get_info()[0] <= 128 << 20
+    # nothing grows from plan to plan (the driver maps small allocations 2 MB at a time)
+    assert free0 - torch.cuda.mem_get_info()[0] <= 8 << 20
 
 
 def test_plans_on_several_threads():
     w = wl.config(2)
     ts = [wl.make_tensors(w, device="cuda:0", seed=9) for _ in range(4)]
     outs = [torch.zeros_like(t.q) for t in ts]
+    ref = torch.zeros_like(ts[0].q)
+    alone = _layer(w, wl.make_tensors(w, device="cuda:0", seed=9), ref)
+    torch.cuda.synchronize()
+    alone.destroy()
     errors = []
 
     def work(k):
@@ -68,8 +74,8 @@ def test_plans_on_several_threads():
         th.join()
     torch.cuda.synchronize()
     assert not errors
-    for o in outs[1:]:
-        assert torch.equal(outs[0], o)
+    for o in outs:
+        assert torch.equal(ref, o)
 
 
 def test_plans_come_and_go_while_another_thread_captures():

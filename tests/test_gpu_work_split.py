@@ -8,6 +8,7 @@ import torch
 from paper_2609_32999_b200 import binding as tb
 from paper_2609_32999_b200 import workloads as wl
 from tests import gpu_util as gu
+from tests.test_cut_rule import items_and_cut
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +37,25 @@ def test_parity_where_the_work_list_changes(shape, requests, unit, units, tail, 
     asm, _, _ = gu.check_assembled(g)
     gu.check_untouched(g)
     gu.check_attention(g, asm)
+
+
+@pytest.mark.parametrize("requests,units,tail,uncut,items", [
+    (20, 6, 60, 160, 640),                        # one to two rounds, cut
+    (38, 8, 20, 304, 912),                        # two to four rounds, cut
+    (57, 8, 4, 456, 456),                         # three to four rounds, left alone
+    (75, 3, 20, 600, 600),                        # more than four rounds: never cut
+])
+def test_parity_of_lists_of_several_rounds(requests, units, tail, uncut, items):
+    shape = wl.ModelShape(8, 8, 64, 64, 500000.0)
+    rng = np.random.default_rng(11)
+    reqs = [[3] + [wl.unit(1024, (r % 4, i), recompute=()) for i in range(units)] + [tail] for r in range(requests)]
+    w = wl.build_workload("rounds", shape, reqs, rng)
+    assert items_and_cut(w) == (items, items > uncut) and tb.Plan(w, host_only=True).info.n_attn_items == items
+    g = gu.run_layer(w, seed=7)
+    assert g.status == 0
+    checked = [0, requests // 2, requests - 1]
+    asm, _, _ = gu.check_assembled(g, requests=checked)
+    gu.check_attention(g, asm, {r: gu.sample_rows(w, r, rng, 0, 8) for r in checked})
 
 
 @pytest.mark.parametrize("masked_steps", [2, 9, 20])
