@@ -143,10 +143,10 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
             const int chunk = (w / CPH) * (D / 8) + c;
             const size_t so = (size_t)s_src[tok[u]] * row_chunks + chunk;
             dso[u] = (size_t)s_dst[tok[u]] * row_chunks + chunk;
-            rk[u][0] = ldg_stream(ks + so);
-            rk[u][1] = ldg_stream(ks + so + HALF);
-            rv[u][0] = ldg_stream(vs + so);
-            rv[u][1] = ldg_stream(vs + so + HALF);
+            rk[u][0] = ldg_pieces(ks + so);
+            rk[u][1] = ldg_pieces(ks + so + HALF);
+            rv[u][0] = ldg_pieces(vs + so);
+            rv[u][1] = ldg_pieces(vs + so + HALF);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -216,10 +216,10 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
                 if (t >= n_tasks) continue;
                 const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
                 const size_t so = (size_t)g_src[rn.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
-                rk[u][0] = ldg_stream(k_src + so);
-                rk[u][1] = ldg_stream(k_src + so + HALF);
-                rv[u][0] = ldg_stream(v_src + so);
-                rv[u][1] = ldg_stream(v_src + so + HALF);
+                rk[u][0] = ldg_pieces(k_src + so);
+                rk[u][1] = ldg_pieces(k_src + so + HALF);
+                rv[u][0] = ldg_pieces(v_src + so);
+                rv[u][1] = ldg_pieces(v_src + so + HALF);
             }
             for (int m = 0; m < rn.n_items; ++m) {
                 const GatherItem it = items[rn.first_item + m];
