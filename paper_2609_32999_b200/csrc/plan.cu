@@ -370,19 +370,15 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         };
         // Split-KV: the key ranges of a batch that leaves SMs idle are cut into parts of at most `limit` steps
         // that run as separate items and are merged afterwards.
-        //   items <= SMs / 2 : the smallest limit whose parts still fit one round (one item per SM).  A common
-        //                      limit, not a common part count: short tiles are not cut as often as long ones
-        //                      (5 312 tokens, 48 items: parts of at most 14 steps before, 9 now; attention
-        //                      39.4 -> 35.7 us; 5 requests of 2 048 tokens, 2 KV heads of 64: the whole layer
-        //                      41.0 -> 28.6 us), unless the merge eats what that gains (448 tokens, 56 items of
-        //                      four steps: 54.2 us in the host-tier path, cut in 80 58.0).
-        //   items <= kSplitMaxRounds x SMs : the limit with the least modelled time, if that is at least 10 %
-        //                      below the uncut list's (168 items of 260 steps take two rounds on 148 SMs; cut in
-        //                      parts they fill all rounds).  Attention of n requests of two tiles each, 12 288
-        //                      keys: 80 items 185 -> 141 us, 96 items 195 -> 153, 152 items 368 -> 282 (in 760 parts;
-        //                      in at most 592, 296); 4 096 keys:
-        //                      left alone, a cut gains nothing (152 items 126-140 us, cut in 456 130-146).  128 items of
-        //                      77 to 224 steps: layer 570 -> 502 us.
+        //   items <= SMs / 2 : the smallest limit whose parts still fit one round (one item per SM), if the model gives
+        //                      it 10 %.  A common limit, not a common part count, so that short tiles are not cut as
+        //                      often as long ones: 48 items of 42 steps in parts of 9 in place of 14, attention
+        //                      39.4 -> 35.7 us.  56 items of four steps stay whole (cut in 80 parts a host-tier
+        //                      layer takes 58.0 us, whole 54.2).
+        //   items <= kSplitMaxRounds x SMs : the limit of the least modelled time, if that is 10 % below the uncut
+        //                      list's.  Attention of n requests of two tiles over 12 288 keys: 80 items 185 -> 141 us,
+        //                      152 items (two rounds on 148 SMs, the second nearly empty) 368 -> 282; over 4 096 keys
+        //                      152 items stay whole (126-140 us, cut in 456 130-146).
         //   more             : never; the rounds are even enough and the merge only costs.
         auto parts_of = [&](int steps, int limit) {
             return std::max(1, std::min({(steps + limit - 1) / limit, kSplitMaxParts, steps / kSplitMinSteps}));
@@ -489,11 +485,9 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             w.seq_len = pl->seq_len[req];
             w.page_begin = pl->page_off[req];
         }
-        // Launch latency is a visible part of a layer while the attention takes tens of microseconds: 2 items
-        // 20.6 -> 19.1 us a layer, 144 items of 9 steps 51.5 -> 51.2 (62.3 -> 56.2 before the lists were cut by modelled
-        // time), 240 items of up to 8 steps 53.0 -> 48.3, 1 680 short items 121.1 -> 114.6.  Layers whose attention runs
-        // for hundreds of microseconds, near the power limit, lose: 1 024 items (219 us modelled) 436 -> 444 us, 1 152
-        // items (1 870 us) 2 715 -> 2 742, 20 696 items 12.35 -> 12.6 ms.
+        // Launch latency is a visible part of a layer while the attention takes tens of microseconds: 240 items of up to 8
+        // steps 53.0 -> 48.3 us a layer, 1 680 short items 121.1 -> 114.6.  Layers whose attention runs for hundreds, near
+        // the power limit, lose: 1 024 items (450 000 modelled cycles an SM) 436 -> 444 us, 1 152 items 2 715 -> 2 742.
         int64_t modelled_cycles = 0;
         for (const AttnWork &w : pl->work) modelled_cycles += cycles_of(w);
         pl->chained = modelled_cycles / num_sms <= kChainedCycles;
@@ -563,11 +557,11 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         sort_items(pl->work.begin(), pl->work.end());
         // With few items per thread block the spread of the blocks' finishing times is what costs (config 3:
         // 7 items per block, slowest block 8-10 % above the mean with the plain walk): the items are then
-        // assigned greedily to the least-loaded block by modelled cycles and laid out so that the kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1
-        // - b : b)) hands every block its own list; holes are marked tile_a = -1.  Measured: config 3 +6 %,
-        // config 4 +-0.  With many items per block (config 5: 131) the plain walk is already even and keeps
-        // neighbours in the list - the same request and head - on the GPU at the same time, which the
-        // greedy assignment does not: it measured 3 % slower there, so it is not used.
+        // assigned greedily to the least-loaded block by modelled cycles and laid out so that the kernel's serpentine
+        // walk (round k, block b -> index k G + (k odd ? G - 1 - b : b)) hands every block its own list; holes are
+        // marked tile_a = -1.  Measured: config 3 +6 %, config 4 +-0.  With many items per block (config 5: 131) the
+        // plain walk is already even and keeps neighbours in the list - the same request and head - on the GPU at the
+        // same time, which the greedy assignment does not: it measured 3 % slower there, so it is not used.
         auto lpt_layout = [&](std::vector<AttnWork> &list) {
             const int G = num_sms;
             if ((int)list.size() <= G || (int)list.size() > kLptMaxItemsPerBlock * G) return;
