@@ -25,7 +25,8 @@ __device__ __forceinline__ uint4 ldg_stream(const uint4 *p) {
 // Rows read once, but in pieces of less than a 128-byte line per instruction (8-bit codes: the two halves of a head are
 // 64 bytes each, 32 at head_dim 64): the line stays in L1 until its other pieces have been read, so that the host link
 // is asked for whole lines.  65 536 rows of codes out of pinned memory: L1::no_allocate 3.19 ms, so 2.62 (head_dim 64:
-// 2.62 and 1.35); 16-bit rows of head_dim 64 in device memory, rounded to codes: plain loads 43.4 us, so 40.4.
+// 2.62 and 1.35); 16-bit rows of head_dim 64 in device memory, rounded to codes: plain loads 43.4 us, so 40.4.  Whole
+// lines are better off without: 16-bit rows of head_dim 128 to codes 86.3 us, L1::no_allocate 85.9.
 __device__ __forceinline__ uint2 ldg_pieces(const uint2 *p) {
     uint2 v;
     asm volatile("ld.global.L1::evict_first.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");

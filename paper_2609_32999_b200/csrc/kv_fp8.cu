@@ -94,6 +94,14 @@ __device__ __forceinline__ int cs_index(int c, int i) {
     return INTERLEAVED ? (i < 4 ? 4 * c + i : 4 * c + D / 4 + (i - 4)) : c * 8 + i;
 }
 
+// A load of one 16-element task's half row: D / 16 neighbouring threads read the half of a head, T each.  Where that is
+// less than a line the line is kept until the other half has been read.
+template <int D, class T>
+__device__ __forceinline__ T ldg_row(const T *p) {
+    if constexpr (sizeof(T) * (D / 16) < 128) return ldg_pieces(p);
+    else return ldg_stream(p);
+}
+
 // One thread block per GatherItem.  TO_8BIT false: sources are e4m3 (mul = scale), destinations bf16;
 // TO_8BIT true: sources are bf16, destinations e4m3 (mul = 1 / scale, applied after the rotation); with V16
 // only the keys go 8-bit and the value rows are bit copies into a 16-bit pool (key pages for the 8-bit
@@ -143,10 +151,10 @@ kv_fp8_kernel(const void *__restrict__ k_src, const void *__restrict__ v_src, vo
             const int chunk = (w / CPH) * (D / 8) + c;
             const size_t so = (size_t)s_src[tok[u]] * row_chunks + chunk;
             dso[u] = (size_t)s_dst[tok[u]] * row_chunks + chunk;
-            rk[u][0] = ldg_pieces(ks + so);
-            rk[u][1] = ldg_pieces(ks + so + HALF);
-            rv[u][0] = ldg_pieces(vs + so);
-            rv[u][1] = ldg_pieces(vs + so + HALF);
+            rk[u][0] = ldg_row<D>(ks + so);
+            rk[u][1] = ldg_row<D>(ks + so + HALF);
+            rv[u][0] = ldg_row<D>(vs + so);
+            rv[u][1] = ldg_row<D>(vs + so + HALF);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -216,10 +224,10 @@ expand_runs_kernel(const uint2 *__restrict__ k_src, const uint2 *__restrict__ v_
                 if (t >= n_tasks) continue;
                 const int tok = t / tasks_per_row, w = t - tok * tasks_per_row;
                 const size_t so = (size_t)g_src[rn.begin + tok] * row_chunks + (w / CPH) * (D / 8) + c;
-                rk[u][0] = ldg_pieces(k_src + so);
-                rk[u][1] = ldg_pieces(k_src + so + HALF);
-                rv[u][0] = ldg_pieces(v_src + so);
-                rv[u][1] = ldg_pieces(v_src + so + HALF);
+                rk[u][0] = ldg_row<D>(k_src + so);
+                rk[u][1] = ldg_row<D>(k_src + so + HALF);
+                rv[u][0] = ldg_row<D>(v_src + so);
+                rv[u][1] = ldg_row<D>(v_src + so + HALF);
             }
             for (int m = 0; m < rn.n_items; ++m) {
                 const GatherItem it = items[rn.first_item + m];
