@@ -144,11 +144,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     const int pps = kStep / page_size;                 // pages per step: 1, 2, 4, 8 or 16
 
     // The block's share of the work list: round k of the grid takes items [k G, (k + 1) G), this block
-    // the b-th of them in even rounds and the b-th from the end in odd rounds.  For a list sorted by
-    // cost the serpentine evens out the sums, and blocks that run at the same time work on neighbours
-    // in the list, i.e. on the same request and KV head, and share their K/V pages in L2.  When a batch
-    // has few items per block the host lays the list out so that this very walk hands each block a
-    // greedily balanced share (holes are marked tile_a = -1).  Taking items off a global counter at
+    // the b-th of them in even rounds and the b-th from the end in odd rounds.  The host lays a list of more than one
+    // item per block out so that this very walk hands each block its balanced share (holes are marked tile_a = -1);
+    // a chunk's list is sorted by cost, and the serpentine evens out the sums.  Taking items off a global counter at
     // run time measured 1-1.5 % slower on the long-context configurations.  Every role walks the
     // same sequence; -1 = nothing in this round.
     const int n_rounds = (n_work + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -160,7 +158,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     auto load_item = [&](int w) {
         Item it;
         it.wk = work[w];
-        if (it.wk.tile_a < 0) {            // a hole of the assignment: nothing to do in this round
+        if (it.wk.tile_a < 0) {            // a hole of the assignment: the block's list has ended
             it.n_tiles = 0;
             return it;
         }
@@ -252,7 +250,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             const int w = item_index(round);
             if (w < 0) continue;
             const Item it = load_item(w);
-            if (it.n_tiles == 0) continue;
+            if (it.n_tiles == 0) break;
             const int kvh = it.wk.kvh;
             if (kv == 0 && lane == 0) {
                 for (int q = 0; q < it.n_tiles; ++q) {
@@ -316,7 +314,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             const int w = item_index(round);
             if (w < 0) continue;
             const Item it = load_item(w);
-            if (it.n_tiles == 0) continue;
+            if (it.n_tiles == 0) break;
             const int n_steps = it.n_steps;
             const int my_steps = q ? it.n_steps1 : it.n_steps0;
             const int T = it.T, step0 = it.step0;
@@ -448,7 +446,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         const int w = item_index(round);
         if (w < 0) continue;
         const Item it = load_item(w);
-        if (it.n_tiles == 0) continue;
+        if (it.n_tiles == 0) break;
         const int n_tiles = it.n_tiles, n_steps = it.n_steps, n_steps0 = it.n_steps0, n_steps1 = it.n_steps1;
         const int step0 = it.step0, kvh = it.wk.kvh;
         const AttnTile &t0 = it.t0, &t1 = it.t1;

@@ -555,21 +555,31 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         // together, so thread blocks that run at the same time stream the same K/V pages and find
         // them in L2.
         sort_items(pl->work.begin(), pl->work.end());
-        // With few items per thread block the spread of the blocks' finishing times is what costs (config 3:
-        // 7 items per block, slowest block 8-10 % above the mean with the plain walk): the items are then
-        // assigned greedily to the least-loaded block by modelled cycles and laid out so that the kernel's serpentine
-        // walk (round k, block b -> index k G + (k odd ? G - 1 - b : b)) hands every block its own list; holes are
-        // marked tile_a = -1.  Measured: config 3 +6 %, config 4 +-0.  With many items per block (config 5: 131) the
-        // plain walk is already even and keeps neighbours in the list - the same request and head - on the GPU at the
-        // same time, which the greedy assignment does not: it measured 3 % slower there, so it is not used.
-        auto lpt_layout = [&](std::vector<AttnWork> &list) {
+        // A list of more than one item per thread block is dealt out here, each item to the least-loaded block by modelled
+        // cycles, in two stretches.  First the long items, request by request and KV head by KV head: the blocks of the
+        // whole GPU work through the same K/V pages at about the same time and find them in L2.  Then the short ones, the
+        // last kTailItems longest items' worth of cycles per block, longest first: they even out what the first stretch
+        // left (slowest block 0.6-2 % above the mean; all items longest first: 0.5-1.5 %).  The order is worth DRAM
+        // traffic, and through the power limit time: 1 152 items of up to 259 steps (modelled 4.6 -> 2.1 GB from DRAM)
+        // attention 2 502 -> 2 405 us at 1.37 -> 1.40 GHz, 20 696 items 11 160 -> 10 790 us.
+        // The kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1 - b : b)) hands every block its own
+        // list; holes, only at the end of a block's list, are marked tile_a = -1.
+        auto deal_out = [&](std::vector<AttnWork> &list) {
             const int G = num_sms;
-            if ((int)list.size() <= G || (int)list.size() > kLptMaxItemsPerBlock * G) return;
+            if ((int)list.size() <= G) return;
             std::vector<int64_t> cycles(list.size());
             for (size_t i = 0; i < list.size(); ++i) cycles[i] = cycles_of(list[i]);
             std::vector<int> order(list.size());
             std::iota(order.begin(), order.end(), 0);
             std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cycles[a] > cycles[b]; });
+            const double tail_cycles = kTailItems * (double)cycles[order[0]] * G;
+            size_t head = order.size();
+            for (double sum = 0; head > 0 && sum < tail_cycles; --head) sum += (double)cycles[order[head - 1]];
+            const AttnTile *tl = pl->tiles.data();
+            std::stable_sort(order.begin(), order.begin() + head, [&](int a, int b) {
+                const int ra = tl[list[a].tile_a].req, rb = tl[list[b].tile_a].req;
+                return ra != rb ? ra < rb : list[a].kvh < list[b].kvh;
+            });
             using Block = std::pair<int64_t, int>;         // (load, block): the lowest block of the least load comes first
             std::priority_queue<Block, std::vector<Block>, std::greater<Block>> blocks;
             for (int b = 0; b < G; ++b) blocks.push({0, b});
@@ -591,7 +601,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             list.swap(out);
         };
         pl->n_work_items = (int32_t)pl->work.size();
-        lpt_layout(pl->work);
+        deal_out(pl->work);
     }
 
     pl->total_tokens = total;
