@@ -600,14 +600,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                 const size_t slot = q ? it.wk.slot_b : it.wk.slot_a;
                 if constexpr (kD == 128) tmem_ld_16x256b_x16(tO, o); else tmem_ld_16x256b_x8(tO, o);
                 tmem_wait_ld();
+                // (in the registers' own order, so that a warp's store is 512 contiguous bytes: row by row, 8 bytes a thread,
+                // a tile took 2 400 cycles, one for each of the 2 048 lines its 256 stores touch)
+                float4 *po = reinterpret_cast<float4 *>(ws_o) + ((slot * (kRows / 16) + lane16 / 16) * (kD / 8)) * 32 + lane;
 #pragma unroll
-                for (int rr = 0; rr < 2; ++rr) {
-                    float *po = ws_o + (slot * kRows + rows[rr]) * kD + cq;
+                for (int k = 0; k < kD / 8; ++k)
+                    po[k * 32] = make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]), __uint_as_float(o[4 * k + 2]), __uint_as_float(o[4 * k + 3]));
+                if ((lane & 3) == 0)
 #pragma unroll
-                    for (int k = 0; k < kD / 8; ++k)
-                        *reinterpret_cast<uint2 *>(po + 8 * k) = make_uint2(o[4 * k + 2 * rr], o[4 * k + 2 * rr + 1]);
-                    if ((lane & 3) == 0) ws_ml[slot * kRows + rows[rr]] = make_float2(m_row[q][rr], l_tot[rr]);
-                }
+                    for (int rr = 0; rr < 2; ++rr) ws_ml[slot * kRows + rows[rr]] = make_float2(m_row[q][rr], l_tot[rr]);
                 continue;
             }
             const float inv[2] = {__frcp_rn(l_tot[0]), __frcp_rn(l_tot[1])};
@@ -682,25 +683,32 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
 }
 
 // Merges the parts of a split-KV launch: for every row, O = sum_p O_p 2^(m_p - m) / sum_p l_p 2^(m_p - m)
-// with m = max_p m_p.  Lanes walk head_dim; a warp has two rows, and the loads of up to four parts of both in
-// flight: the kernel is a chain of L2 latencies, and with one row a warp its 1 152 blocks (144 items of 5 312
-// tokens) took two waves; 8 parts in flight of one row: layer 50.8 us, two rows with 4: 49.2.
-constexpr int kCombineBlocks = kRows / 16;     // thread blocks per (tile, KV head): 8 warps, two rows each
+// with m = max_p m_p.  The parts lie in the workspace in the order of accumulator fragments: [slot][16 rows][8 columns]
+// [lane][4], lane t holding rows t/4 and t/4 + 8, columns 2 (t%4) and + 1.  A warp merges two neighbouring groups of 8
+// columns of 16 rows, with the loads of up to four parts of both in flight: the kernel is a chain of L2 latencies.  Layer of
+// 48 items of up to 42 steps in 144 parts, workspace row by row 47.2 us, in fragment order 46.8.
+template <int kD>
+struct CombineGeo {
+    static constexpr int kPairs = kD / 16;                        // pairs of column groups
+    static constexpr int kBlocks = kRows / 16 * kPairs / 8;       // thread blocks (8 warps) per (tile, KV head)
+};
 template <int kD>
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const CombineItem *__restrict__ items, const float *__restrict__ ws_o, const float2 *__restrict__ ws_ml, __nv_bfloat16 *__restrict__ out,
                     float *__restrict__ lse, int H_q, int g) {
-    const CombineItem it = items[blockIdx.x / kCombineBlocks];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row0 = (blockIdx.x % kCombineBlocks) * 16 + warp * 2;
+    using C = CombineGeo<kD>;
+    const CombineItem it = items[blockIdx.x / C::kBlocks];
+    const int lane = threadIdx.x & 31, unit = (blockIdx.x % C::kBlocks) * 8 + (threadIdx.x >> 5);
+    const int rb = unit / C::kPairs, pair = unit % C::kPairs;
+    const int rows[2] = {rb * 16 + (lane >> 2), rb * 16 + (lane >> 2) + 8};
     grid_wait();
     grid_release();
-    if (row0 >= it.n_tok * g) return;
+    if (rb * 16 >= it.n_tok * g) return;
     constexpr int kBatch = 4;          // one batch holds all parts as a rule
     // The running maximum starts at the lowest finite value: a part whose scores are all -inf (overflowed products;
     // every row sees the key at position 0, so not for want of keys) then has weight 2^-inf = 0, not 2^(-inf + inf).
     float m[2] = {-FLT_MAX, -FLT_MAX}, l[2] = {0.f, 0.f};
-    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};     // (x, y): row 0, (z, w): row 1
     for (int p0 = 0; p0 < it.n_parts; p0 += kBatch) {
         float2 ml[2][kBatch];
         float4 o[2][kBatch];
@@ -709,40 +717,49 @@ attn_combine_kernel(const CombineItem *__restrict__ items, const float *__restri
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 // L2 loads: the workspace is rewritten by every launch
-                const size_t r = (size_t)(it.slot0 + p0 + p) * kRows + row0 + i;
+                const size_t slot = (size_t)it.slot0 + p0 + p;
                 const bool there = p0 + p < it.n_parts;
-                ml[i][p] = there ? __ldcg(ws_ml + r) : make_float2(-INFINITY, 0.f);
-                o[i][p] = there && lane * 4 < kD ? __ldcg(reinterpret_cast<const float4 *>(ws_o + r * kD + lane * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                ml[i][p] = there ? __ldcg(ws_ml + slot * kRows + rows[i]) : make_float2(-INFINITY, 0.f);
+                o[i][p] = there ? __ldcg(reinterpret_cast<const float4 *>(ws_o) + ((slot * (kRows / 16) + rb) * (kD / 8) + 2 * pair + i) * 32 + lane)
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
             }
+        float w0[2], w[2][kBatch];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            float mb = m[i];
+        for (int r = 0; r < 2; ++r) {
+            float mb = m[r];
 #pragma unroll
-            for (int p = 0; p < kBatch; ++p) mb = fmaxf(mb, ml[i][p].x);
-            const float w0 = exp2f(m[i] - mb);
-            m[i] = mb;
-            l[i] *= w0;
-            acc[i].x *= w0; acc[i].y *= w0; acc[i].z *= w0; acc[i].w *= w0;
+            for (int p = 0; p < kBatch; ++p) mb = fmaxf(mb, ml[r][p].x);
+            w0[r] = exp2f(m[r] - mb);
+            m[r] = mb;
+            l[r] *= w0[r];
 #pragma unroll
             for (int p = 0; p < kBatch; ++p) {
-                const float w = exp2f(ml[i][p].x - mb);
-                l[i] += ml[i][p].y * w;
-                acc[i].x = fmaf(o[i][p].x, w, acc[i].x); acc[i].y = fmaf(o[i][p].y, w, acc[i].y);
-                acc[i].z = fmaf(o[i][p].z, w, acc[i].z); acc[i].w = fmaf(o[i][p].w, w, acc[i].w);
+                w[r][p] = exp2f(ml[r][p].x - mb);
+                l[r] += ml[r][p].y * w[r][p];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            acc[i].x *= w0[0]; acc[i].y *= w0[0]; acc[i].z *= w0[1]; acc[i].w *= w0[1];
+#pragma unroll
+            for (int p = 0; p < kBatch; ++p) {
+                acc[i].x = fmaf(o[i][p].x, w[0][p], acc[i].x); acc[i].y = fmaf(o[i][p].y, w[0][p], acc[i].y);
+                acc[i].z = fmaf(o[i][p].z, w[1][p], acc[i].z); acc[i].w = fmaf(o[i][p].w, w[1][p], acc[i].w);
             }
         }
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int row = row0 + i;
-        if (row >= it.n_tok * g) break;
-        const float inv = 1.f / l[i];
-        const int tok = it.q_begin + row / g, head = it.kvh * g + row % g;
-        uint2 pk;
-        pk.x = pack_bf16(acc[i].x * inv, acc[i].y * inv);
-        pk.y = pack_bf16(acc[i].z * inv, acc[i].w * inv);
-        if (lane * 4 < kD) *reinterpret_cast<uint2 *>(out + ((size_t)tok * H_q + head) * kD + lane * 4) = pk;
-        if (lse && lane == 0) lse[(size_t)tok * H_q + head] = (m[i] + log2f(l[i])) * 0.6931471805599453f;
+    for (int r = 0; r < 2; ++r) {
+        const float inv = 1.f / l[r];
+        // neighbouring lanes swap: the even one ends up with 4 columns of the first group, the odd one with 4 of the second
+        const uint32_t a = r ? pack_bf16(acc[0].z * inv, acc[0].w * inv) : pack_bf16(acc[0].x * inv, acc[0].y * inv);
+        const uint32_t b = r ? pack_bf16(acc[1].z * inv, acc[1].w * inv) : pack_bf16(acc[1].x * inv, acc[1].y * inv);
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, lane & 1 ? a : b, 1);
+        if (rows[r] >= it.n_tok * g) continue;
+        const int tok = it.q_begin + rows[r] / g, head = it.kvh * g + rows[r] % g;
+        const uint2 y = lane & 1 ? make_uint2(got, b) : make_uint2(a, got);
+        *reinterpret_cast<uint2 *>(out + ((size_t)tok * H_q + head) * kD + (2 * pair + (lane & 1)) * 8 + (lane & 2) * 2) = y;
+        if (lse && pair == 0 && (lane & 3) == 0) lse[(size_t)tok * H_q + head] = (m[r] + log2f(l[r])) * 0.6931471805599453f;
     }
 }
 
@@ -784,7 +801,7 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
         const int c0 = chunk < 0 ? 0 : pl->chunk_combine_off[chunk];
         const int c1 = chunk < 0 ? (int)pl->combine.size() : pl->chunk_combine_off[chunk + 1];
         if (c1 > c0)
-            e = launch_kernel(attn_combine_kernel<D>, (unsigned)(c1 - c0) * kCombineBlocks, 256, 0, st, chained,
+            e = launch_kernel(attn_combine_kernel<D>, (unsigned)(c1 - c0) * CombineGeo<D>::kBlocks, 256, 0, st, chained,
                               d.combine + c0, d.ws_o, d.ws_ml, static_cast<__nv_bfloat16 *>(out), lse, Hq, g);
     }
     if (e != cudaSuccess) *err = "kernel launch";

@@ -58,6 +58,23 @@ def test_parity_of_lists_of_several_rounds(requests, units, tail, uncut, items):
     gu.check_attention(g, asm, {r: gu.sample_rows(w, r, rng, 0, 8) for r in checked})
 
 
+@pytest.mark.parametrize("heads,kv_heads,dim,fresh", [
+    (7, 1, 128, 1), (7, 1, 128, 2), (14, 2, 128, 5),      # 7, 14 and 35 rows: less than one group of 16, and a remainder
+    (3, 1, 64, 11), (16, 1, 64, 8), (16, 2, 128, 17),     # 33 rows; a full tile; a full tile and one row
+])
+def test_merge_of_row_groups(heads, kv_heads, dim, fresh):
+    """Cut lists whose tiles end inside a group of 16 rows, both head sizes."""
+    shape = wl.ModelShape(heads, kv_heads, dim, 32, 10000.0)
+    rng = np.random.default_rng(5)
+    w = wl.build_workload("merge", shape, [[wl.unit(1500, ("u", i), recompute=()) for i in range(2)] + [fresh]], rng)
+    assert items_and_cut(w)[1]
+    g = gu.run_layer(w, seed=17)
+    assert g.status == 0
+    asm, _, _ = gu.check_assembled(g)
+    gu.check_untouched(g)
+    gu.check_attention(g, asm)
+
+
 @pytest.mark.parametrize("masked_steps", [2, 9, 20])
 def test_parts_whose_scores_all_overflow_count_for_nothing(masked_steps):
     """Scores of -inf in whole parts of a cut key range - more parts than the merge reads at once, too - leave the
