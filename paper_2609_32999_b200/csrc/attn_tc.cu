@@ -115,6 +115,14 @@ struct Item {
     const int32_t *bt;
 };
 
+// The block's first item, as the descriptor tables have it: brought to shared memory while the launch still waits for its
+// predecessor, because the chain of loads through the tables (item, tiles or page ids) takes 1 800 cycles.
+struct FirstItem {
+    AttnWork wk;
+    AttnTile t[2];
+    int32_t page[32];          // pages of the first steps
+};
+
 // kMaxPages: most pages a 128-key step can consist of in this instantiation - 8 (pages of 16 tokens or
 // more) or 16 (pages of 8 tokens); the wider producer loop is kept out of the common instantiation.
 // K8: queries and keys are 8-bit floats (e4m3 codes; the scales are folded into scale_log2 by the host):
@@ -139,6 +147,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     __shared__ __align__(8) Barriers bars;
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort, s_skip;
+    __shared__ FirstItem s_first;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int pps = kStep / page_size;                 // pages per step: 1, 2, 4, 8 or 16
@@ -155,16 +164,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         const int w = round * (int)gridDim.x + b;
         return w < n_work ? w : -1;
     };
-    auto load_item = [&](int w) {
+    auto load_item = [&](int w, bool staged) {
         Item it;
-        it.wk = work[w];
+        it.wk = staged ? s_first.wk : work[w];
         if (it.wk.tile_a < 0) {            // a hole of the assignment: the block's list has ended
             it.n_tiles = 0;
             return it;
         }
         it.n_tiles = it.wk.tile_b >= 0 ? 2 : 1;
-        it.t0 = tiles[it.wk.tile_a];
-        it.t1 = tiles[it.n_tiles == 2 ? it.wk.tile_b : it.wk.tile_a];
+        it.t0 = staged ? s_first.t[0] : tiles[it.wk.tile_a];
+        it.t1 = staged ? s_first.t[1] : tiles[it.n_tiles == 2 ? it.wk.tile_b : it.wk.tile_a];
         // the item covers the 128-key steps [step0, step_end) of its tiles (all of them unless it was
         // split); step indices below are relative to step0
         it.step0 = it.wk.step_begin;
@@ -203,6 +212,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         prefetch_tmap(&tmap_k);
         prefetch_tmap(&tmap_v);
         prefetch_tmap(&tmap_o);
+    }
+    if (warp == 10 && (int)blockIdx.x < n_work) {
+        const Item it = load_item(blockIdx.x, false);
+        if (lane == 0) {
+            s_first.wk = it.wk;
+            s_first.t[0] = it.t0;
+            s_first.t[1] = it.t1;
+        }
+        const int pi = pps * it.step0 + lane;
+        s_first.page[lane] = pi < it.req_pages ? it.bt[pi] : num_pool_pages;
     }
     tc_fence_before();
     // Nothing above touches global memory the stream's earlier kernels write, so it runs beside their tail.
@@ -249,7 +268,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         for (int round = 0; round < n_rounds; ++round) {
             const int w = item_index(round);
             if (w < 0) continue;
-            const Item it = load_item(w);
+            const Item it = load_item(w, round == 0);
             if (it.n_tiles == 0) break;
             const int kvh = it.wk.kvh;
             if (kv == 0 && lane == 0) {
@@ -270,7 +289,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                 // lane l holds the id of page (pps * (step0 + j0) + l); a page past the request's last one
                 // is fetched from outside the pool, which TMA fills with zeros
                 const int pi = pps * (it.step0 + j0) + lane;
-                const int my_page = pi < it.req_pages ? it.bt[pi] : num_pool_pages;
+                const int my_page = round == 0 && j0 == 0 ? s_first.page[lane] : pi < it.req_pages ? it.bt[pi] : num_pool_pages;
                 const int jn = min(steps_per_fetch, it.n_steps - j0);
                 for (int jj = 0; jj < jn; ++jj) {
                     int pg[kMaxPages];
@@ -313,7 +332,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         for (int round = 0; round < n_rounds; ++round) {
             const int w = item_index(round);
             if (w < 0) continue;
-            const Item it = load_item(w);
+            const Item it = load_item(w, round == 0);
             if (it.n_tiles == 0) break;
             const int n_steps = it.n_steps;
             const int my_steps = q ? it.n_steps1 : it.n_steps0;
@@ -445,7 +464,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         for (int round = 0; round < n_rounds; ++round) {
         const int w = item_index(round);
         if (w < 0) continue;
-        const Item it = load_item(w);
+        const Item it = load_item(w, round == 0);
         if (it.n_tiles == 0) break;
         const int n_tiles = it.n_tiles, n_steps = it.n_steps, n_steps0 = it.n_steps0, n_steps1 = it.n_steps1;
         const int step0 = it.step0, kvh = it.wk.kvh;
