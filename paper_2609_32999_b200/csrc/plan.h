@@ -75,10 +75,10 @@ struct DeviceTables {
     int32_t *q_pos = nullptr;      // [n_q]
     int32_t *pages = nullptr;      // block tables
     AttnTile *tiles = nullptr;
-    AttnWork *work = nullptr;      // tcgen05 work items, longest first
-    AttnWork *work_chunked = nullptr;  // the same items grouped by request chunk (host-buffer entry)
+    AttnWork *work = nullptr;      // tcgen05 work items, dealt out to the thread blocks
+    AttnWork *work_chunked = nullptr;  // the same items grouped by request chunk, longest first (host-buffer entry)
     CombineItem *combine = nullptr;    // (tile, head) pairs to merge, grouped by request chunk
-    float *ws_o = nullptr;             // split-KV partials: [slot][128 rows][128] unnormalised O ...
+    float *ws_o = nullptr;             // split-KV partials: [slot][16 rows][8 columns][lane][4] unnormalised O ...
     float2 *ws_ml = nullptr;           // ... and [slot][128] (reference maximum in log2 units, sum)
     int32_t *status = nullptr;     // device status word(s)
     double *inv_freq = nullptr;    // [D/2] rotary frequencies
