@@ -453,6 +453,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         const int rows[2] = {lane16 + (lane >> 2), lane16 + (lane >> 2) + 8};
         const int cq = (lane & 3) * 2;                                 // first of the thread's two columns in every group of 8
         // (divisions by the group size, once: in the items they cost 1 680 short ones 2 % - 109.8 -> 107.2 us a layer)
+        const int tile_tok = kRows / g;
         const int row_tok[2] = {rows[0] / g, rows[1] / g}, row_head[2] = {rows[0] % g, rows[1] % g};
         int step_base[2] = {0, 0};                     // steps of each tile in earlier work items (barrier phases go on)
         auto quad_max = [](float v) {
@@ -634,7 +635,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                 continue;
             }
             const float inv[2] = {__frcp_rn(l_tot[0]), __frcp_rn(l_tot[1])};
-            const bool full_tile = t.n_tok == kRows / g;
+            // (head_dim 64, whose epilogues come twice as fast: the quotient is kept, 425.3 -> 418.6 us a layer of 416 items;
+            // at 128 a register kept through the step loop costs more, 2 610 -> 2 641 us a layer of 1 152)
+            const bool full_tile = t.n_tok == (kD == 64 ? tile_tok : kRows / g);
             uint8_t *stage = sm + G::kSmemStage;
             if (full_tile) {
                 // A full tile leaves through shared memory and one tiled bulk store per 64 columns: the
