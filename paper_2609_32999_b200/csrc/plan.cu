@@ -566,6 +566,17 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 sort_items(list.begin(), list.end());
                 return;
             }
+            // (a list of less than kHeadItems longest items per block has no first stretch: two requests of 33 024 tokens, 2.1
+            // of them, lost up to 2 % to the coarser balance, four, 4.3, gained 4; equal items then keep their pages' order)
+            double all = 0;
+            int64_t longest_item = 0;
+            for (const AttnWork &w : list) {
+                const int64_t c = cycles_of(w);
+                all += (double)c;
+                longest_item = std::max(longest_item, c);
+            }
+            const bool two_stretches = all >= kHeadItems * (double)longest_item * G;
+            if (!two_stretches) sort_items(list.begin(), list.end());
             // (sorted as runs of equal items - the KV heads of a tile pair - and dealt with a heap of packed (load, block)
             // values: 20 696 items item by item took 5 ms of a plan's 11)
             struct Run { int64_t cycles; int32_t first, n, req; };
@@ -583,7 +594,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             for (const Run &r : runs)
                 for (int32_t i = 0; i < r.n; ++i) order.push_back({r.cycles, r.first + i, r.req * Hkv + list[r.first + i].kvh});
             const double tail_cycles = kTailItems * (double)order[0].cycles * G;
-            size_t head = order.size();
+            size_t head = two_stretches ? order.size() : 0;
             for (double sum = 0; head > 0 && sum < tail_cycles; --head) sum += (double)order[head - 1].cycles;
             {
                 // the first stretch by request and KV head, longest first within: a counting sort

@@ -21,6 +21,7 @@ constexpr int kChainedCycles = 300000;   // modelled attention cycles per SM up 
 constexpr int kSplitMaxRounds = 4;       // batches of more attention items per SM than this are never split, and a split
                                          // list has at most twice as many parts (each with up to two workspace slots)
 constexpr int kHostChunks = 4;          // request chunks of the host-buffer entry point's copy / compute pipeline
+constexpr double kHeadItems = 2.5;       // lists of less work, in longest items per block, are dealt longest first throughout
 constexpr double kTailItems = 0.6;       // work kept back to even out the blocks, in longest items per block (0.3: up to 13 % slower, 0.9 and
                                          // 1.3: 1-4 % slower on lists of 7 to 140 items per block)
 constexpr int kAttnCostBands = 16;      // cost bands of the attention work list (longest band first)
