@@ -398,9 +398,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                     // The rows are one stretch of bytes in each half.  (Row by row with 16 lanes, 80 rows took 3 000 cycles
                     // while the step's P waited: layer of a lone 304-token request 12.46 -> 12.17 us.)
                     uint8_t *v = sm + kSmemRing + vslot * kSlotBytes;
-                    for (uint32_t o = (uint32_t)(T - (step0 + j) * kStep) * 128 + lane * 16; o < kHalfBytes; o += 512)
+                    if constexpr (K8) {                        // (with 8-bit keys the compiler's step loop loses more: 1 194 -> 1 216 us)
+                        for (int r = T - (step0 + j) * kStep; r < kStep; ++r)
+                            if (lane < 8 * G::kHalves) *reinterpret_cast<uint4 *>(v + (lane >> 3) * kHalfBytes + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
+                    } else {
+                        for (uint32_t o = (uint32_t)(T - (step0 + j) * kStep) * 128 + lane * 16; o < kHalfBytes; o += 512)
 #pragma unroll
-                        for (int hf = 0; hf < G::kHalves; ++hf) *reinterpret_cast<uint4 *>(v + hf * kHalfBytes + o) = make_uint4(0, 0, 0, 0);
+                            for (int hf = 0; hf < G::kHalves; ++hf) *reinterpret_cast<uint4 *>(v + hf * kHalfBytes + o) = make_uint4(0, 0, 0, 0);
+                    }
                     fence_proxy_async_smem();
                     __syncwarp();
                 }
