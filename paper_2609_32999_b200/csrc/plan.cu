@@ -551,12 +551,13 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         for (const CombineItem &ci : pl->combine) ++pl->chunk_combine_off[chunk_of[pl->tiles[ci.tile].req] + 1];
         for (int c = 0; c < used_chunks; ++c) pl->chunk_combine_off[c + 1] += pl->chunk_combine_off[c];
         // A list of more than one item per thread block is dealt out here, each item to the least-loaded block by modelled
-        // cycles, in two stretches.  First the long items, request by request and KV head by KV head: the blocks of the
-        // whole GPU work through the same K/V pages at about the same time and find them in L2.  Then the short ones, the
-        // last kTailItems longest items' worth of cycles per block, longest first: they even out what the first stretch
-        // left (slowest block 0.6-2 % above the mean; all items longest first: 0.5-1.5 %).  The order is worth DRAM
-        // traffic, and through the power limit time: 1 152 items of up to 259 steps (modelled 4.6 -> 2.1 GB from DRAM)
-        // attention 2 502 -> 2 405 us at 1.37 -> 1.40 GHz, 20 696 items 11 160 -> 10 790 us.
+        // cycles, longest first.  Lists of long items over more K/V than L2 holds are dealt in two stretches: first the long
+        // items, request by request and KV head by KV head, so that the blocks of the whole GPU work through the same K/V
+        // pages at about the same time and find them in L2; then the short ones, the last kTailItems longest items' worth of
+        // cycles per block, longest first, to even out what the first stretch left.  That order is worth DRAM traffic, and
+        // through the power limit time, back to back: 1 152 items of up to 258 steps a layer of 2 719 -> 2 608 us, 20 696
+        // items 12 921 -> 11 546.  It costs where the items are short: many blocks then ask for the same lines at the same
+        // time (see kPageOrderSteps), and chained lists do not run at the power limit.
         // The kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1 - b : b)) hands every block its own
         // list; holes, only at the end of a block's list, are marked tile_a = -1.
         auto deal_out = [&](std::vector<AttnWork> &list) {
@@ -566,17 +567,18 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 sort_items(list.begin(), list.end());
                 return;
             }
-            // (a list of less than kHeadItems longest items per block has no first stretch: two requests of 33 024 tokens, 2.1
-            // of them, lost up to 2 % to the coarser balance, four, 4.3, gained 4; equal items then keep their pages' order)
-            double all = 0;
+            double all = 0, steps = 0;
             int64_t longest_item = 0;
             for (const AttnWork &w : list) {
                 const int64_t c = cycles_of(w);
                 all += (double)c;
+                steps += w.step_end - w.step_begin;
                 longest_item = std::max(longest_item, c);
             }
-            const bool two_stretches = all >= kHeadItems * (double)longest_item * G;
-            if (!two_stretches) sort_items(list.begin(), list.end());
+            const double kv_bytes = (double)total * Hkv * D * 4;
+            const bool two_stretches = !pl->chained && kv_bytes >= kPageOrderBytes && all >= kHeadItems * (double)longest_item * G &&
+                                       steps >= (D == 64 ? kPageOrderSteps64 : kPageOrderSteps) * (double)list.size();
+            if (!two_stretches) sort_items(list.begin(), list.end());       // equal items keep their pages' order
             // (sorted as runs of equal items - the KV heads of a tile pair - and dealt with a heap of packed (load, block)
             // values: 20 696 items item by item took 5 ms of a plan's 11)
             struct Run { int64_t cycles; int32_t first, n, req; };
