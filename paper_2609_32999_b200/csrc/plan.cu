@@ -557,7 +557,9 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         // cycles per block, longest first, to even out what the first stretch left.  That order is worth DRAM traffic, and
         // through the power limit time, back to back: 1 152 items of up to 258 steps a layer of 2 719 -> 2 608 us, 20 696
         // items 12 921 -> 11 546.  It costs where the items are short: many blocks then ask for the same lines at the same
-        // time (see kPageOrderSteps), and chained lists do not run at the power limit.
+        // time (see kPageOrderSteps), and chained lists do not run at the power limit.  Balance is the lesser matter: 720 and
+        // 1 224 items whose slowest block is modelled 4 and 3 % later in page order than longest first took 503 and 1 235 us,
+        // against 514 and 1 292.
         // The kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1 - b : b)) hands every block its own
         // list; holes, only at the end of a block's list, are marked tile_a = -1.
         auto deal_out = [&](std::vector<AttnWork> &list) {
