@@ -167,7 +167,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     auto load_item = [&](int w, bool staged) {
         Item it;
         it.wk = staged ? s_first.wk : work[w];
-        if (it.wk.tile_a < 0) {            // a hole of the assignment: the block's list has ended
+        if (it.wk.tile_a < 0) {            // a hole of the assignment: the block's list has ended (see attn_grid)
             it.n_tiles = 0;
             return it;
         }
@@ -799,6 +799,11 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
     const AttnWork *work = chunk < 0 ? pl->dev.work : pl->dev.work_chunked + pl->chunk_work_off[chunk];
     const size_t n_work = chunk < 0 ? pl->work.size() : (size_t)(pl->chunk_work_off[chunk + 1] - pl->chunk_work_off[chunk]);
     if (n_work == 0) return cudaSuccess;
+    unsigned grid = (unsigned)attn_grid(pl, chunk, max_blocks);        // persistent
+    if (grid == 0) {
+        *err = "the whole work list is walked by the full grid";
+        return cudaErrorInvalidValue;
+    }
     const int Hq = pl->cfg.num_q_heads, Hkv = pl->cfg.num_kv_heads, g = Hq / Hkv, ps = pl->cfg.page_size;
     CUtensorMap tq, tk, tv, to;
     if (K8) {      // q and k_pool hold one byte per element
@@ -814,16 +819,13 @@ cudaError_t launch_attn_tc_d(const tessera_plan *pl, void *k_pool, void *v_pool,
     if (e != cudaSuccess) { *err = "cudaFuncSetAttribute(shared memory)"; return e; }
     const DeviceTables &d = pl->dev;
     const float scale_log2 = pl->sm_scale * 1.4426950408889634f * qk_scale;
-    // persistent: one thread block per SM (fewer when the list is shorter)
-    const int sms = max_blocks > 0 ? std::min(max_blocks, pl->num_sms) : pl->num_sms;
-    unsigned grid = (unsigned)std::min<size_t>(n_work, (size_t)sms);
     // A chained grid comes in clusters of two, though the blocks share nothing by themselves: neighbours in the list
     // read the same K/V pages at about the same time, and the two SMs of a TPC fetch a line that both ask for once.
     // An ordinary launch places blocks 2 i and 2 i + 1 that way by itself, a chained one wherever an SM becomes free:
     // 1 680 items, head_dim 64: 93 us of mean block time with neighbours together, 103 us without.  (Ordinary
     // launches stay without: beside the host-tier reader not every TPC has both its SMs free.)
     const bool chained = pl->chained && chunk < 0;
-    if (chained && grid % 2 != 0 && grid < (unsigned)sms) ++grid;      // (a block without an item ends at once)
+    if (chained && grid % 2 != 0 && max_blocks <= 0 && grid < (unsigned)pl->num_sms) ++grid;      // (a block without an item ends at once)
     e = launch_clusters(
         attn_tc_kernel<D, kMaxPages, K8>, grid, kThreads, chained && grid % 2 == 0 ? 2 : 1, Geo<D>::kSmemAlloc, st, chained, tq, tk, tv, to, d.tiles, work, (int)n_work, d.q_pos, d.pages,
         static_cast<__nv_bfloat16 *>(out), lse, Hq, g, ps, pl->num_pool_pages, scale_log2, d.ws_o, d.ws_ml, d.status);

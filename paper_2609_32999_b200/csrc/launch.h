@@ -70,7 +70,8 @@ cudaError_t launch_scatter_fresh(const tessera_plan *pl, void *k_pool, void *v_p
                                  const void *v_new, int chunk, cudaStream_t st);
 // tcgen05 attention; returns cudaErrorNotSupported when the plan's shape is outside its range (the plan
 // builder accepts no such shape).
-// max_blocks > 0 caps the persistent grid below one block per SM (SMs left to a concurrent reader kernel).
+// max_blocks > 0 caps the persistent grid below one block per SM (SMs left to a concurrent reader kernel); refused where
+// the whole list has more items than SMs, because it is dealt out for the full grid.
 cudaError_t launch_attn_tc(const tessera_plan *pl, void *k_pool, void *v_pool, const void *q, void *out,
                            float *lse, int chunk, int max_blocks, cudaStream_t st, std::string *err);
 

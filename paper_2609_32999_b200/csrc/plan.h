@@ -150,4 +150,14 @@ namespace tessera {
 // `num_sms`: multiprocessor count the work lists are sized for.  `may_cut`: key ranges may be cut (split-KV).
 int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc *desc,
                         int32_t num_pool_pages, int num_sms, bool may_cut, tessera_plan *plan, std::string *err);
+
+// Thread blocks of an attention launch over the whole list (chunk < 0) or a chunk's: one per SM, `max_blocks` > 0 at most,
+// no more than items.  0 where the list cannot be walked by so few: a dealt list has holes that end a block's share only
+// on the grid it was dealt for.
+inline int attn_grid(const tessera_plan *pl, int chunk, int max_blocks) {
+    const size_t n = chunk < 0 ? pl->work.size() : (size_t)(pl->chunk_work_off[chunk + 1] - pl->chunk_work_off[chunk]);
+    const size_t sms = (size_t)(max_blocks > 0 && max_blocks < pl->num_sms ? max_blocks : pl->num_sms);
+    if (chunk < 0 && sms < (size_t)pl->num_sms && n > (size_t)pl->num_sms) return 0;
+    return (int)(n < sms ? n : sms);
+}
 }  // namespace tessera

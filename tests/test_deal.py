@@ -30,7 +30,8 @@ def view(tmp_path_factory):
         getattr(lib, n).argtypes, getattr(lib, n).restype = getattr(tb._lib, n).argtypes, ctypes.c_int32
     lib.view_work.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int]
     lib.view_tile_steps.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]
-    lib.view_chained.argtypes = [ctypes.c_void_p]
+    lib.view_chained.argtypes = lib.view_chunks.argtypes = [ctypes.c_void_p]
+    lib.view_grid.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     real, tb._lib = tb._lib, lib
     yield lib
     tb._lib = real
@@ -118,3 +119,29 @@ def test_long_lists_over_many_pages_keep_to_few_requests_at_a_time(view, request
     begin = d.work[:, 9]                       # first block-table entry: names the request
     for k in range(len(d.work) // SMS // 2):
         assert len(set(begin[[m[k] for m in d.mine]])) <= 3 * requests // 4
+
+
+@pytest.mark.parametrize("requests,tail", [(1, 40), (6, 200), (20, 250)])
+@pytest.mark.parametrize("blocks", [0, 1, 37, SMS - 16, SMS - 1, SMS, 2 * SMS])
+def test_every_grid_a_launch_may_have_reaches_every_item(view, requests, tail, blocks):
+    """Over the whole list and over every chunk: a block walks until its first hole, and what that leaves out is refused."""
+    plan = tb.Plan(_batch(random.Random(requests), requests, 3, 100, 300, tail, 16, _shape(8, 4)), host_only=True)
+    lists = {-1: np.zeros((view.view_work(plan._h, 0, None, 0), 12), np.int32)}
+    view.view_work(plan._h, 0, lists[-1].ctypes.data, len(lists[-1]))
+    grids = {c: view.view_grid(plan._h, c, blocks) for c in range(-1, view.view_chunks(plan._h))}
+    plan.destroy()
+    assert all(g > 0 for c, g in grids.items() if c >= 0)
+    work, g = lists[-1], grids[-1]
+    if g == 0:
+        assert 0 < blocks < SMS < len(work)
+        return
+    reached = 0
+    for b in range(g):
+        for k in range(-(-len(work) // g)):
+            i = k * g + (g - 1 - b if k & 1 else b)
+            if i >= len(work):
+                continue
+            if work[i, 0] < 0:
+                break
+            reached += 1
+    assert reached == (work[:, 0] >= 0).sum()
