@@ -215,13 +215,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     }
     if (warp == 10 && (int)blockIdx.x < n_work) {
         const Item it = load_item(blockIdx.x, false);
-        if (lane == 0) {
-            s_first.wk = it.wk;
-            s_first.t[0] = it.t0;
-            s_first.t[1] = it.t1;
+        if (lane == 0) s_first.wk = it.wk;
+        if (it.n_tiles > 0) {              // (of a hole there is nothing else to bring)
+            if (lane == 0) {
+                s_first.t[0] = it.t0;
+                s_first.t[1] = it.t1;
+            }
+            const int pi = pps * it.step0 + lane;
+            s_first.page[lane] = pi < it.req_pages ? it.bt[pi] : num_pool_pages;
         }
-        const int pi = pps * it.step0 + lane;
-        s_first.page[lane] = pi < it.req_pages ? it.bt[pi] : num_pool_pages;
     }
     tc_fence_before();
     // Nothing above touches global memory the stream's earlier kernels write, so it runs beside their tail.
