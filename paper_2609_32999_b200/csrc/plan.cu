@@ -535,18 +535,12 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         pl->chunk_run_off[0] = 0;
         for (int r = 1; r < batch; ++r)
             if (chunk_of[r] != chunk_of[r - 1]) pl->chunk_run_off[chunk_of[r]] = req_run_off[r];
-        pl->work_chunked = pl->work;
-        std::stable_sort(pl->work_chunked.begin(), pl->work_chunked.end(), [&](const AttnWork &x, const AttnWork &y) {
-            return chunk_of[pl->tiles[x.tile_a].req] < chunk_of[pl->tiles[y.tile_a].req];
-        });
+        pl->work_chunked = pl->work;           // (built request by request, so chunk by chunk too, as the list to merge is)
         pl->chunk_work_off.assign(used_chunks + 1, 0);
         for (const AttnWork &w : pl->work_chunked) ++pl->chunk_work_off[chunk_of[pl->tiles[w.tile_a].req] + 1];
         for (int c = 0; c < used_chunks; ++c) pl->chunk_work_off[c + 1] += pl->chunk_work_off[c];
         for (int c = 0; c < used_chunks; ++c)
             sort_items(pl->work_chunked.begin() + pl->chunk_work_off[c], pl->work_chunked.begin() + pl->chunk_work_off[c + 1]);
-        std::stable_sort(pl->combine.begin(), pl->combine.end(), [&](const CombineItem &x, const CombineItem &y) {
-            return chunk_of[pl->tiles[x.tile].req] < chunk_of[pl->tiles[y.tile].req];
-        });
         pl->chunk_combine_off.assign(used_chunks + 1, 0);
         for (const CombineItem &ci : pl->combine) ++pl->chunk_combine_off[chunk_of[pl->tiles[ci.tile].req] + 1];
         for (int c = 0; c < used_chunks; ++c) pl->chunk_combine_off[c + 1] += pl->chunk_combine_off[c];
@@ -581,8 +575,8 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             const bool two_stretches = !pl->chained && kv_bytes >= kPageOrderBytes && all >= kHeadItems * (double)longest_item * G &&
                                        steps >= (D == 64 ? kPageOrderSteps64 : kPageOrderSteps) * (double)list.size();
             if (!two_stretches) sort_items(list.begin(), list.end());       // equal items keep their pages' order
-            // (sorted as runs of equal items - the KV heads of a tile pair - and dealt with a heap of packed (load, block)
-            // values: 20 696 items item by item took 5 ms of a plan's 11)
+            // (sorted as runs of equal items - the KV heads of a tile pair - and dealt by a tree: 20 696 items item by item from
+            // a priority queue took 5 ms of a plan's 11)
             struct Run { int64_t cycles; int32_t first, n, req; };
             std::vector<Run> runs;
             for (int32_t i = 0; i < (int32_t)list.size(); ++i) {
@@ -609,28 +603,25 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 for (size_t i = 0; i < head; ++i) sorted[at[order[i].group]++] = order[i];
                 std::copy(sorted.begin(), sorted.end(), order.begin());
             }
-            std::vector<int64_t> loads(G);                 // a heap of load x 2^16 + block, least first
-            for (int b = 0; b < G; ++b) loads[b] = b;
-            std::vector<std::vector<int>> mine(G);
-            for (const Entry &e : order) {
-                mine[loads[0] & 0xffff].push_back(e.item);
-                const int64_t l = loads[0] + (e.cycles << 16);
-                size_t i = 0;
-                for (size_t k = 1; k < loads.size(); i = k, k = 2 * i + 1) {
-                    if (k + 1 < loads.size() && loads[k + 1] < loads[k]) ++k;
-                    if (loads[k] >= l) break;
-                    loads[i] = loads[k];
-                }
-                loads[i] = l;
+            // the blocks' loads (x 2^16, + block) are the leaves of a tree whose nodes hold the least of their two
+            int leaves = 1;
+            while (leaves < G) leaves *= 2;
+            std::vector<int64_t> least(2 * leaves, INT64_MAX);
+            for (int b = 0; b < G; ++b) least[leaves + b] = b;
+            for (int i = leaves - 1; i > 0; --i) least[i] = std::min(least[2 * i], least[2 * i + 1]);
+            std::vector<int32_t> taken(G, 0), at(order.size());           // items a block has; where in the list an item goes
+            int32_t rounds = 0;
+            for (size_t n = 0; n < order.size(); ++n) {
+                const int b = (int)(least[1] & 0xffff), k = taken[b]++;
+                rounds = std::max(rounds, k + 1);
+                at[n] = k * G + ((k & 1) ? G - 1 - b : b);
+                least[leaves + b] += order[n].cycles << 16;
+                for (int i = (leaves + b) / 2; i > 0; i /= 2) least[i] = std::min(least[2 * i], least[2 * i + 1]);
             }
-            size_t rounds = 0;
-            for (auto &m : mine) rounds = std::max(rounds, m.size());
             AttnWork hole{};
             hole.tile_a = -1; hole.tile_b = -1;
-            std::vector<AttnWork> out(rounds * G, hole);
-            for (int b = 0; b < G; ++b)
-                for (size_t k = 0; k < mine[b].size(); ++k)
-                    out[k * G + ((k & 1) ? G - 1 - b : b)] = list[mine[b][k]];
+            std::vector<AttnWork> out((size_t)rounds * G, hole);
+            for (size_t n = 0; n < order.size(); ++n) out[at[n]] = list[order[n].item];
             list.swap(out);
         };
         pl->n_work_items = (int32_t)pl->work.size();
