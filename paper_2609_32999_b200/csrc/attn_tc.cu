@@ -397,10 +397,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
                     // V rows past the end of the sequence hold whatever the page held before; their
                     // probabilities are zero, but 0 x NaN would still poison the accumulator.  (Both
                     // issuing warps may write these zeros; the values agree.)
-                    // The rows are one stretch of bytes in each half.  (Row by row with 16 lanes, 80 rows took 3 000 cycles
-                    // while the step's P waited: layer of a lone 304-token request 12.46 -> 12.17 us.)
+                    // The rows are one stretch of bytes in each half.  (Layer of a lone request of 304 tokens, head_dim 64: row
+                    // by row with 8 lanes a half, 80 rows, 12.46 us; by whole warps, 20 rounds, 12.17.)
                     uint8_t *v = sm + kSmemRing + vslot * kSlotBytes;
-                    if constexpr (K8) {                        // (with 8-bit keys the compiler's step loop loses more: 1 194 -> 1 216 us)
+                    if constexpr (K8) {                        // (the loop below spills 8 bytes here, read in the steps: 1 194 -> 1 216 us)
                         for (int r = T - (step0 + j) * kStep; r < kStep; ++r)
                             if (lane < 8 * G::kHalves) *reinterpret_cast<uint4 *>(v + (lane >> 3) * kHalfBytes + r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
                     } else {

@@ -344,7 +344,7 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             pl->tiles.push_back(t);
         }
     // tcgen05 work items: consecutive tiles of a request share one thread block (and every K/V page
-    // they read); longest first, so that the tail of the grid is made of short items.
+    // they read).
     pl->work.clear();
     {
         const int page = 128;        // keys per step of the tensor-core kernel
@@ -390,8 +390,9 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
             for (auto &pr : pairs) n += parts_of(long_steps(pr), limit);
             return n * Hkv;
         };
-        // Time of the list cut at `limit`: longest-first assignment to the least-loaded SM, plus the merge.  Returns at
-        // once - with no more than that time - where even a perfectly even assignment reaches `enough`.
+        // Time of the list cut at `limit`: longest-first assignment to the least-loaded SM (also of a list that will be dealt
+        // in page order), plus the merge.  Returns at once - with no more than that time - where even a perfectly even
+        // assignment reaches `enough`.
         std::vector<int64_t> part_cost, load;
         auto modelled = [&](int limit, int64_t enough) -> int64_t {
             part_cost.clear();          // of the parts of one head; every head has the same
@@ -549,8 +550,8 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         // items, request by request and KV head by KV head, so that the blocks of the whole GPU work through the same K/V
         // pages at about the same time and find them in L2; then the short ones, the last kTailItems longest items' worth of
         // cycles per block, longest first, to even out what the first stretch left.  That order is worth DRAM traffic, and
-        // through the power limit time, back to back: 1 152 items of up to 258 steps a layer of 2 719 -> 2 608 us, 20 696
-        // items 12 921 -> 11 546.  It costs where the items are short: many blocks then ask for the same lines at the same
+        // through the power limit time, back to back: 1 152 items of up to 258 steps read 3.51 -> 1.77 GB from DRAM, a layer
+        // of them takes 2 719 -> 2 608 us; 20 696 items 12 921 -> 11 546.  It costs where the items are short: many blocks then ask for the same lines at the same
         // time (see kPageOrderSteps), and chained lists do not run at the power limit.  Balance is the lesser matter: 720 and
         // 1 224 items whose slowest block is modelled 4 and 3 % later in page order than longest first took 503 and 1 235 us,
         // against 514 and 1 292.

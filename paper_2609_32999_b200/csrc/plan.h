@@ -26,12 +26,13 @@ constexpr double kPageOrderSteps = 9;    // ... its items have this many 128-key
                                          // back over 285 MB of K/V and more, 3-5 steps 8-20 % slower, 7-8 4-10 %, 8.8 0.6 %; 9.2 2.8 % faster,
                                          // 12-13 0.4-3 %, 17-21 4-8 %, 33 and more 4-13 %
 constexpr double kPageOrderSteps64 = 13; // (at head_dim 64, half the bytes a step: 9.2 steps 2.4 % slower, 17-22 1.4 % faster)
-constexpr double kPageOrderBytes = 80e6; // ... its K and V are more than L2 keeps (126 MB in two halves): items of 17-24 steps over 51-71 MB
-                                         // 0.5 % faster to 1.2 % slower, 12-19 over 88-91 MB 0.2-2 % faster, 21 over 130 MB 6 %
-constexpr double kHeadItems = 2.5;       // ... it has this much work per block, in longest items (2.1: 2 % slower, 4.3: 4 % faster)
+constexpr double kPageOrderBytes = 60e6; // ... its K and V are about half of L2's 126 MB (two halves) or more: over 17-51 MB 1.2 % slower to
+                                         // 0.5 % faster, over 64-71 MB 1.2 % slower to 0.5 % faster with 17-21 steps an item and 0.3-1 %
+                                         // faster with 33 and more, over 88-91 MB 0.2-2 % faster, over 130 MB 3-6 %
+constexpr double kHeadItems = 2.5;       // ... it has this much work per block, in longest items (2.1: 2 % slower; 2.6, 3.6 and 4.3: 3-4 % faster)
 constexpr double kTailItems = 0.6;       // work kept back to even out the blocks, in longest items per block (0.3: up to 13 % slower, 0.9 and
                                          // 1.3: 1-4 % slower on lists of 7 to 140 items per block)
-constexpr int kAttnCostBands = 16;      // cost bands of the attention work list (longest band first)
+constexpr int kAttnCostBands = 16;      // cost bands (longest band first) of a list of one item a block or of a chunk; elsewhere the order of equal items
 
 // One thread block of the gather / shift kernel: `count` consecutive entries of the copy list that
 // belong to one cached unit.  Entry i uses row (row0 + i * row_step) of the cos/sin table.
