@@ -546,15 +546,15 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
         for (const CombineItem &ci : pl->combine) ++pl->chunk_combine_off[chunk_of[pl->tiles[ci.tile].req] + 1];
         for (int c = 0; c < used_chunks; ++c) pl->chunk_combine_off[c + 1] += pl->chunk_combine_off[c];
         // A list of more than one item per thread block is dealt out here, each item to the least-loaded block by modelled
-        // cycles, longest first.  Lists of long items over more K/V than L2 holds are dealt in two stretches: first the long
-        // items, request by request and KV head by KV head, so that the blocks of the whole GPU work through the same K/V
-        // pages at about the same time and find them in L2; then the short ones, the last kTailItems longest items' worth of
-        // cycles per block, longest first, to even out what the first stretch left.  That order is worth DRAM traffic, and
+        // cycles, longest first.  Long lists of long items over much K/V are dealt in two stretches: first the long items,
+        // request by request and KV head by KV head (page order), so that the blocks of the whole GPU work through the same
+        // K/V pages at about the same time and find them in L2; then the short ones, the last kTailItems longest items' worth
+        // of cycles per block, longest first, to even out what the first stretch left.  That order is worth DRAM traffic, and
         // through the power limit time, back to back: 1 152 items of up to 258 steps read 3.51 -> 1.77 GB from DRAM, a layer
-        // of them takes 2 719 -> 2 608 us; 20 696 items 12 921 -> 11 546.  It costs where the items are short: many blocks then ask for the same lines at the same
-        // time (see kPageOrderSteps), and chained lists do not run at the power limit.  Balance is the lesser matter: 720 and
-        // 1 224 items whose slowest block is modelled 4 and 3 % later in page order than longest first took 503 and 1 235 us,
-        // against 514 and 1 292.
+        // of them takes 2 719 -> 2 608 us; 20 696 items 12 921 -> 11 546.  It costs where the items are short, because many
+        // blocks then ask for the same lines at the same time.  Balance is the lesser matter: 720 and 1 224 items whose
+        // slowest block is modelled 4 and 3 % later in page order than longest first took 503 and 1 235 us, against 514 and
+        // 1 292.
         // The kernel's serpentine walk (round k, block b -> index k G + (k odd ? G - 1 - b : b)) hands every block its own
         // list; holes, only at the end of a block's list, are marked tile_a = -1.
         auto deal_out = [&](std::vector<AttnWork> &list) {
@@ -572,9 +572,10 @@ int32_t build_plan_host(const tessera_model_cfg *cfg, const tessera_compose_desc
                 steps += w.step_end - w.step_begin;
                 longest_item = std::max(longest_item, c);
             }
-            const double kv_bytes = (double)total * Hkv * D * 4;
-            const bool two_stretches = !pl->chained && kv_bytes >= kPageOrderBytes && all >= kHeadItems * (double)longest_item * G &&
-                                       steps >= (D == 64 ? kPageOrderSteps64 : kPageOrderSteps) * (double)list.size();
+            steps /= (double)list.size();
+            const double kv_bytes = (double)total * Hkv * D * 4, item_bytes = steps * page * D * 4;
+            const bool two_stretches = all >= kPageOrderCycles * G && steps >= kPageOrderSteps && all >= kHeadItems * (double)longest_item * G &&
+                                       kv_bytes * item_bytes >= kPageOrderBytes * kPageOrderBytes;
             if (!two_stretches) sort_items(list.begin(), list.end());       // equal items keep their pages' order
             // (sorted as runs of equal items - the KV heads of a tile pair - and dealt by a tree: 20 696 items item by item from
             // a priority queue took 5 ms of a plan's 11)

@@ -21,14 +21,15 @@ constexpr int kChainedCycles = 300000;   // modelled attention cycles per SM up 
 constexpr int kSplitMaxRounds = 4;       // batches of more attention items per SM than this are never split, and a split
                                          // list has at most twice as many parts (each with up to two workspace slots)
 constexpr int kHostChunks = 4;          // request chunks of the host-buffer entry point's copy / compute pipeline
-// An attention list is dealt out in page order first (see build_plan_host) where its launches are not chained and ...
-constexpr double kPageOrderSteps = 9;    // ... its items have this many 128-key steps on average: page order against longest first, back to
-                                         // back over 285 MB of K/V and more, 3-5 steps 8-20 % slower, 7-8 4-10 %, 8.8 0.6 %; 9.2 2.8 % faster,
-                                         // 12-13 0.4-3 %, 17-21 4-8 %, 33 and more 4-13 %
-constexpr double kPageOrderSteps64 = 13; // (at head_dim 64, half the bytes a step: 9.2 steps 2.4 % slower, 17-22 1.4 % faster)
-constexpr double kPageOrderBytes = 60e6; // ... its K and V are about half of L2's 126 MB (two halves) or more: over 17-51 MB 1.2 % slower to
-                                         // 0.5 % faster, over 64-71 MB 1.2 % slower to 0.5 % faster with 17-21 steps an item and 0.3-1 %
-                                         // faster with 33 and more, over 88-91 MB 0.2-2 % faster, over 130 MB 3-6 %
+// An attention list is dealt out in page order first (see build_plan_host) where, modelled and averaged over the list, ...
+constexpr double kPageOrderCycles = 225000;   // ... an SM has this many cycles of it and more, so that calls back to back reach the power limit:
+                                              // 9 to 12 steps an item, 130-220 000 cycles 1-3 % slower in page order, 230-260 000 3 % faster
+constexpr double kPageOrderSteps = 9;         // ... an item has this many 128-key steps: 3-5 steps 8-20 % slower (over 285 MB and more of K/V),
+                                              // 7-8 4-10 %, 8.8 0.6 %; 9.2 2.8 % faster, 17-21 4-8 %, 33 and more 4-13 %
+constexpr double kPageOrderBytes = 8.4e6;     // ... and this is at most the geometric mean of what an item reads (64 KB a step at head_dim 128)
+                                              // and the batch's K/V: 12 steps, 75 MB (7.7e6) 2.7 % slower; 10.6, 131 (9.5e6) 0.3 %; 12.6, 88
+                                              // (8.5e6) and 13, 120 (10e6) 2.2 and 3.6 % faster; 42, 35 (9.8e6) 1.6 %; at head_dim 64 14.5, 78
+                                              // (6.1e6) 3.8 % slower; 26, 83 (8.4e6) 0.9 %; 17, 138 (8.8e6) 1.4 % faster.  From 17e6 on 3-13 %.
 constexpr double kHeadItems = 2.5;       // ... it has this much work per block, in longest items (2.1: 2 % slower; 2.6, 3.6 and 4.3: 3-4 % faster)
 constexpr double kTailItems = 0.6;       // work kept back to even out the blocks, in longest items per block (0.3: up to 13 % slower, 0.9 and
                                          // 1.3: 1-4 % slower on lists of 7 to 140 items per block)

@@ -18,5 +18,4 @@ __attribute__((visibility("default"))) int view_tile_steps(const tessera_plan *p
 }
 __attribute__((visibility("default"))) int view_grid(const tessera_plan *p, int chunk, int max_blocks) { return tessera::attn_grid(p, chunk, max_blocks); }
 __attribute__((visibility("default"))) int view_chunks(const tessera_plan *p) { return (int)p->chunk_work_off.size() - 1; }
-__attribute__((visibility("default"))) int view_chained(const tessera_plan *p) { return p->chained; }
 }

@@ -30,7 +30,7 @@ def view(tmp_path_factory):
         getattr(lib, n).argtypes, getattr(lib, n).restype = getattr(tb._lib, n).argtypes, ctypes.c_int32
     lib.view_work.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int]
     lib.view_tile_steps.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]
-    lib.view_chained.argtypes = lib.view_chunks.argtypes = [ctypes.c_void_p]
+    lib.view_chunks.argtypes = [ctypes.c_void_p]
     lib.view_grid.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     real, tb._lib = tb._lib, lib
     yield lib
@@ -48,9 +48,7 @@ class Deal:
         view.view_work(plan._h, 1, self.items.ctypes.data, len(self.items))
         tiles = np.zeros(max(1, view.view_tile_steps(plan._h, None, 0)), np.int32)
         view.view_tile_steps(plan._h, tiles.ctypes.data, len(tiles))
-        self.chained = bool(view.view_chained(plan._h))
-        self.min_steps = 13 if w.shape.head_dim == 64 else 9
-        self.kv_bytes = int(w.seq_len.sum()) * w.shape.num_kv_heads * w.shape.head_dim * 4
+        self.row_bytes, self.kv_heads, self.tokens = w.shape.head_dim * 4, w.shape.num_kv_heads, int(w.seq_len.sum())
         plan.destroy()
         self.grid = min(n, SMS)
         self.mine = [[] for _ in range(self.grid)]              # the kernel's walk
@@ -65,6 +63,12 @@ class Deal:
     def _cycles(x, tiles):
         a, b = min(x[4], tiles[x[0]]) - x[3], min(x[4], tiles[x[1]]) - x[3] if x[1] >= 0 else 0
         return 1700 + (2 if x[1] >= 0 else 1) * 4700 + min(a, b) * 3180 + (max(a, b) - min(a, b)) * 2400
+
+    def page_order(self):
+        """Whether the list is dealt out request by request first."""
+        all_cycles, item, kv = int(self.cycles.sum()), self.mean_steps * 128 * self.row_bytes, self.tokens * self.kv_heads * self.row_bytes
+        return (len(self.items) > SMS and all_cycles >= 225000 * SMS and self.mean_steps >= 9 and all_cycles >= 2.5 * self.cycles.max() * SMS
+                and item * kv >= 8.4e6 ** 2)
 
     def end(self):
         return max(int(self.cycles[m].sum()) for m in self.mine)
@@ -95,7 +99,7 @@ def _shape(heads, group, dim=128):
 
 @pytest.mark.parametrize("seed", range(4))
 def test_lists_whose_pages_need_no_order_are_dealt_longest_first(view, seed):
-    """Chained lists, lists of short items and of few pages: no block is later than longest first leaves it."""
+    """Short lists, lists of short items and of few pages: no block is later than longest first leaves it."""
     rng = random.Random(seed)
     dealt = 0
     for _ in range(15):
@@ -103,7 +107,7 @@ def test_lists_whose_pages_need_no_order_are_dealt_longest_first(view, seed):
                    _shape(rng.choice([2, 4, 8]), rng.choice([2, 4, 5, 7, 8]), rng.choice([64, 128])))
         d = Deal(view, w)
         d.check()
-        if len(d.items) > SMS and (d.chained or d.mean_steps < d.min_steps or d.kv_bytes < 60e6):
+        if len(d.items) > SMS and not d.page_order():
             assert d.end() == d.longest_first()
             dealt += 1
     assert dealt >= 5
@@ -114,8 +118,7 @@ def test_long_lists_over_many_pages_keep_to_few_requests_at_a_time(view, request
     """Over the first half of the rounds, the thread blocks' n-th items belong to three quarters of the requests at most."""
     d = Deal(view, _batch(random.Random(0), requests, units, 512, 512, 128, again, _shape(8, 4)))
     d.check()
-    assert not d.chained and d.mean_steps >= d.min_steps and d.kv_bytes >= 60e6
-    assert d.end() <= 1.02 * d.longest_first()
+    assert d.page_order() and d.end() <= 1.02 * d.longest_first()
     begin = d.work[:, 9]                       # first block-table entry: names the request
     for k in range(len(d.work) // SMS // 2):
         assert len(set(begin[[m[k] for m in d.mine]])) <= 3 * requests // 4
