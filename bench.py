@@ -49,9 +49,9 @@ def measured_peaks():
 
 
 def kernel_traffic():
-    """DRAM bytes per launch of the two main kernels as ncu measured them on ONE config-4 request
-    (profiles/traffic.json, which also records the kernel sources the capture was taken on).  Returns
-    (per-request bytes or None, stale flag): stale when a kernel source has changed since."""
+    """DRAM bytes per launch of the two main kernels as ncu measured them on config 4 (profiles/traffic.json,
+    which also records the sources the capture was taken on).  Returns (the capture or None, stale flag):
+    stale when one of the sources has changed since."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None, True
@@ -811,13 +811,10 @@ def main():
     value = all_tokens / (ms_per_step / 1e3)
     attn_tflops, gather_gbs = leg.rates(head)
     traffic, stale = kernel_traffic()
-    scale = w.batch if (traffic and args.config == 4) else None
+    captured = traffic["config4"] if traffic and args.config == 4 and w.batch == traffic["config4"]["requests"] else None
 
     def traffic_of(kernel):
-        if not scale:
-            return None
-        k = traffic["config4_one_request"][kernel]
-        return (k["dram_bytes_read"] + k["dram_bytes_write"]) * scale
+        return captured[kernel]["dram_bytes_read"] + captured[kernel]["dram_bytes_write"] if captured else None
 
     long_region = total_ms_max > 1000.0
     tensor_peak = peaks["bf16_tflops_sustained"] if long_region else peaks["bf16_tflops"]
@@ -844,7 +841,7 @@ def main():
                      "frac_of_nominal_2250": attn_tflops / NOMINAL_TFLOPS,
                      "ms_per_launch": head["attn_ms"], "flops_per_launch": int(info.attn_flops),
                      "traffic": traffic_of("attn"), "traffic_stale": bool(stale),
-                     "traffic_note": "DRAM bytes per launch: ncu capture of one request (profiles/traffic.json) x requests; "
+                     "traffic_note": "DRAM bytes per launch: ncu capture (profiles/traffic.json); "
                                      "algorithmic minimum (assembled K,V once + Q + O) %.1f MB"
                                      % ((w.total_tokens * sh.num_kv_heads * sh.head_dim * 2 * 2
                                          + 2 * w.n_q * sh.num_q_heads * sh.head_dim * 2) / 1e6)},
@@ -853,7 +850,7 @@ def main():
                             "peak_source": peaks["source"] + " copy", "frac_of_nominal_8000": gather_gbs / NOMINAL_GBS,
                             "ms_per_launch": head["gather_ms"], "bytes_per_launch": int(info.gather_bytes),
                             "traffic": traffic_of("gather"), "traffic_stale": bool(stale),
-                            "dram_level_GBps": (traffic_of("gather") / (head["gather_ms"] / 1e3) / 1e9) if scale else None},
+                            "dram_level_GBps": (traffic_of("gather") / (head["gather_ms"] / 1e3) / 1e9) if captured else None},
         "recompute_tokens_per_s": w.n_q * world / (ms_per_step / 1e3),
         "plan_create_ms": leg.plan_create_ms,
         "masked_mma_fraction": leg.plan.masked_mma_fraction,

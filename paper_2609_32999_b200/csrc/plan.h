@@ -25,7 +25,7 @@ constexpr int kHostChunks = 4;          // request chunks of the host-buffer ent
 constexpr double kPageOrderCycles = 225000;   // ... an SM has this many cycles of it and more, so that calls back to back reach the power limit:
                                               // 9 to 12 steps an item, 130-220 000 cycles 1-3 % slower in page order, 230-260 000 3 % faster
 constexpr double kPageOrderSteps = 9;         // ... an item has this many 128-key steps: 3-5 steps 8-20 % slower (over 285 MB and more of K/V),
-                                              // 7-8 4-10 %, 8.8 0.6 %; 9.2 2.8 % faster, 17-21 4-8 %, 33 and more 4-13 %
+                                              // 7-8 5 % slower to 4 % faster, 9.2 2.8 % faster, 17-21 4-8 %, 33 and more 4-13 %
 constexpr double kPageOrderBytes = 8.4e6;     // ... and this is at most the geometric mean of what an item reads (64 KB a step at head_dim 128)
                                               // and the batch's K/V: 12 steps, 75 MB (7.7e6) 2.7 % slower; 10.6, 131 (9.5e6) 0.3 %; 12.6, 88
                                               // (8.5e6) and 13, 120 (10e6) 2.2 and 3.6 % faster; 42, 35 (9.8e6) 1.6 %; at head_dim 64 14.5, 78
